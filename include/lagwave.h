@@ -221,7 +221,8 @@ int  lag_dst_f64_slice_products(int n);
  * lag_precond_apply and the solvers) of nrhs right-hand sides launches on this plan and device:
  *   LAG_GEMM_SIMT           no tensor-core GEMM (SIMT kernels)
  *   LAG_GEMM_SPLIT_BF16     mixed plan: split-bf16 operands, FP32 accumulation
- *   LAG_GEMM_SLICE_TILES    float64 exact slices, one CTA per 128 x 128 output tile
+ *   LAG_GEMM_SLICE_TILES    float64 exact slices, one CTA per output tile (128 x 64 for ceil(n/2) <=
+ *                           1024, else 128 x 128)
  *   LAG_GEMM_SLICE_STREAMK  float64 exact slices, the steps of all tiles cut into equal ranges, one
  *                           per SM (LAGWAVE_OZ_SK=1, opt-in: one right-hand side whose tile count is
  *                           not a multiple of the SM count)

@@ -62,6 +62,11 @@ int stencil_blocks(const lag_grid &g) { return ((g.nx + 31) / 32) * ((g.nz + 7) 
 
 // ------------------------------------------------------------------------------ preconditioner
 void lag_precond::ensure_scratch(int nrhs) {
+  if (dst.ow_b != nullptr && dst.oz_b == nullptr && dst_oz_variant_opted_in()) {
+    slice_store.alloc(ctx, dst_oz_slice_store_bytes(dst));
+    dst_build_oz_slices(dst, slice_store.as<uint8_t>(), cudaStreamPerThread);
+    LAG_CUDA_CHECK(cudaStreamSynchronize(cudaStreamPerThread));
+  }
   if (nrhs <= scratch_rhs) return;
   const size_t per = (size_t)grid.nx * grid.nz;
   scratch.alloc(ctx, per * nrhs * (prec == LAG_FP64 ? sizeof(double) : sizeof(float)));
@@ -187,7 +192,7 @@ lag_precond *lag::precond_new(lag_ctx *ctx, const lag_grid &gu, double ax, doubl
   p->ax = ax;
   p->az = az;
   p->d = d;
-  p->dst_store.ctx = p->tri_store.ctx = p->tri32_store.ctx = p->scratch.ctx = p->tc_scratch.ctx = ctx;
+  p->dst_store.ctx = p->slice_store.ctx = p->tri_store.ctx = p->tri32_store.ctx = p->scratch.ctx = p->tc_scratch.ctx = ctx;
   p->zrows.ctx = ctx;
   p->layered = layered != nullptr;
   const bool gen = !zr.empty();

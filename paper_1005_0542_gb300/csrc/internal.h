@@ -136,8 +136,12 @@ struct DstPlan {
   uint8_t *tc_scratch = nullptr;
   int *tc_err = nullptr;
   int tc_products = 3;        // split products per K step: 3 (hi*hi+hi*lo+lo*hi), 2 or 1
-  // float64 path on the tensor cores (exact slices): packed B slices [2][9][n tile][k stage]
+  // float64 path on the tensor cores (exact slices): packed B digits of the weight-stacked kernel
+  // (8-bit format), packed B slices [2][9][n tile][k stage] of the tile kernel (other formats, or
+  // built when an opt-in variant first runs)
   bool oz = false;
+  uint8_t *ow_b = nullptr;
+  uint8_t *ow_bi = nullptr;   // DCT-II inverse operands (kind 1)
   uint8_t *oz_b = nullptr;
   uint8_t *oz_bi = nullptr;   // DCT-II inverse operands (kind 1): [2][9][n tile][k stage]
   size_t oz_slice_bytes = 0;
@@ -169,6 +173,10 @@ size_t dst_oz_scratch_bytes(const DstPlan &dp, int rows);
 // exact-slice GEMM kernels (the values of LAG_GEMM_SLICE_* in lagwave.h)
 constexpr int OZ_GEMM_TILES = 2, OZ_GEMM_STREAMK = 3, OZ_GEMM_PAIRS = 4, OZ_GEMM_CLUSTER = 5;
 int dst_oz_gemm_variant(const DstPlan &dp, int rows, int rpr, int inv);
+// the opt-in variants' slice tiles, for plans that run the weight-stacked kernel by default
+bool dst_oz_variant_opted_in();
+size_t dst_oz_slice_store_bytes(const DstPlan &dp);
+void dst_build_oz_slices(DstPlan &dp, uint8_t *store, cudaStream_t s);
 // inverse (DCT-II plans only): gather the even / odd modes, GEMM with the inverse operands into
 // E / O sums (plan scratch), butterfly into y
 void dst_apply_oz(const DstPlan &dp, const double *x, double *y, int rows, int rows_per_rhs,
@@ -207,6 +215,7 @@ struct lag_precond {
   lag::DstPlan dst;
   lag::TriFactors tri64, tri32;
   lag::DevBuf dst_store, tri_store, tri32_store;
+  lag::DevBuf slice_store;  // slice tiles of the opt-in float64 GEMM variants, built on first use
   lag::DevBuf scratch;      // intermediate spectra (float64 or float32), grows with nrhs
   lag::DevBuf tc_scratch;   // tensor-core DST: packed A operands and E/O halves
   int scratch_rhs = 0;

@@ -857,7 +857,9 @@ __device__ __forceinline__ void oz_store(const long long (&acci)[64], int ncols,
   else oz_store_row<false>(acci, ncols, kx, scale, unit, yp, ystride);
 }
 
-// |v| < 2^e: NBITS-bit fixed-point expansion of |v| 2^-e, truncated (integer arithmetic on the bits)
+// |v| < 2^e: NBITS-bit fixed-point expansion of |v| 2^-e (integer arithmetic on the bits), rounded to
+// nearest for the 8-bit digits (a result of 2^55 still has its top digit at 128, as in the
+// weight-stacked kernel's ow_fixed), truncated for the 7- and 6-bit slices (whose top slice would overflow)
 template <int NBITS>
 __device__ __forceinline__ unsigned long long oz_fixed(double v, int e) {
   static_assert(NBITS >= 53 && NBITS <= 63, "fixed-point width");
@@ -866,6 +868,7 @@ __device__ __forceinline__ unsigned long long oz_fixed(double v, int e) {
   const unsigned long long M = (bits & 0xfffffffffffffull) | (E ? (1ull << 52) : 0ull);
   const int s = (E ? E : 1) - 1075 + NBITS - e;  // |v| = M 2^((E ? E : 1) - 1075)
   if (s >= 0) return M << s;                      // s <= NBITS - 52 since |v| < 2^e
+  if constexpr (NBITS == 55) return (s < -54) ? 0ull : ((M + (1ull << (-s - 1))) >> (-s));
   return (s <= -64) ? 0ull : (M >> (-s));
 }
 // slice i (1-based) of an NB*NS-bit fixed-point value, pre-scaled by 2^-(NB (i - 1)) and signed, as
@@ -2316,6 +2319,8 @@ __global__ void __launch_bounds__(320, 1) oz_gemm_mc_kernel(const uint8_t *__res
   if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(OZ_NACC * OZ_TN) : "memory");
 }
 
+#include "oz_weights.cuh"
+
 // Schedule of one output tile.  Exact groups: units of one weight d < tail over one K chunk (the
 // longest multiple of 64 K values whose sum stays exact, kc), at most gmax units per accumulator.
 // The tail (d >= tail, FP32-rounded) is cut into chunks of at most 3 pairs over the whole K range,
@@ -2457,24 +2462,59 @@ bool dst_oz_supported(int n) {
   return n >= 16 && 63LL * 63LL * kpad <= (1LL << 24);  // one pair per accumulator at least
 }
 
+// the weight-stacked kernel runs the 8-bit format
+static bool ow_supported(int n) { return oz_format(div_up((n + 1) / 2, TK) * TK).nb == 8; }
+static size_t ow_bytes(int n) {
+  const int ku = (n + 1) / 2;
+  return 2 * (size_t)div_up(ku, OW_N) * div_up(ku, OW_K) * OW_B;
+}
+
 size_t dst_oz_bytes(int n, int kind) {
   const int ku = (n + 1) / 2;
-  return (kind == 1 ? 2 : 1) * 2 * (size_t)OZ_SMAX * div_up(ku, OZ_TN) * div_up(ku, TK) * OZ_BT;
+  const size_t mats = kind == 1 ? 2 : 1;
+  if (ow_supported(n)) return mats * ow_bytes(n);
+  return mats * 2 * (size_t)OZ_SMAX * div_up(ku, OZ_TN) * div_up(ku, TK) * OZ_BT;
 }
 
 void dst_build_oz(DstPlan &dp, DevBuf &store, size_t off, cudaStream_t s) {
-  const int nks = div_up(dp.ku, TK), nnt = div_up(dp.ku, OZ_TN);
-  dp.kpad_u = nks;
-  dp.npad_u = nnt;
-  dp.oz_slice_bytes = (size_t)nnt * nks * OZ_BT;
-  dp.oz_b = store.as<uint8_t>() + off;
   int eB = 0;
   // every |S| <= sqrt(2 / (n + 1)) < 2^eB (DST-I); every |V| <= sqrt(2 / n) < 2^eB (DCT-II)
   frexp(std::sqrt(2.0 / (double)(dp.kind == 1 ? dp.n : dp.n + 1)), &eB);
   dp.oz_eB = eB;
-  const OzFmt f = oz_format(nks * TK);
+  dp.kpad_u = div_up(dp.ku, TK);
+  dp.npad_u = div_up(dp.ku, OZ_TN);
+  const OzFmt f = oz_format(dp.kpad_u * TK);
   dp.oz_nb = f.nb;
   dp.oz_ns = f.ns;
+  dp.oz = true;
+  if (f.nb != 8) {
+    dst_build_oz_slices(dp, store.as<uint8_t>() + off, s);
+    return;
+  }
+  dp.ow_b = store.as<uint8_t>() + off;
+  const int nk = div_up(dp.ku, OW_K), nnt = div_up(dp.ku, OW_N);
+  dim3 g(div_up(nnt * OW_N, 128), 2 * nk, 2);
+  ow_pack_b_kernel<<<g, 128, 0, s>>>(dp.su, dp.ku, dp.ku, dp.ku, dp.sv, dp.kv, dp.kv, dp.kv, nk, nnt, eB, dp.ow_b);
+  count_launch();
+  LAG_LAUNCH_CHECK();
+  if (dp.kind == 1) {  // inverse operands: even / odd input modes x ceil(n/2) output columns
+    dp.ow_bi = dp.ow_b + ow_bytes(dp.n);
+    ow_pack_b_kernel<<<g, 128, 0, s>>>(dp.ie, dp.ku, dp.ku, dp.ku, dp.io, dp.kv, dp.ku, dp.ku, nk, nnt, eB, dp.ow_bi);
+    count_launch();
+    LAG_LAUNCH_CHECK();
+  }
+}
+
+size_t dst_oz_slice_store_bytes(const DstPlan &dp) {
+  return (dp.kind == 1 ? 2 : 1) * 2 * (size_t)OZ_SMAX * dp.npad_u * dp.kpad_u * OZ_BT;
+}
+
+// slice tiles of S for the tile kernel and its variants (formats of 6 and 7 bits, or an opt-in variant)
+void dst_build_oz_slices(DstPlan &dp, uint8_t *store, cudaStream_t s) {
+  const int nks = dp.kpad_u, nnt = dp.npad_u, eB = dp.oz_eB;
+  dp.oz_slice_bytes = (size_t)nnt * nks * OZ_BT;
+  dp.oz_b = store;
+  const OzFmt f{dp.oz_nb, dp.oz_ns};
   dim3 g(div_up(nks * TK, 128), nnt * OZ_TN, 2);
   auto pack_b = [&](const double *m0, int k0n, int n0n, int ld0, const double *m1, int k1n, int n1n, int ld1,
                     uint8_t *out) {
@@ -2495,7 +2535,6 @@ void dst_build_oz(DstPlan &dp, DevBuf &store, size_t off, cudaStream_t s) {
     dp.oz_bi = dp.oz_b + 2 * (size_t)f.ns * dp.oz_slice_bytes;
     pack_b(dp.ie, dp.ku, dp.ku, dp.ku, dp.io, dp.kv, dp.ku, dp.ku, dp.oz_bi);
   }
-  dp.oz = true;
 }
 
 // 2-D tensor map over `nrows` rows of 128 bytes (64 bf16) at base: TMA copies of box_rows whole
@@ -2612,6 +2651,12 @@ static void oz_cluster_shape(int &cm, int &cn) {
   if (cm * cn == 1) cm = cn = 0;
 }
 
+bool dst_oz_variant_opted_in() {
+  int cm, cn;
+  oz_cluster_shape(cm, cn);
+  return cm > 0 || oz_pair_enabled() || oz_sk_enabled();
+}
+
 // the GEMM kernel of a forward (inv = 0) or DCT-II inverse (inv = 1) transform of `rows` rows,
 // rpr rows per right-hand side
 int dst_oz_gemm_variant(const DstPlan &dp, int rows, int rpr, int inv) {
@@ -2669,6 +2714,37 @@ static void oz_launch_mc(const uint8_t *apack, size_t a_slice, const uint8_t *bp
   LAG_CUDA_CHECK(cudaLaunchKernelEx(&cfg, oz_gemm_mc_kernel<NB, NS, CM, CN>, apack, a_slice, bpack, dp.oz_slice_bytes,
                                     erow, dp.oz_eB, nks, nmt, nnt, rows, y, dp.n, dp.ku, dp.kv, sch, sc, rpr, dp.tc_err,
                                     inv));
+}
+
+// the weight-stacked kernel (8-bit format, no opt-in variant)
+static void ow_apply(const DstPlan &dp, const double *x, double *y, int rows, int rpr, const KrylovScalars *sc,
+                     cudaStream_t s, int inv) {
+  static PerDeviceOnce attr;
+  attr.run([] {
+    LAG_CUDA_CHECK(cudaFuncSetAttribute(oz_wgemm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, OW_SMEM));
+    LAG_CUDA_CHECK(cudaFuncSetAttribute(ow_pack_a_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                        (int)oz_pack_smem(OZ_PACK_MAXK / TK + 1)));
+  });
+  const int nk = div_up(dp.ku, OW_K), nnt = div_up(dp.ku, OW_N), nmt = div_up(rows, TM);
+  uint8_t *apack = dp.tc_scratch + oz_sk_bytes();
+  int *erow = reinterpret_cast<int *>(apack + 2 * (size_t)nmt * nk * OW_A);
+  // E / O sums of the inverse: after the digits and the row exponents, 256-byte aligned
+  double *eo = reinterpret_cast<double *>(
+      (reinterpret_cast<uintptr_t>(erow + 2 * (size_t)nmt * TM) + 255) & ~(uintptr_t)255);
+  ow_pack_a_kernel<<<nmt * TM, OZ_PACK_THREADS, oz_pack_smem(dp.kpad_u), s>>>(x, rows, dp.n, dp.ku, dp.kv, nk, nmt,
+                                                                              apack, erow, sc, rpr, inv);
+  count_launch();
+  LAG_LAUNCH_CHECK();
+  oz_wgemm_kernel<<<std::min(2 * nmt * nnt, device_sms()), 320, OW_SMEM, s>>>(
+      apack, inv ? dp.ow_bi : dp.ow_b, erow, dp.oz_eB, nk, nmt, nnt, rows, inv ? eo : y, dp.n, dp.ku, dp.kv, sc, rpr,
+      dp.tc_err, inv);
+  count_launch();
+  LAG_LAUNCH_CHECK();
+  if (inv) {
+    oz_butterfly_kernel<<<rows, 256, 0, s>>>(eo, y, rows, dp.n, dp.ku, sc, rpr);
+    count_launch();
+    LAG_LAUNCH_CHECK();
+  }
 }
 
 template <int NB, int NS>
@@ -2745,6 +2821,11 @@ void dst_apply_oz(const DstPlan &dp, const double *x, double *y, int rows, int r
   if (rows <= 0) return;
   ProfScope prof(KC_DST64, s);
   const int inv = (inverse && dp.kind == 1) ? 1 : 0;
+  if (dp.ow_b != nullptr && dst_oz_gemm_variant(dp, rows, rpr, inv) == OZ_GEMM_TILES) {
+    ow_apply(dp, x, y, rows, rpr, sc, s, inv);
+    return;
+  }
+  if (dp.oz_b == nullptr) throw Error(LAG_EINVAL, "exact-slice DST: the slice tiles of this variant are not built");
   if (dp.oz_nb == 8) oz_apply_fmt<8, 7>(dp, x, y, rows, rpr, sc, s, inv);
   else if (dp.oz_nb == 7) oz_apply_fmt<7, 8>(dp, x, y, rows, rpr, sc, s, inv);
   else oz_apply_fmt<6, 9>(dp, x, y, rows, rpr, sc, s, inv);

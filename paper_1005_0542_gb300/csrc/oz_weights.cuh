@@ -1,0 +1,568 @@
+// Exact-slice float64 DST: the weight-stacked GEMM (the default for ceil(n/2) <= 1024).
+//
+// Same arithmetic as the 8-bit format of the tile kernel: 7 balanced base-256 digits per operand,
+// the 28 digit products with i + j <= 8, exact sums in FP32 tensor memory combined in int64.  What
+// differs is where the products of one K step meet.  The tile kernel runs one (or two) digit
+// products at a time over the whole K range of a 128 x 128 tile, so every digit tile crosses into
+// the SM several times (44 tiles per K step for 28 products) and the SM's 64 B/clk port from the L2
+// bounds it (59 B/clk measured).  Here a stage holds ALL seven digit tiles of both operands for 16
+// values of K, each crosses once (21 tile halves for the same 28 products: 47 B/clk at the tensor
+// pipe's full rate), and every weight w = i + j keeps its own 64-column accumulator:
+//   * tile 128 rows x 64 columns; accumulator of weight w = 2..8 at tensor-memory column 64 (w - 2);
+//   * the B digits lie behind one another in shared memory (64 rows each), so A_i x [B_j .. B_j+m-1]
+//     is ONE tcgen05.mma of N = 64 m whose column blocks are the m consecutive weights i + j ..:
+//     ten MMAs of 64..256 columns per K step do the 28 products in 908 clocks (896 at the tensor
+//     pipe's peak).  They are issued narrow ones first: the three 256-column ones at the end of a
+//     stage keep the pipe busy while the issuer commits the stage and waits for the next one
+//     (the other way round the pipe idled 75 - 275 clocks per stage);
+//   * weight w sums w - 1 products per K value, each at most 2^14, so it stays exact (up to 2^24)
+//     for 1024 / (w - 1) values of K; eight epilogue warps drain it in time (ow_drain) into int64
+//     sums held in registers and zero it.  Drains go by group of weights ({2,3,4}, {5,6}, {7,8}), each
+//     group with its own pair of barriers: the stage after a drain issues the other groups' MMAs first;
+//   * the FP32-rounded tail is weights 7 and 8 (2^-40 and 2^-48 of the leading products); weight 7 is
+//     drained once on the way so that its accumulation error (directed, about linear in the number of
+//     MMAs and the size of the sum) stays below the tile kernel's.
+// Digits are plain integers (not pre-scaled: every accumulator holds one weight), and both operands'
+// expansions are rounded to nearest at 2^-55 instead of truncated (row errors against extended
+// precision 2.1e-16 - 2.8e-16 on random rows of 40..2048 values, 2.2e-16 - 3.7e-16 with truncation).
+// Measured, whole preconditioner applies (two transforms each), tile kernel -> this one: 1024 x 1024 x
+// 256 right-hand sides 21.1 -> 14.3 ms, 2048 x 1024 x 1 287 -> 257 us, 63 x 40 65.6 -> 45.1 us.
+constexpr int OW_NS = 7;                          // digits per operand
+constexpr int OW_K = 16;                          // K values per stage (one MMA K step)
+constexpr int OW_N = 64;                          // output columns per tile
+constexpr int OW_ASL = TM * OW_K * 2;             // one A digit of a stage: 128 rows of 32 bytes
+constexpr int OW_BSL = OW_N * OW_K * 2;           // one B digit of a stage: 64 rows of 32 bytes
+constexpr int OW_A = OW_NS * OW_ASL;              // 28 KB
+constexpr int OW_B = OW_NS * OW_BSL;              // 14 KB
+constexpr int OW_STAGE = OW_A + OW_B;
+constexpr int OW_NST = 4;                         // three stages in flight: 2.7 k clocks of MMAs
+constexpr int OW_TPITCH = 17;                     // doubles per row of a warp's transposition buffer
+constexpr int OW_TBUF = 32 * OW_TPITCH * 8;       // per epilogue warp: 32 rows x 16 columns
+constexpr int OW_SMEM = OW_NST * OW_STAGE + 8 * OW_TBUF + 1024 + 256;
+constexpr uint32_t OW_TMEM = 512;                 // allocated columns (7 x 64 used)
+constexpr int OW_FIX = 38;                        // sums in units of 2^-38 of a weight-2 unit
+
+// element (r, k) of a rows x 16 digit tile: 32-byte rows, K-major SWIZZLE_32B (byte offset)
+__device__ __forceinline__ uint32_t ow_swz(int r, int kchunk) {
+  return (uint32_t)r * 32u + (uint32_t)((kchunk ^ (r >> 2)) & 1) * 16u;
+}
+
+// Stages after which a group of weights is drained (bit c: after c stages of a tile of nk <= 64; every
+// group at the tile's end).  Exactness allows weight 3 32 stages (2 x 512 x 2^14 = 2^24), 4 20, 5 16,
+// 6 12; a drain costs the MMA stream about 700 clocks (narrower MMAs, a commit and a wait on the
+// issuing thread), so the weights of a group go together, at stages no two groups share; none
+// before stage 12, while the epilogue warps still convert and store the previous tile.
+constexpr unsigned long long OW_E0 = (1ull << 18) | (1ull << 38) | (1ull << 58);                            // 3, 4
+constexpr unsigned long long OW_E1 = (1ull << 12) | (1ull << 24) | (1ull << 36) | (1ull << 48) | (1ull << 60);  // 5, 6
+constexpr unsigned long long OW_E2 = 1ull << 30;                                                            // 7
+__device__ __forceinline__ uint32_t ow_bit(unsigned long long m, int c) { return (uint32_t)(m >> c) & 1u; }
+
+// rn(v 2^(55 - e)) for |v| < 2^e, signed (integer arithmetic on the bits); |result| <= 2^55
+__device__ __forceinline__ long long ow_fixed(double v, int e) {
+  const long long b = __double_as_longlong(v);
+  const int E = (int)((b >> 52) & 0x7ff);
+  const unsigned long long M = ((unsigned long long)b & 0xfffffffffffffull) | (E ? (1ull << 52) : 0ull);
+  const int s = (E ? E : 1) - 1020 - e;  // |v| 2^(55 - e) = M 2^s
+  unsigned long long t;
+  if (s >= 0) t = M << s;                // s <= 3 since |v| < 2^e
+  else t = (s < -54) ? 0ull : ((M + (1ull << (-s - 1))) >> (-s));
+  return b < 0 ? -(long long)t : (long long)t;
+}
+
+// the seven digits of 8 values |T| <= 2^55 (8 consecutive K of one row), as bf16, 16 bytes per digit
+// at dst + digit * OW_ASL: T plus 128 in each byte position has bytes d_i + 128 (the leading one up to
+// 256); 2^23 + byte as a float by one byte permute, minus 2^23 + 128 is the digit, exact in bf16
+template <int STRIDE>
+__device__ __forceinline__ void ow_store_digits(const long long (&T)[8], uint8_t *dst) {
+  uint32_t th[8], tl[8];
+#pragma unroll
+  for (int q = 0; q < 8; ++q) {
+    const unsigned long long Tb = (unsigned long long)(T[q] + 0x0080808080808080ll);
+    tl[q] = (uint32_t)Tb;
+    th[q] = (uint32_t)(Tb >> 32);
+  }
+#pragma unroll
+  for (int i = 1; i <= OW_NS; ++i) {
+    uint32_t hw[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      float d[2];
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const int v = 2 * q + h;
+        uint32_t fb;
+        if (i == 1) fb = 0x4B000000u | (th[v] >> 16);
+        else if (i <= 3) fb = __byte_perm(th[v], 0x4B00u, 0x5440u | (uint32_t)(3 - i));
+        else fb = __byte_perm(tl[v], 0x4B00u, 0x5440u | (uint32_t)(7 - i));
+        d[h] = __uint_as_float(fb) - 8388736.0f;
+      }
+      hw[q] = oz_pack2(d[0], d[1]);
+    }
+    *reinterpret_cast<uint4 *>(dst + (i - 1) * STRIDE) = make_uint4(hw[0], hw[1], hw[2], hw[3]);
+  }
+}
+
+// B digits, once per plan: [mat][column tile of 64][K stage][digit][64 x 16]; the matrices as in
+// oz_pack_b_kernel.  One thread per 8 consecutive K values of one output column.
+__global__ void ow_pack_b_kernel(const double *m0, int k0n, int n0n, int ld0, const double *m1, int k1n, int n1n,
+                                 int ld1, int nk, int nnt, int eB, uint8_t *out) {
+  const int which = blockIdx.z;
+  const int n = blockIdx.x * blockDim.x + threadIdx.x;  // consecutive columns: coalesced reads
+  const int ch = blockIdx.y;
+  if (n >= nnt * OW_N || ch >= 2 * nk) return;
+  const double *m = which ? m1 : m0;
+  const int kn = which ? k1n : k0n, nn = which ? n1n : n0n, ld = which ? ld1 : ld0;
+  long long T[8];
+#pragma unroll
+  for (int q = 0; q < 8; ++q) {
+    const int k = ch * 8 + q;
+    T[q] = (n < nn && k < kn) ? ow_fixed(m[(size_t)k * ld + n], eB) : 0;
+  }
+  uint8_t *base = out + (((size_t)which * nnt + n / OW_N) * nk + (ch >> 1)) * OW_B;
+  ow_store_digits<OW_BSL>(T, base + ow_swz(n % OW_N, ch & 1));
+}
+
+// A digits per apply: one CTA per row, both parities, as oz_pack_a_kernel (row staged in shared memory,
+// row exponent from the largest |input|, fold as exact integer sums).
+// Layout [parity][m tile][K stage][digit][128 x 16]; erow[parity][row].
+__global__ void __launch_bounds__(OZ_PACK_THREADS) ow_pack_a_kernel(const double *__restrict__ x, int rows, int n,
+                                                                    int ku, int kv, int nk, int nmt,
+                                                                    uint8_t *__restrict__ out, int *__restrict__ erow,
+                                                                    const KrylovScalars *__restrict__ sc, int rpr,
+                                                                    int gather) {
+  extern __shared__ double xs[];  // the row's n inputs at OZ_PAD(j)
+  const int row = blockIdx.x;
+  // rows of finished right-hand sides keep whatever digits they had (bounded integers; nothing reads
+  // those rows' outputs any more)
+  if (row < rows && sc != nullptr && sc[row / rpr].state != ST_RUN) return;
+  const bool live = row < rows;  // the padding rows of the last tile pack as zeros
+  const double *xr = x + (size_t)(live ? row : 0) * n;
+  unsigned long long b0 = 0, b1 = 0;
+  constexpr int PB = 16;  // a batch of loads all issue before any is used
+  for (int jb = 0; jb < n; jb += PB * OZ_PACK_THREADS) {
+    double vb[PB];
+#pragma unroll
+    for (int u = 0; u < PB; ++u) {
+      const int j = jb + u * OZ_PACK_THREADS + threadIdx.x;
+      vb[u] = (live && j < n) ? __ldg(xr + j) : 0.0;
+    }
+#pragma unroll
+    for (int u = 0; u < PB; ++u) {
+      const int j = jb + u * OZ_PACK_THREADS + threadIdx.x;
+      if (j < n) {
+        xs[OZ_PAD(j)] = vb[u];
+        const unsigned long long m = (unsigned long long)__double_as_longlong(vb[u]) & 0x7fffffffffffffffull;
+        if (gather && (j & 1)) b1 = max(b1, m);
+        else b0 = max(b0, m);
+      }
+    }
+  }
+  __shared__ unsigned long long red[2][OZ_PACK_THREADS / 32];
+  for (int o = 16; o > 0; o >>= 1) {
+    b0 = max(b0, __shfl_xor_sync(0xffffffffu, b0, o));
+    b1 = max(b1, __shfl_xor_sync(0xffffffffu, b1, o));
+  }
+  if ((threadIdx.x & 31) == 0) {
+    red[0][threadIdx.x >> 5] = b0;
+    red[1][threadIdx.x >> 5] = b1;
+  }
+  __syncthreads();
+  int e[2];
+#pragma unroll
+  for (int par = 0; par < 2; ++par) {
+    unsigned long long m = 0;
+#pragma unroll
+    for (int w = 0; w < OZ_PACK_THREADS / 32; ++w) m = max(m, red[gather ? par : 0][w]);
+    const int E = (int)(m >> 52);
+    // |inputs| <= m < 2^(E - 1022) for normal m, < 2^-1022 for subnormal m; 0 for a zero row; the
+    // fold's sums and differences of two inputs stay below 2^(that + 1)
+    e[par] = (E == 0x7ff) ? OZ_EXP_NAN : (m == 0 ? 0 : (E == 0 ? -1022 : E - 1022) + (gather ? 0 : 1));
+  }
+  // a non-finite value anywhere in the row makes every output of the row non-finite
+  const bool bad = e[0] == OZ_EXP_NAN || e[1] == OZ_EXP_NAN;
+  if (threadIdx.x < 2 && live)
+    erow[threadIdx.x * (nmt * TM) + row] = bad ? OZ_EXP_NAN : (threadIdx.x ? e[1] : e[0]);
+  const int mt = row / TM, r = row % TM;
+  const bool odd_n = (n & 1) != 0;
+  for (int ch = threadIdx.x; ch < 2 * nk; ch += OZ_PACK_THREADS) {
+    long long U[8], W[8];
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+      const int j = ch * 8 + q;
+      long long u = 0, w = 0;
+      if (!bad) {
+        if (gather) {
+          if (j < ku) u = ow_fixed(xs[OZ_PAD(2 * j)], e[0]);
+          if (j < kv) w = ow_fixed(xs[OZ_PAD(2 * j + 1)], e[1]);
+        } else if (j < kv) {
+          const long long a1 = ow_fixed(xs[OZ_PAD(j)], e[0]), a2 = ow_fixed(xs[OZ_PAD(n - 1 - j)], e[0]);
+          u = a1 + a2;
+          w = a1 - a2;
+        } else if (odd_n && j == ku - 1) {
+          u = ow_fixed(xs[OZ_PAD(j)], e[0]);  // middle element of an odd-length row
+        }
+      }
+      U[q] = u;
+      W[q] = w;
+    }
+    uint8_t *t0 = out + ((size_t)mt * nk + (ch >> 1)) * OW_A + ow_swz(r, ch & 1);
+    ow_store_digits<OW_ASL>(U, t0);
+    ow_store_digits<OW_ASL>(W, t0 + (size_t)nmt * nk * OW_A);
+  }
+}
+
+// shared-memory descriptor constant bits: K-major SWIZZLE_32B, 8-row groups 256 bytes apart
+constexpr uint64_t OW_DHI = ((uint64_t)(256 >> 4) << 32) | (1ull << 46) | (6ull << 61) | (1ull << 16);
+constexpr uint32_t ow_idesc(int n) {
+  return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(TM >> 4) << 24);
+}
+__device__ __forceinline__ void ow_mma(uint32_t d, uint64_t a, uint64_t b, uint32_t idesc) {
+  asm volatile("{\n .reg .pred p;\n setp.ne.b32 p, 1, 0;\n tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(d),
+               "l"(a), "l"(b), "r"(idesc)
+               : "memory");
+}
+// A digit I (0-based) times the LEN B digits that meet it in weights W0 .. (0-based: w - 2)
+template <int I, int W0, int LEN>
+__device__ __forceinline__ void ow_mmas(uint32_t tmem, uint32_t sa, uint32_t sb) {
+  ow_mma(tmem + (uint32_t)(W0 * OW_N), OW_DHI | (sa + I * (OW_ASL >> 4)), OW_DHI | (sb + (W0 - I) * (OW_BSL >> 4)),
+         ow_idesc(LEN * OW_N));
+}
+// all 28 products, narrow ones first
+__device__ __forceinline__ void ow_issue_all(uint32_t tmem, uint32_t sa, uint32_t sb) {
+  ow_mmas<6, 6, 1>(tmem, sa, sb);
+  ow_mmas<5, 5, 2>(tmem, sa, sb);
+  ow_mmas<4, 4, 3>(tmem, sa, sb);
+  ow_mmas<2, 2, 3>(tmem, sa, sb);
+  ow_mmas<2, 5, 2>(tmem, sa, sb);
+  ow_mmas<1, 5, 2>(tmem, sa, sb);
+  ow_mmas<0, 4, 3>(tmem, sa, sb);
+  ow_mmas<1, 1, 4>(tmem, sa, sb);
+  ow_mmas<0, 0, 4>(tmem, sa, sb);
+  ow_mmas<3, 3, 4>(tmem, sa, sb);
+}
+// the products of one group of weights
+template <int G>
+__device__ __forceinline__ void ow_issue_group(uint32_t tmem, uint32_t sa, uint32_t sb) {
+  if constexpr (G == 0) {  // weights 2, 3, 4
+    ow_mmas<2, 2, 1>(tmem, sa, sb);
+    ow_mmas<1, 1, 2>(tmem, sa, sb);
+    ow_mmas<0, 0, 3>(tmem, sa, sb);
+  } else if constexpr (G == 1) {  // 5, 6
+    ow_mmas<4, 4, 1>(tmem, sa, sb);
+    ow_mmas<3, 3, 2>(tmem, sa, sb);
+    ow_mmas<2, 3, 2>(tmem, sa, sb);
+    ow_mmas<1, 3, 2>(tmem, sa, sb);
+    ow_mmas<0, 3, 2>(tmem, sa, sb);
+  } else {  // 7, 8
+    ow_mmas<6, 6, 1>(tmem, sa, sb);
+    ow_mmas<5, 5, 2>(tmem, sa, sb);
+    ow_mmas<4, 5, 2>(tmem, sa, sb);
+    ow_mmas<3, 5, 2>(tmem, sa, sb);
+    ow_mmas<2, 5, 2>(tmem, sa, sb);
+    ow_mmas<1, 5, 2>(tmem, sa, sb);
+    ow_mmas<0, 5, 2>(tmem, sa, sb);
+  }
+}
+__device__ __forceinline__ void ow_commit(uint32_t bar) {
+  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
+}
+
+// 32 columns of zeros for this warp's 32 lanes
+__device__ __forceinline__ void ow_tmem_zero32(uint32_t taddr) {
+  asm volatile(
+      "tcgen05.st.sync.aligned.32x32b.x32.b32 [%0], {%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,"
+      "%1,%1,%1,%1,%1,%1,%1,%1,%1,%1};\n" ::"r"(taddr),
+      "r"(0)
+      : "memory");
+}
+
+// acc += the weight's sums (integers G, or FP32-rounded ones for the tail) in units of 2^-OW_FIX
+template <int W>
+__device__ __forceinline__ void ow_add(const float (&v)[32], long long (&acc)[32]) {
+  constexpr int sh = OW_FIX - 8 * (W - 2);
+  if constexpr (sh >= 32) {
+#pragma unroll
+    for (int q = 0; q < 32; ++q) acc[q] += (long long)__float2int_rz(v[q]) << sh;
+  } else if constexpr (sh >= 0) {
+#pragma unroll
+    for (int q = 0; q < 32; ++q) acc[q] += (long long)__float2int_rz(v[q]) * (1 << sh);
+  } else {
+    constexpr float s = 1.0f / (float)(1 << -sh);
+#pragma unroll
+    for (int q = 0; q < 32; ++q) acc[q] += (long long)__float2int_rn(v[q] * s);
+  }
+}
+
+// Persistent warp-specialised GEMM over (parity, m tile, 64-column tile): warp 0 streams the stages
+// (two bulk copies each), warp 1 issues the MMAs, warps 2-9 drain (warp w: rows 32 (w % 4).., columns
+// 32 ((w - 2) / 4).. of every weight) and store the tile, its rows transposed through shared memory.
+__global__ void __launch_bounds__(320, 1) oz_wgemm_kernel(const uint8_t *__restrict__ apack,
+                                                          const uint8_t *__restrict__ bpack,
+                                                          const int *__restrict__ erow, int eB, int nk, int nmt, int nnt,
+                                                          int rows, double *__restrict__ y, int ld, int ku, int kv,
+                                                          const KrylovScalars *__restrict__ sc, int rpr,
+                                                          int *__restrict__ err, int inv) {
+  extern __shared__ uint8_t smem_raw[];
+  const uint32_t raw = smem_u32(smem_raw);
+  const uint32_t base = (raw + 1023u) & ~1023u;
+  uint8_t *gbase = smem_raw + (base - raw);
+  constexpr int BAR_OFF = OW_NST * OW_STAGE + 8 * OW_TBUF;
+  const uint32_t full0 = base + BAR_OFF, empty0 = full0 + 8 * OW_NST, tfull0 = empty0 + 8 * OW_NST, tempty0 = tfull0 + 24;
+  volatile uint32_t *holder = reinterpret_cast<volatile uint32_t *>(gbase + BAR_OFF + 16 * OW_NST + 48);
+  volatile int *abort_flag = reinterpret_cast<volatile int *>(gbase + BAR_OFF + 16 * OW_NST + 56);
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int ntiles = 2 * nmt * nnt;
+
+  if (warp == 0) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32((const void *)holder)),
+                 "r"(OW_TMEM)
+                 : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+  }
+  if (tid == 32) {
+    for (int s = 0; s < OW_NST; ++s) {
+      mbar_init(full0 + 8 * s, 1);
+      mbar_init(empty0 + 8 * s, 1);
+    }
+    for (int g = 0; g < 3; ++g) {
+      mbar_init(tfull0 + 8 * g, 1);
+      mbar_init(tempty0 + 8 * g, 8);  // one arrive per epilogue warp
+    }
+    *abort_flag = 0;
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  __syncthreads();
+  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+  const uint32_t tmem = *holder;
+
+  auto decode = [&](int t, int &par, int &mt, int &nt) {
+    nt = t % nnt;
+    mt = (t / nnt) % nmt;
+    par = t / (nnt * nmt);
+  };
+  auto wanted = [&](int par, int mt, int nt) -> bool {
+    if (nt * OW_N >= ((par && !inv) ? kv : ku)) return false;
+    if (mt * TM >= rows) return false;
+    if (sc == nullptr) return true;
+    const int m0 = mt * TM;
+    const int r0 = m0 / rpr, r1 = (min(m0 + TM, rows) - 1) / rpr;
+    for (int r = r0; r <= r1; ++r)
+      if (sc[r].state == ST_RUN) return true;
+    return false;
+  };
+
+  if (warp == 0) {
+    if (lane == 0) {  // producer
+      int s = 0, it = 0;
+      uint32_t ph = 0;
+      for (int t = blockIdx.x; t < ntiles && !*abort_flag; t += gridDim.x) {
+        int par, mt, nt;
+        decode(t, par, mt, nt);
+        if (!wanted(par, mt, nt)) continue;
+        const uint8_t *at = apack + ((size_t)par * nmt + mt) * nk * OW_A;
+        const uint8_t *bt = bpack + ((size_t)par * nnt + nt) * nk * OW_B;
+        for (int k = 0; k < nk; ++k) {
+          if (it >= OW_NST && !mbar_wait(empty0 + 8 * s, ph ^ 1u)) {
+            atomicExch(err, 11);
+            *abort_flag = 1;
+            break;
+          }
+          const uint32_t st = base + s * OW_STAGE, fb = full0 + 8 * s;
+          mbar_expect_tx(fb, (uint32_t)OW_STAGE);
+          bulk_g2s(st, at + (size_t)k * OW_A, OW_A, fb);
+          bulk_g2s(st + OW_A, bt + (size_t)k * OW_B, OW_B, fb);
+          ++it;
+          if (++s == OW_NST) {
+            s = 0;
+            ph ^= 1u;
+          }
+        }
+      }
+      // after an abort nobody has waited for the last copies: no CTA leaves with copies in flight
+      if (*abort_flag)
+        for (int i = max(0, it - OW_NST); i < it; ++i) mbar_wait(full0 + 8 * (i % OW_NST), (uint32_t)(i / OW_NST) & 1u);
+    }
+  } else if (warp == 1) {
+    if (lane == 0) {  // MMA issuer
+      int s = 0;
+      uint32_t ph = 0, eph = 0;  // eph: next parity of each group's tempty barrier
+      uint32_t pend = 7u;        // groups handed to the epilogue and not seen back (at first: to be zeroed)
+      for (int t = blockIdx.x; t < ntiles && !*abort_flag; t += gridDim.x) {
+        int par, mt, nt;
+        decode(t, par, mt, nt);
+        if (!wanted(par, mt, nt)) continue;
+        for (int k = 0; k < nk; ++k) {
+          if (!mbar_wait(full0 + 8 * s, ph)) {
+            atomicExch(err, 12);
+            *abort_flag = 1;
+            break;
+          }
+          asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+          const uint32_t sa = (base + s * OW_STAGE) >> 4, sb = sa + (OW_A >> 4);
+          const bool last = k + 1 == nk;
+          if (pend == 0 && !last) {
+            ow_issue_all(tmem, sa, sb);
+          } else {
+            // groups at rest first, then those the epilogue still drains; on a tile's last stage each
+            // group goes to the epilogue as soon as its products are issued
+            bool ok = true;
+            const uint32_t was = pend;
+            auto rest = [&](auto g) {
+              constexpr int G = decltype(g)::value;
+              if ((was >> G) & 1u) return;
+              ow_issue_group<G>(tmem, sa, sb);
+              if (last) ow_commit(tfull0 + 8 * G);
+            };
+            auto busy = [&](auto g) {
+              constexpr int G = decltype(g)::value;
+              if (!((was >> G) & 1u)) return;
+              ok = mbar_wait(tempty0 + 8 * G, (eph >> G) & 1u) && ok;
+              eph ^= 1u << G;
+              asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+              ow_issue_group<G>(tmem, sa, sb);
+              if (last) ow_commit(tfull0 + 8 * G);
+            };
+            rest(std::integral_constant<int, 0>());
+            rest(std::integral_constant<int, 1>());
+            rest(std::integral_constant<int, 2>());
+            busy(std::integral_constant<int, 0>());
+            busy(std::integral_constant<int, 1>());
+            busy(std::integral_constant<int, 2>());
+            if (!ok) {
+              atomicExch(err, 14);
+              *abort_flag = 1;
+              break;
+            }
+          }
+          ow_commit(empty0 + 8 * s);
+          pend = last ? 7u : (ow_bit(OW_E0, k + 1) | ow_bit(OW_E1, k + 1) << 1 | ow_bit(OW_E2, k + 1) << 2);
+          if (pend != 0 && !last) {
+            if (pend & 1u) ow_commit(tfull0);
+            if (pend & 2u) ow_commit(tfull0 + 8);
+            if (pend & 4u) ow_commit(tfull0 + 16);
+          }
+          if (++s == OW_NST) {
+            s = 0;
+            ph ^= 1u;
+          }
+        }
+      }
+    }
+  } else {  // epilogue warps 2..9
+    const int lg = warp & 3, h = (warp - 2) >> 2;
+    const uint32_t tw = tmem + ((uint32_t)(lg * 32) << 16) + (uint32_t)(h * 32);  // + 64 (w - 2)
+    double *tbuf = reinterpret_cast<double *>(gbase + OW_NST * OW_STAGE + (warp - 2) * OW_TBUF);
+    auto hand_back = [&](int g) {
+      asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+      asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+      __syncwarp();
+      if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(tempty0 + 8 * g) : "memory");
+    };
+#pragma unroll
+    for (int w = 0; w < OW_NS; ++w) ow_tmem_zero32(tw + w * OW_N);
+    for (int g = 0; g < 3; ++g) hand_back(g);
+    uint32_t fph = 0;  // next parity of each group's tfull barrier
+    for (int t = blockIdx.x; t < ntiles; t += gridDim.x) {
+      int par, mt, nt;
+      decode(t, par, mt, nt);
+      if (!wanted(par, mt, nt)) continue;
+      const int row = mt * TM + lg * 32 + lane;
+      const int e = row < rows ? erow[par * (nmt * TM) + row] : 0;
+      long long acc[32];
+#pragma unroll
+      for (int q = 0; q < 32; ++q) acc[q] = 0;
+      bool stop = false;
+      for (int c = 1; c <= nk; ++c) {
+        const bool last = c == nk;
+        if (!last && !ow_bit(OW_E0 | OW_E1 | OW_E2, c)) continue;
+        // a group's accumulators: at most two weights in registers at a time, handed back before the
+        // last ones are added up
+        auto wait_group = [&](int g) {
+          const bool ok = mbar_wait(tfull0 + 8 * g, (fph >> g) & 1u);
+          fph ^= 1u << g;
+          __syncwarp();
+          if (!ok) {
+            if (lane == 0) atomicExch(err, 13);
+            *abort_flag = 1;
+            stop = true;
+          }
+          asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+          return ok;
+        };
+        float va[32], vb[32];
+        auto take = [&](int w, float (&v)[32]) {
+          tmem_ld32(tw + (w - 2) * OW_N, v);
+          ow_tmem_zero32(tw + (w - 2) * OW_N);
+        };
+        if ((last || ow_bit(OW_E0, c)) && !stop && wait_group(0)) {
+          if (last) {
+            take(2, va);
+            ow_add<2>(va, acc);
+          }
+          take(3, va);
+          take(4, vb);
+          hand_back(0);
+          ow_add<3>(va, acc);
+          ow_add<4>(vb, acc);
+        }
+        if ((last || ow_bit(OW_E1, c)) && !stop && wait_group(1)) {
+          take(5, va);
+          take(6, vb);
+          hand_back(1);
+          ow_add<5>(va, acc);
+          ow_add<6>(vb, acc);
+        }
+        if ((last || ow_bit(OW_E2, c)) && !stop && wait_group(2)) {
+          take(7, va);
+          if (last) take(8, vb);
+          hand_back(2);
+          ow_add<7>(va, acc);
+          if (last) ow_add<8>(vb, acc);
+        }
+        if (stop) break;
+      }
+      if (stop) break;
+      // the one float64 rounding: int64 -> float64, then exact power-of-two scales (added to the
+      // exponent field where every result of the row is a normal float64)
+      const int kx = e + eB - 2 * 7 - OW_FIX;
+      const bool fast = __all_sync(0xffffffffu, oz_fast_row(e, kx));  // a branch of the whole warp
+      const int c0 = nt * OW_N + h * 32;
+      const int ncols = min(32, ((par && !inv) ? kv : ku) - c0);
+      const int r0 = mt * TM + lg * 32;
+      const int nr = min(32, rows - r0);
+      const int ys = inv ? 1 : 2;
+      double *yt = y + (inv ? ((size_t)par * rows + r0) * ku + c0 : (size_t)r0 * ld + par + 2 * (size_t)c0);
+      const size_t ystep = inv ? (size_t)ku : (size_t)ld;
+#pragma unroll
+      for (int half = 0; half < 2; ++half) {
+        if (fast) {
+          // half of the values on the FP64 pipe, half on the integer pipe (the same bits)
+#pragma unroll
+          for (int q = 0; q < 16; q += 2) {
+            const long long db = __double_as_longlong(__ll2double_rn(acc[half * 16 + q]));
+            tbuf[lane * OW_TPITCH + q] = __longlong_as_double(db == 0 ? 0ll : db + ((long long)kx << 52));
+            tbuf[lane * OW_TPITCH + q + 1] = oz_to_f64(acc[half * 16 + q + 1], kx);
+          }
+        } else {
+          const double scale = e == OZ_EXP_NAN ? __longlong_as_double(0x7ff8000000000000ll) : ldexp(1.0, e + eB - 2 * 7);
+          const double unit = 1.0 / (double)(1LL << OW_FIX);
+#pragma unroll
+          for (int q = 0; q < 16; ++q) tbuf[lane * OW_TPITCH + q] = scale * (unit * __ll2double_rn(acc[half * 16 + q]));
+        }
+        __syncwarp();
+        const int cq = lane & 15, col = half * 16 + cq;
+#pragma unroll
+        for (int rr = 0; rr < 32; rr += 2) {
+          const int r = rr + (lane >> 4);
+          if (r < nr && col < ncols) yt[(size_t)r * ystep + (size_t)ys * col] = tbuf[r * OW_TPITCH + cq];
+        }
+        __syncwarp();
+      }
+    }
+  }
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  __syncthreads();
+  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+  if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(OW_TMEM) : "memory");
+}
