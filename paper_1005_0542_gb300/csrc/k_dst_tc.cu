@@ -2716,12 +2716,26 @@ static void oz_launch_mc(const uint8_t *apack, size_t a_slice, const uint8_t *bp
                                     inv));
 }
 
+static int ow_tiles(const DstPlan &dp, int nmt, int n, int inv) {
+  return nmt * (div_up(dp.ku, n) + div_up(inv ? dp.ku : dp.kv, n));
+}
+template <int N>
+static void ow_gemm_launch(const DstPlan &dp, const uint8_t *apack, const int *erow, int nk, int nmt, int nnt, int rows,
+                           double *y, const KrylovScalars *sc, int rpr, int inv, cudaStream_t s) {
+  static PerDeviceOnce attr;
+  attr.run([] {
+    LAG_CUDA_CHECK(cudaFuncSetAttribute(oz_wgemm_kernel<N>, cudaFuncAttributeMaxDynamicSharedMemorySize, OwCfg<N>::SMEM));
+  });
+  const int tiles = ow_tiles(dp, nmt, N, inv);
+  oz_wgemm_kernel<N><<<std::min(tiles, device_sms()), 320, OwCfg<N>::SMEM, s>>>(
+      apack, inv ? dp.ow_bi : dp.ow_b, erow, dp.oz_eB, nk, nmt, nnt, rows, y, dp.n, dp.ku, dp.kv, sc, rpr, dp.tc_err, inv);
+}
+
 // the weight-stacked kernel (8-bit format, no opt-in variant)
 static void ow_apply(const DstPlan &dp, const double *x, double *y, int rows, int rpr, const KrylovScalars *sc,
                      cudaStream_t s, int inv) {
   static PerDeviceOnce attr;
   attr.run([] {
-    LAG_CUDA_CHECK(cudaFuncSetAttribute(oz_wgemm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, OW_SMEM));
     LAG_CUDA_CHECK(cudaFuncSetAttribute(ow_pack_a_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                         (int)oz_pack_smem(OZ_PACK_MAXK / TK + 1)));
   });
@@ -2735,9 +2749,12 @@ static void ow_apply(const DstPlan &dp, const double *x, double *y, int rows, in
                                                                               apack, erow, sc, rpr, inv);
   count_launch();
   LAG_LAUNCH_CHECK();
-  oz_wgemm_kernel<<<std::min(2 * nmt * nnt, device_sms()), 320, OW_SMEM, s>>>(
-      apack, inv ? dp.ow_bi : dp.ow_b, erow, dp.oz_eB, nk, nmt, nnt, rows, inv ? eo : y, dp.n, dp.ku, dp.kv, sc, rpr,
-      dp.tc_err, inv);
+  // the narrowest tiles that still run in one wave (see OwCfg)
+  double *yo = inv ? eo : y;
+  const int sms = device_sms();
+  if (ow_tiles(dp, nmt, 16, inv) <= sms) ow_gemm_launch<16>(dp, apack, erow, nk, nmt, nnt, rows, yo, sc, rpr, inv, s);
+  else if (ow_tiles(dp, nmt, 32, inv) <= sms) ow_gemm_launch<32>(dp, apack, erow, nk, nmt, nnt, rows, yo, sc, rpr, inv, s);
+  else ow_gemm_launch<64>(dp, apack, erow, nk, nmt, nnt, rows, yo, sc, rpr, inv, s);
   count_launch();
   LAG_LAUNCH_CHECK();
   if (inv) {

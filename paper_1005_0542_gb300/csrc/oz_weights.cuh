@@ -8,13 +8,16 @@
 // bounds it (59 B/clk measured).  Here a stage holds ALL seven digit tiles of both operands for 16
 // values of K, each crosses once (21 tile halves for the same 28 products: 47 B/clk at the tensor
 // pipe's full rate), and every weight w = i + j keeps its own 64-column accumulator:
-//   * tile 128 rows x 64 columns; accumulator of weight w = 2..8 at tensor-memory column 64 (w - 2);
+//   * tile 128 rows x 64 columns (N below: 32 or 16 for small transforms); accumulator of weight w =
+//     2..8 at tensor-memory column 64 (w - 2);
 //   * the B digits lie behind one another in shared memory (64 rows each), so A_i x [B_j .. B_j+m-1]
 //     is ONE tcgen05.mma of N = 64 m whose column blocks are the m consecutive weights i + j ..:
 //     ten MMAs of 64..256 columns per K step do the 28 products in 908 clocks (896 at the tensor
 //     pipe's peak).  They are issued narrow ones first: the three 256-column ones at the end of a
 //     stage keep the pipe busy while the issuer commits the stage and waits for the next one
-//     (the other way round the pipe idled 75 - 275 clocks per stage);
+//     (the other way round the pipe idled 75 - 275 clocks per stage).  The issuing loop is uniform over
+//     its warp with one elected lane issuing (256 against 265 us as a one-lane branch: descriptors stay in
+//     uniform registers);
 //   * weight w sums w - 1 products per K value, each at most 2^14, so it stays exact (up to 2^24)
 //     for 1024 / (w - 1) values of K; eight epilogue warps drain it in time (ow_drain) into int64
 //     sums held in registers and zero it.  Drains go by group of weights ({2,3,4}, {5,6}, {7,8}), each
@@ -26,21 +29,32 @@
 // expansions are rounded to nearest at 2^-55 instead of truncated (row errors against extended
 // precision 2.1e-16 - 2.8e-16 on random rows of 40..2048 values, 2.2e-16 - 3.7e-16 with truncation).
 // Measured, whole preconditioner applies (two transforms each), tile kernel -> this one: 1024 x 1024 x
-// 256 right-hand sides 21.1 -> 14.3 ms, 2048 x 1024 x 1 287 -> 257 us, 63 x 40 65.6 -> 45.1 us.
+// 256 right-hand sides 21.1 -> 14.2 ms, 2048 x 1024 x 1 287 -> 254 us, 63 x 40 65.6 -> 35 us (45 with
+// 64-column tiles only).
 constexpr int OW_NS = 7;                          // digits per operand
 constexpr int OW_K = 16;                          // K values per stage (one MMA K step)
-constexpr int OW_N = 64;                          // output columns per tile
+constexpr int OW_N = 64;                          // columns of a packed B tile
 constexpr int OW_ASL = TM * OW_K * 2;             // one A digit of a stage: 128 rows of 32 bytes
-constexpr int OW_BSL = OW_N * OW_K * 2;           // one B digit of a stage: 64 rows of 32 bytes
+constexpr int OW_BSL = OW_N * OW_K * 2;           // one digit of a packed B tile: 64 rows of 32 bytes
 constexpr int OW_A = OW_NS * OW_ASL;              // 28 KB
 constexpr int OW_B = OW_NS * OW_BSL;              // 14 KB
-constexpr int OW_STAGE = OW_A + OW_B;
-constexpr int OW_NST = 4;                         // three stages in flight: 2.7 k clocks of MMAs
-constexpr int OW_TPITCH = 17;                     // doubles per row of a warp's transposition buffer
-constexpr int OW_TBUF = 32 * OW_TPITCH * 8;       // per epilogue warp: 32 rows x 16 columns
-constexpr int OW_SMEM = OW_NST * OW_STAGE + 8 * OW_TBUF + 1024 + 256;
-constexpr uint32_t OW_TMEM = 512;                 // allocated columns (7 x 64 used)
 constexpr int OW_FIX = 38;                        // sums in units of 2^-38 of a weight-2 unit
+// Tiles of N = 64, 32 or 16 columns (a packed B tile or its halves / quarters).  A tile's time is its
+// MMAs plus a tail that grows with N (the last drains, the conversion and the store: 12 k clocks at
+// N = 64), so transforms whose tiles leave SMs idle anyway take the narrowest tile that still runs in
+// one wave; above one wave N = 64 (N = 32: 496 clocks a K step for half of the 908's work).
+template <int N>
+struct OwCfg {
+  static constexpr int BSL = N * OW_K * 2;
+  static constexpr int STAGE = OW_A + OW_NS * BSL;
+  static constexpr int NST = N == 64 ? 4 : (N == 32 ? 5 : 6);
+  static constexpr int CW = N / 2;                 // columns per epilogue warp (of each weight)
+  static constexpr int CH = CW < 16 ? CW : 16;     // columns transposed at a time
+  static constexpr int TPITCH = CH + 1;            // doubles per row of a warp's transposition buffer
+  static constexpr int TBUF = 32 * TPITCH * 8;
+  static constexpr uint32_t TMEM = N == 64 ? 512 : (N == 32 ? 256 : 128);  // allocated columns (7 N used)
+  static constexpr int SMEM = NST * STAGE + 8 * TBUF + 1024 + 256;
+};
 
 // element (r, k) of a rows x 16 digit tile: 32-byte rows, K-major SWIZZLE_32B (byte offset)
 __device__ __forceinline__ uint32_t ow_swz(int r, int kchunk) {
@@ -49,12 +63,12 @@ __device__ __forceinline__ uint32_t ow_swz(int r, int kchunk) {
 
 // Stages after which a group of weights is drained (bit c: after c stages of a tile of nk <= 64; every
 // group at the tile's end).  Exactness allows weight 3 32 stages (2 x 512 x 2^14 = 2^24), 4 20, 5 16,
-// 6 12; a drain costs the MMA stream about 700 clocks (narrower MMAs, a commit and a wait on the
-// issuing thread), so the weights of a group go together, at stages no two groups share; none
-// before stage 12, while the epilogue warps still convert and store the previous tile.
-constexpr unsigned long long OW_E0 = (1ull << 18) | (1ull << 38) | (1ull << 58);                            // 3, 4
+// 6 12; a drain costs the MMA stream about 1000 clocks (commit, hand-over, hand-back, the pipe refilling),
+// so the weights of a group go together and groups share stages where they can (60, 40; 14.18 against
+// 14.31 ms for 1024 x 1024 x 256 with 3, 4 at 18, 38, 58 and 7 at 30).
+constexpr unsigned long long OW_E0 = (1ull << 20) | (1ull << 40) | (1ull << 60);                            // 3, 4
 constexpr unsigned long long OW_E1 = (1ull << 12) | (1ull << 24) | (1ull << 36) | (1ull << 48) | (1ull << 60);  // 5, 6
-constexpr unsigned long long OW_E2 = 1ull << 30;                                                            // 7
+constexpr unsigned long long OW_E2 = 1ull << 40;                                                            // 7
 __device__ __forceinline__ uint32_t ow_bit(unsigned long long m, int c) { return (uint32_t)(m >> c) & 1u; }
 
 // rn(v 2^(55 - e)) for |v| < 2^e, signed (integer arithmetic on the bits); |result| <= 2^55
@@ -216,111 +230,176 @@ constexpr uint64_t OW_DHI = ((uint64_t)(256 >> 4) << 32) | (1ull << 46) | (6ull 
 constexpr uint32_t ow_idesc(int n) {
   return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(TM >> 4) << 24);
 }
+template <int ACC>
 __device__ __forceinline__ void ow_mma(uint32_t d, uint64_t a, uint64_t b, uint32_t idesc) {
-  asm volatile("{\n .reg .pred p;\n setp.ne.b32 p, 1, 0;\n tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(d),
-               "l"(a), "l"(b), "r"(idesc)
+  asm volatile("{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(d),
+               "l"(a), "l"(b), "r"(idesc), "n"(ACC)
                : "memory");
 }
-// A digit I (0-based) times the LEN B digits that meet it in weights W0 .. (0-based: w - 2)
-template <int I, int W0, int LEN>
+// A digit I (0-based) times the LEN B digits that meet it in weights W0 .. (0-based: w - 2); ACC 0 overwrites
+template <int N, int I, int W0, int LEN, int ACC = 1>
 __device__ __forceinline__ void ow_mmas(uint32_t tmem, uint32_t sa, uint32_t sb) {
-  ow_mma(tmem + (uint32_t)(W0 * OW_N), OW_DHI | (sa + I * (OW_ASL >> 4)), OW_DHI | (sb + (W0 - I) * (OW_BSL >> 4)),
-         ow_idesc(LEN * OW_N));
+  ow_mma<ACC>(tmem + (uint32_t)(W0 * N), OW_DHI | (sa + I * (OW_ASL >> 4)),
+              OW_DHI | (sb + (W0 - I) * (OwCfg<N>::BSL >> 4)), ow_idesc(LEN * N));
 }
 // all 28 products, narrow ones first
+template <int N>
 __device__ __forceinline__ void ow_issue_all(uint32_t tmem, uint32_t sa, uint32_t sb) {
-  ow_mmas<6, 6, 1>(tmem, sa, sb);
-  ow_mmas<5, 5, 2>(tmem, sa, sb);
-  ow_mmas<4, 4, 3>(tmem, sa, sb);
-  ow_mmas<2, 2, 3>(tmem, sa, sb);
-  ow_mmas<2, 5, 2>(tmem, sa, sb);
-  ow_mmas<1, 5, 2>(tmem, sa, sb);
-  ow_mmas<0, 4, 3>(tmem, sa, sb);
-  ow_mmas<1, 1, 4>(tmem, sa, sb);
-  ow_mmas<0, 0, 4>(tmem, sa, sb);
-  ow_mmas<3, 3, 4>(tmem, sa, sb);
-}
-// the products of one group of weights
-template <int G>
-__device__ __forceinline__ void ow_issue_group(uint32_t tmem, uint32_t sa, uint32_t sb) {
-  if constexpr (G == 0) {  // weights 2, 3, 4
-    ow_mmas<2, 2, 1>(tmem, sa, sb);
-    ow_mmas<1, 1, 2>(tmem, sa, sb);
-    ow_mmas<0, 0, 3>(tmem, sa, sb);
-  } else if constexpr (G == 1) {  // 5, 6
-    ow_mmas<4, 4, 1>(tmem, sa, sb);
-    ow_mmas<3, 3, 2>(tmem, sa, sb);
-    ow_mmas<2, 3, 2>(tmem, sa, sb);
-    ow_mmas<1, 3, 2>(tmem, sa, sb);
-    ow_mmas<0, 3, 2>(tmem, sa, sb);
-  } else {  // 7, 8
-    ow_mmas<6, 6, 1>(tmem, sa, sb);
-    ow_mmas<5, 5, 2>(tmem, sa, sb);
-    ow_mmas<4, 5, 2>(tmem, sa, sb);
-    ow_mmas<3, 5, 2>(tmem, sa, sb);
-    ow_mmas<2, 5, 2>(tmem, sa, sb);
-    ow_mmas<1, 5, 2>(tmem, sa, sb);
-    ow_mmas<0, 5, 2>(tmem, sa, sb);
+  ow_mmas<N, 6, 6, 1>(tmem, sa, sb);
+  ow_mmas<N, 5, 5, 2>(tmem, sa, sb);
+  ow_mmas<N, 4, 4, 3>(tmem, sa, sb);
+  if constexpr (N == 64) {
+    ow_mmas<N, 2, 2, 3>(tmem, sa, sb);
+    ow_mmas<N, 2, 5, 2>(tmem, sa, sb);
+    ow_mmas<N, 1, 5, 2>(tmem, sa, sb);
+    ow_mmas<N, 0, 4, 3>(tmem, sa, sb);
+    ow_mmas<N, 1, 1, 4>(tmem, sa, sb);
+    ow_mmas<N, 0, 0, 4>(tmem, sa, sb);
+    ow_mmas<N, 3, 3, 4>(tmem, sa, sb);
+  } else {
+    ow_mmas<N, 3, 3, 4>(tmem, sa, sb);
+    ow_mmas<N, 2, 2, 5>(tmem, sa, sb);
+    ow_mmas<N, 1, 1, 6>(tmem, sa, sb);
+    ow_mmas<N, 0, 0, 7>(tmem, sa, sb);
   }
+}
+// the products of one group of weights.  FIRST (a tile's first stage): the leading A digit, which meets
+// every weight, goes first and overwrites, which starts the group's sums afresh; else it goes last
+// (the widest MMA)
+template <int N, int G, bool FIRST>
+__device__ __forceinline__ void ow_issue_group(uint32_t tmem, uint32_t sa, uint32_t sb) {
+  constexpr int W0 = G == 0 ? 0 : (G == 1 ? 3 : 5), LEN = G == 0 ? 3 : 2;
+  if constexpr (FIRST) ow_mmas<N, 0, W0, LEN, 0>(tmem, sa, sb);
+  if constexpr (G == 0) {  // weights 2, 3, 4
+    ow_mmas<N, 2, 2, 1>(tmem, sa, sb);
+    ow_mmas<N, 1, 1, 2>(tmem, sa, sb);
+  } else if constexpr (G == 1) {  // 5, 6
+    ow_mmas<N, 4, 4, 1>(tmem, sa, sb);
+    ow_mmas<N, 3, 3, 2>(tmem, sa, sb);
+    ow_mmas<N, 2, 3, 2>(tmem, sa, sb);
+    ow_mmas<N, 1, 3, 2>(tmem, sa, sb);
+  } else {  // 7, 8
+    ow_mmas<N, 6, 6, 1>(tmem, sa, sb);
+    ow_mmas<N, 5, 5, 2>(tmem, sa, sb);
+    ow_mmas<N, 4, 5, 2>(tmem, sa, sb);
+    ow_mmas<N, 3, 5, 2>(tmem, sa, sb);
+    ow_mmas<N, 2, 5, 2>(tmem, sa, sb);
+    ow_mmas<N, 1, 5, 2>(tmem, sa, sb);
+  }
+  if constexpr (!FIRST) ow_mmas<N, 0, W0, LEN>(tmem, sa, sb);
+}
+__device__ __forceinline__ bool elect_one() {
+  uint32_t p;
+  asm volatile("{\n .reg .pred p;\n elect.sync _|p, 0xffffffff;\n selp.u32 %0, 1, 0, p;\n}\n" : "=r"(p));
+  return p != 0;
 }
 __device__ __forceinline__ void ow_commit(uint32_t bar) {
   asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
 }
 
-// 32 columns of zeros for this warp's 32 lanes
-__device__ __forceinline__ void ow_tmem_zero32(uint32_t taddr) {
-  asm volatile(
-      "tcgen05.st.sync.aligned.32x32b.x32.b32 [%0], {%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,"
-      "%1,%1,%1,%1,%1,%1,%1,%1,%1,%1};\n" ::"r"(taddr),
-      "r"(0)
-      : "memory");
+// C columns of this warp's 32 lanes: read, or set to zero
+template <int C>
+__device__ __forceinline__ void ow_tmem_ld(uint32_t taddr, float (&v)[C]) {
+  if constexpr (C == 32) {
+    tmem_ld32(taddr, v);
+  } else if constexpr (C == 16) {
+    tmem_ld16(taddr, v);
+  } else {
+    static_assert(C == 8, "columns per epilogue warp");
+    uint32_t r[8];
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];\n"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+                 : "r"(taddr));
+    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+    for (int i = 0; i < 8; ++i) v[i] = __uint_as_float(r[i]);
+  }
+}
+template <int C>
+__device__ __forceinline__ void ow_tmem_zero(uint32_t taddr) {
+  for (int c = 0; c < C; c += 8)
+    asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1,%1,%1,%1,%1,%1,%1,%1};\n" ::"r"(taddr + c), "r"(0)
+                 : "memory");
 }
 
 // acc += the weight's sums (integers G, or FP32-rounded ones for the tail) in units of 2^-OW_FIX
-template <int W>
-__device__ __forceinline__ void ow_add(const float (&v)[32], long long (&acc)[32]) {
+template <int W, int C>
+__device__ __forceinline__ void ow_add(const float (&v)[C], long long (&acc)[C]) {
   constexpr int sh = OW_FIX - 8 * (W - 2);
   if constexpr (sh >= 32) {
 #pragma unroll
-    for (int q = 0; q < 32; ++q) acc[q] += (long long)__float2int_rz(v[q]) << sh;
+    for (int q = 0; q < C; ++q) acc[q] += (long long)__float2int_rz(v[q]) << sh;
   } else if constexpr (sh >= 0) {
 #pragma unroll
-    for (int q = 0; q < 32; ++q) acc[q] += (long long)__float2int_rz(v[q]) * (1 << sh);
+    for (int q = 0; q < C; ++q) acc[q] += (long long)__float2int_rz(v[q]) * (1 << sh);
   } else {
     constexpr float s = 1.0f / (float)(1 << -sh);
 #pragma unroll
-    for (int q = 0; q < 32; ++q) acc[q] += (long long)__float2int_rn(v[q] * s);
+    for (int q = 0; q < C; ++q) acc[q] += (long long)__float2int_rn(v[q] * s);
   }
 }
 
-// Persistent warp-specialised GEMM over (parity, m tile, 64-column tile): warp 0 streams the stages
-// (two bulk copies each), warp 1 issues the MMAs, warps 2-9 drain (warp w: rows 32 (w % 4).., columns
-// 32 ((w - 2) / 4).. of every weight) and store the tile, its rows transposed through shared memory.
+// RN(v) 2^kx of an int64 v (|v| < 2^63, the result a normal float64 or zero) on 32-bit integer
+// operations: the bits of __ll2double_rn(v) with kx added to the exponent.  The FP64 pipe converts one
+// value per clock and SM at best; a quarter of the values there and the rest here took 3.5 k clocks for
+// a 128 x 64 tile's values against 4.6 k (all FP64) and 5.3 k (oz_to_f64's 64-bit form).
+__device__ __forceinline__ double ow_to_f64(long long v, int kx) {
+  const uint32_t sg = (uint32_t)(v >> 63);
+  const unsigned long long u = (unsigned long long)(v < 0 ? -v : v);
+  uint32_t hi = (uint32_t)(u >> 32), lo = (uint32_t)u;
+  int ef = 1022 + 63 + kx;
+  if (hi == 0) {
+    hi = lo;
+    lo = 0;
+    ef -= 32;
+  }
+  const int lz = __clz((int)hi);
+  hi = __funnelshift_l(lo, hi, lz);  // leading one at bit 63 of hi:lo
+  lo <<= (lz & 31);
+  // to nearest even at bit 11; a carry out of the top leaves a zero fraction one exponent up
+  const uint32_t l2 = lo + 0x3ffu + ((lo >> 11) & 1u);
+  const uint32_t c = l2 < lo ? 1u : 0u;
+  const uint32_t h2 = hi + c;
+  const uint32_t top = (c && h2 == 0) ? (1u << 21) : 0u;
+  const uint32_t rl = __funnelshift_r(l2, h2, 11);
+  const uint32_t rh = (h2 >> 11) + top + ((uint32_t)(ef - lz) << 20);
+  return hi == 0 ? 0.0 : __hiloint2double((int)(rh | (sg & 0x80000000u)), (int)rl);
+}
+
+// Persistent warp-specialised GEMM over (parity, m tile, N-column tile): warp 0 streams the stages,
+// warp 1 issues the MMAs, warps 2-9 drain (warp w: rows 32 (w % 4).., columns N/2 ((w - 2) / 4).. of every
+// weight) and store the tile, its rows transposed through shared memory.  nnt: packed 64-column B tiles.
+template <int N>
 __global__ void __launch_bounds__(320, 1) oz_wgemm_kernel(const uint8_t *__restrict__ apack,
                                                           const uint8_t *__restrict__ bpack,
                                                           const int *__restrict__ erow, int eB, int nk, int nmt, int nnt,
                                                           int rows, double *__restrict__ y, int ld, int ku, int kv,
                                                           const KrylovScalars *__restrict__ sc, int rpr,
                                                           int *__restrict__ err, int inv) {
+  using Cfg = OwCfg<N>;
+  constexpr int NST = Cfg::NST, STAGE = Cfg::STAGE, CW = Cfg::CW, CH = Cfg::CH, TPITCH = Cfg::TPITCH;
+  constexpr int SUB = OW_N / N;  // tiles per packed B tile
   extern __shared__ uint8_t smem_raw[];
   const uint32_t raw = smem_u32(smem_raw);
   const uint32_t base = (raw + 1023u) & ~1023u;
   uint8_t *gbase = smem_raw + (base - raw);
-  constexpr int BAR_OFF = OW_NST * OW_STAGE + 8 * OW_TBUF;
-  const uint32_t full0 = base + BAR_OFF, empty0 = full0 + 8 * OW_NST, tfull0 = empty0 + 8 * OW_NST, tempty0 = tfull0 + 24;
-  volatile uint32_t *holder = reinterpret_cast<volatile uint32_t *>(gbase + BAR_OFF + 16 * OW_NST + 48);
-  volatile int *abort_flag = reinterpret_cast<volatile int *>(gbase + BAR_OFF + 16 * OW_NST + 56);
+  constexpr int BAR_OFF = NST * STAGE + 8 * Cfg::TBUF;
+  const uint32_t full0 = base + BAR_OFF, empty0 = full0 + 8 * NST, tfull0 = empty0 + 8 * NST, tempty0 = tfull0 + 24;
+  volatile uint32_t *holder = reinterpret_cast<volatile uint32_t *>(gbase + BAR_OFF + 16 * NST + 48);
+  volatile int *abort_flag = reinterpret_cast<volatile int *>(gbase + BAR_OFF + 16 * NST + 56);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int ntiles = 2 * nmt * nnt;
+  // column tiles with valid columns, by parity
+  const int nt0 = (ku + N - 1) / N, nt1 = ((inv ? ku : kv) + N - 1) / N;
+  const int ntiles = nmt * (nt0 + nt1);
 
   if (warp == 0) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32((const void *)holder)),
-                 "r"(OW_TMEM)
+                 "r"(Cfg::TMEM)
                  : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
   if (tid == 32) {
-    for (int s = 0; s < OW_NST; ++s) {
+    for (int s = 0; s < NST; ++s) {
       mbar_init(full0 + 8 * s, 1);
       mbar_init(empty0 + 8 * s, 1);
     }
@@ -337,13 +416,12 @@ __global__ void __launch_bounds__(320, 1) oz_wgemm_kernel(const uint8_t *__restr
   const uint32_t tmem = *holder;
 
   auto decode = [&](int t, int &par, int &mt, int &nt) {
-    nt = t % nnt;
-    mt = (t / nnt) % nmt;
-    par = t / (nnt * nmt);
+    par = t >= nmt * nt0;
+    const int u = par ? t - nmt * nt0 : t, ntp = par ? nt1 : nt0;
+    nt = u % ntp;
+    mt = u / ntp;
   };
-  auto wanted = [&](int par, int mt, int nt) -> bool {
-    if (nt * OW_N >= ((par && !inv) ? kv : ku)) return false;
-    if (mt * TM >= rows) return false;
+  auto wanted = [&](int mt) -> bool {  // some row of the tile belongs to a running right-hand side
     if (sc == nullptr) return true;
     const int m0 = mt * TM;
     const int r0 = m0 / rpr, r1 = (min(m0 + TM, rows) - 1) / rpr;
@@ -359,21 +437,27 @@ __global__ void __launch_bounds__(320, 1) oz_wgemm_kernel(const uint8_t *__restr
       for (int t = blockIdx.x; t < ntiles && !*abort_flag; t += gridDim.x) {
         int par, mt, nt;
         decode(t, par, mt, nt);
-        if (!wanted(par, mt, nt)) continue;
+        if (!wanted(mt)) continue;
         const uint8_t *at = apack + ((size_t)par * nmt + mt) * nk * OW_A;
-        const uint8_t *bt = bpack + ((size_t)par * nnt + nt) * nk * OW_B;
+        const uint8_t *bt = bpack + ((size_t)par * nnt + nt / SUB) * nk * OW_B + (nt % SUB) * Cfg::BSL;
         for (int k = 0; k < nk; ++k) {
-          if (it >= OW_NST && !mbar_wait(empty0 + 8 * s, ph ^ 1u)) {
+          if (it >= NST && !mbar_wait(empty0 + 8 * s, ph ^ 1u)) {
             atomicExch(err, 11);
             *abort_flag = 1;
             break;
           }
-          const uint32_t st = base + s * OW_STAGE, fb = full0 + 8 * s;
-          mbar_expect_tx(fb, (uint32_t)OW_STAGE);
+          const uint32_t st = base + s * STAGE, fb = full0 + 8 * s;
+          mbar_expect_tx(fb, (uint32_t)STAGE);
           bulk_g2s(st, at + (size_t)k * OW_A, OW_A, fb);
-          bulk_g2s(st + OW_A, bt + (size_t)k * OW_B, OW_B, fb);
+          if constexpr (SUB == 1) {
+            bulk_g2s(st + OW_A, bt + (size_t)k * OW_B, OW_B, fb);
+          } else {
+#pragma unroll
+            for (int i = 0; i < OW_NS; ++i)
+              bulk_g2s(st + OW_A + i * Cfg::BSL, bt + (size_t)k * OW_B + i * OW_BSL, Cfg::BSL, fb);
+          }
           ++it;
-          if (++s == OW_NST) {
+          if (++s == NST) {
             s = 0;
             ph ^= 1u;
           }
@@ -381,97 +465,90 @@ __global__ void __launch_bounds__(320, 1) oz_wgemm_kernel(const uint8_t *__restr
       }
       // after an abort nobody has waited for the last copies: no CTA leaves with copies in flight
       if (*abort_flag)
-        for (int i = max(0, it - OW_NST); i < it; ++i) mbar_wait(full0 + 8 * (i % OW_NST), (uint32_t)(i / OW_NST) & 1u);
+        for (int i = max(0, it - NST); i < it; ++i) mbar_wait(full0 + 8 * (i % NST), (uint32_t)(i / NST) & 1u);
     }
-  } else if (warp == 1) {
-    if (lane == 0) {  // MMA issuer
-      int s = 0;
-      uint32_t ph = 0, eph = 0;  // eph: next parity of each group's tempty barrier
-      uint32_t pend = 7u;        // groups handed to the epilogue and not seen back (at first: to be zeroed)
-      for (int t = blockIdx.x; t < ntiles && !*abort_flag; t += gridDim.x) {
-        int par, mt, nt;
-        decode(t, par, mt, nt);
-        if (!wanted(par, mt, nt)) continue;
-        for (int k = 0; k < nk; ++k) {
-          if (!mbar_wait(full0 + 8 * s, ph)) {
-            atomicExch(err, 12);
-            *abort_flag = 1;
-            break;
-          }
+  } else if (warp == 1) {  // MMA issuer: the loop is uniform over the warp, one lane issues
+    const bool lead = elect_one();
+    int s = 0;
+    uint32_t ph = 0, eph = 0;  // eph: next parity of each group's tempty barrier
+    uint32_t pend = 0;         // groups handed to the epilogue and not seen back
+    for (int t = blockIdx.x; t < ntiles && !*abort_flag; t += gridDim.x) {
+      int par, mt, nt;
+      decode(t, par, mt, nt);
+      if (!wanted(mt)) continue;
+      for (int k = 0; k < nk; ++k) {
+        bool ok = mbar_wait(full0 + 8 * s, ph);
+        if (!ok && lead) atomicExch(err, 12);
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        const uint32_t sa = (base + s * STAGE) >> 4, sb = sa + (OW_A >> 4);
+        auto wait = [&](int g) {
+          const bool got = mbar_wait(tempty0 + 8 * g, (eph >> g) & 1u);
+          if (!got && lead) atomicExch(err, 14);
+          ok = ok && got;
+          eph ^= 1u << g;
           asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-          const uint32_t sa = (base + s * OW_STAGE) >> 4, sb = sa + (OW_A >> 4);
-          const bool last = k + 1 == nk;
-          if (pend == 0 && !last) {
-            ow_issue_all(tmem, sa, sb);
-          } else {
-            // groups at rest first, then those the epilogue still drains; on a tile's last stage each
-            // group goes to the epilogue as soon as its products are issued
-            bool ok = true;
-            const uint32_t was = pend;
-            auto rest = [&](auto g) {
-              constexpr int G = decltype(g)::value;
-              if ((was >> G) & 1u) return;
-              ow_issue_group<G>(tmem, sa, sb);
-              if (last) ow_commit(tfull0 + 8 * G);
-            };
-            auto busy = [&](auto g) {
-              constexpr int G = decltype(g)::value;
-              if (!((was >> G) & 1u)) return;
-              ok = mbar_wait(tempty0 + 8 * G, (eph >> G) & 1u) && ok;
-              eph ^= 1u << G;
-              asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-              ow_issue_group<G>(tmem, sa, sb);
-              if (last) ow_commit(tfull0 + 8 * G);
-            };
-            rest(std::integral_constant<int, 0>());
-            rest(std::integral_constant<int, 1>());
-            rest(std::integral_constant<int, 2>());
-            busy(std::integral_constant<int, 0>());
-            busy(std::integral_constant<int, 1>());
-            busy(std::integral_constant<int, 2>());
-            if (!ok) {
-              atomicExch(err, 14);
-              *abort_flag = 1;
-              break;
+        };
+        if (k > 0) {
+          if (pend == 0) {
+            if (lead) ow_issue_all<N>(tmem, sa, sb);
+          } else if (pend == 2u) {  // the most frequent drain (weights 5, 6): the other groups meanwhile
+            if (lead) {
+              ow_issue_group<N, 0, false>(tmem, sa, sb);
+              ow_issue_group<N, 2, false>(tmem, sa, sb);
             }
+            wait(1);
+            if (lead) ow_issue_group<N, 1, false>(tmem, sa, sb);
+          } else {
+            if (pend & 1u) wait(0);
+            if (pend & 2u) wait(1);
+            if (pend & 4u) wait(2);
+            if (lead) ow_issue_all<N>(tmem, sa, sb);
           }
+        } else {  // a tile's first stage starts every sum afresh
+          if (pend & 1u) wait(0);
+          if (lead) ow_issue_group<N, 0, true>(tmem, sa, sb);
+          if (pend & 2u) wait(1);
+          if (lead) ow_issue_group<N, 1, true>(tmem, sa, sb);
+          if (pend & 4u) wait(2);
+          if (lead) ow_issue_group<N, 2, true>(tmem, sa, sb);
+        }
+        if (!ok) {
+          *abort_flag = 1;
+          break;
+        }
+        pend = k + 1 == nk ? 7u : (ow_bit(OW_E0, k + 1) | ow_bit(OW_E1, k + 1) << 1 | ow_bit(OW_E2, k + 1) << 2);
+        if (lead) {
           ow_commit(empty0 + 8 * s);
-          pend = last ? 7u : (ow_bit(OW_E0, k + 1) | ow_bit(OW_E1, k + 1) << 1 | ow_bit(OW_E2, k + 1) << 2);
-          if (pend != 0 && !last) {
-            if (pend & 1u) ow_commit(tfull0);
-            if (pend & 2u) ow_commit(tfull0 + 8);
-            if (pend & 4u) ow_commit(tfull0 + 16);
-          }
-          if (++s == OW_NST) {
-            s = 0;
-            ph ^= 1u;
-          }
+          if (pend & 1u) ow_commit(tfull0);
+          if (pend & 2u) ow_commit(tfull0 + 8);
+          if (pend & 4u) ow_commit(tfull0 + 16);
+        }
+        if (++s == NST) {
+          s = 0;
+          ph ^= 1u;
         }
       }
     }
   } else {  // epilogue warps 2..9
     const int lg = warp & 3, h = (warp - 2) >> 2;
-    const uint32_t tw = tmem + ((uint32_t)(lg * 32) << 16) + (uint32_t)(h * 32);  // + 64 (w - 2)
-    double *tbuf = reinterpret_cast<double *>(gbase + OW_NST * OW_STAGE + (warp - 2) * OW_TBUF);
+    const uint32_t tw = tmem + ((uint32_t)(lg * 32) << 16) + (uint32_t)(h * CW);  // + N (w - 2)
+    double *tbuf = reinterpret_cast<double *>(gbase + NST * STAGE + (warp - 2) * Cfg::TBUF);
     auto hand_back = [&](int g) {
       asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
       asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
       __syncwarp();
       if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(tempty0 + 8 * g) : "memory");
     };
-#pragma unroll
-    for (int w = 0; w < OW_NS; ++w) ow_tmem_zero32(tw + w * OW_N);
-    for (int g = 0; g < 3; ++g) hand_back(g);
     uint32_t fph = 0;  // next parity of each group's tfull barrier
     for (int t = blockIdx.x; t < ntiles; t += gridDim.x) {
       int par, mt, nt;
       decode(t, par, mt, nt);
-      if (!wanted(par, mt, nt)) continue;
+      if (!wanted(mt)) continue;
       const int row = mt * TM + lg * 32 + lane;
       const int e = row < rows ? erow[par * (nmt * TM) + row] : 0;
-      long long acc[32];
+      long long acc[CW];
 #pragma unroll
-      for (int q = 0; q < 32; ++q) acc[q] = 0;
+      for (int q = 0; q < CW; ++q) acc[q] = 0;
       bool stop = false;
       for (int c = 1; c <= nk; ++c) {
         const bool last = c == nk;
@@ -490,10 +567,10 @@ __global__ void __launch_bounds__(320, 1) oz_wgemm_kernel(const uint8_t *__restr
           asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
           return ok;
         };
-        float va[32], vb[32];
-        auto take = [&](int w, float (&v)[32]) {
-          tmem_ld32(tw + (w - 2) * OW_N, v);
-          ow_tmem_zero32(tw + (w - 2) * OW_N);
+        float va[CW], vb[CW];
+        auto take = [&](int w, float (&v)[CW]) {
+          ow_tmem_ld<CW>(tw + (w - 2) * N, v);
+          if (!last) ow_tmem_zero<CW>(tw + (w - 2) * N);
         };
         if ((last || ow_bit(OW_E0, c)) && !stop && wait_group(0)) {
           if (last) {
@@ -527,35 +604,41 @@ __global__ void __launch_bounds__(320, 1) oz_wgemm_kernel(const uint8_t *__restr
       // exponent field where every result of the row is a normal float64)
       const int kx = e + eB - 2 * 7 - OW_FIX;
       const bool fast = __all_sync(0xffffffffu, oz_fast_row(e, kx));  // a branch of the whole warp
-      const int c0 = nt * OW_N + h * 32;
-      const int ncols = min(32, ((par && !inv) ? kv : ku) - c0);
+      const int c0 = nt * N + h * CW;
+      const int ncols = min(CW, ((par && !inv) ? kv : ku) - c0);
       const int r0 = mt * TM + lg * 32;
       const int nr = min(32, rows - r0);
       const int ys = inv ? 1 : 2;
       double *yt = y + (inv ? ((size_t)par * rows + r0) * ku + c0 : (size_t)r0 * ld + par + 2 * (size_t)c0);
       const size_t ystep = inv ? (size_t)ku : (size_t)ld;
 #pragma unroll
-      for (int half = 0; half < 2; ++half) {
+      for (int part = 0; part < CW / CH; ++part) {
         if (fast) {
-          // half of the values on the FP64 pipe, half on the integer pipe (the same bits)
+          // a quarter of the values on the FP64 pipe, the rest on the integer pipe (the same bits)
 #pragma unroll
-          for (int q = 0; q < 16; q += 2) {
-            const long long db = __double_as_longlong(__ll2double_rn(acc[half * 16 + q]));
-            tbuf[lane * OW_TPITCH + q] = __longlong_as_double(db == 0 ? 0ll : db + ((long long)kx << 52));
-            tbuf[lane * OW_TPITCH + q + 1] = oz_to_f64(acc[half * 16 + q + 1], kx);
+          for (int q = 0; q < CH; ++q) {
+            const long long a = acc[part * CH + q];
+            double d;
+            if ((q & 3) == 0) {
+              const long long db = __double_as_longlong(__ll2double_rn(a));
+              d = __longlong_as_double(db == 0 ? 0ll : db + ((long long)kx << 52));
+            } else {
+              d = ow_to_f64(a, kx);
+            }
+            tbuf[lane * TPITCH + q] = d;
           }
         } else {
           const double scale = e == OZ_EXP_NAN ? __longlong_as_double(0x7ff8000000000000ll) : ldexp(1.0, e + eB - 2 * 7);
           const double unit = 1.0 / (double)(1LL << OW_FIX);
 #pragma unroll
-          for (int q = 0; q < 16; ++q) tbuf[lane * OW_TPITCH + q] = scale * (unit * __ll2double_rn(acc[half * 16 + q]));
+          for (int q = 0; q < CH; ++q) tbuf[lane * TPITCH + q] = scale * (unit * __ll2double_rn(acc[part * CH + q]));
         }
         __syncwarp();
-        const int cq = lane & 15, col = half * 16 + cq;
+        const int cq = lane % CH, col = part * CH + cq;
 #pragma unroll
-        for (int rr = 0; rr < 32; rr += 2) {
-          const int r = rr + (lane >> 4);
-          if (r < nr && col < ncols) yt[(size_t)r * ystep + (size_t)ys * col] = tbuf[r * OW_TPITCH + cq];
+        for (int rr = 0; rr < 32; rr += 32 / CH) {
+          const int r = rr + lane / CH;
+          if (r < nr && col < ncols) yt[(size_t)r * ystep + (size_t)ys * col] = tbuf[r * TPITCH + cq];
         }
         __syncwarp();
       }
@@ -564,5 +647,5 @@ __global__ void __launch_bounds__(320, 1) oz_wgemm_kernel(const uint8_t *__restr
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-  if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(OW_TMEM) : "memory");
+  if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(Cfg::TMEM) : "memory");
 }
