@@ -199,6 +199,8 @@ template <typename TI>
 __global__ void __launch_bounds__(256) pack_a_fwd_kernel(const TI *__restrict__ x, int rows, int n, int ku, int kv,
                                                          int nks, int nmt, uint8_t *__restrict__ out,
                                                          const KrylovScalars *__restrict__ sc, int rpr, int rscale) {
+  pdl_next();
+  pdl_wait();
   const int chunks = nks * (TK / 8);
   const unsigned t = blockIdx.x * blockDim.x + threadIdx.x;  // < nmt TM chunks, far below 2^32
   if (t >= (unsigned)(nmt * TM * chunks)) return;
@@ -239,6 +241,8 @@ __global__ void __launch_bounds__(256) pack_a_fwd_kernel(const TI *__restrict__ 
 __global__ void __launch_bounds__(256) pack_a_inv_kernel(const float *__restrict__ y, int rows, int n, int ku, int kv,
                                                          int nks, int nmt, uint8_t *__restrict__ out,
                                                          const KrylovScalars *__restrict__ sc, int rpr) {
+  pdl_next();
+  pdl_wait();
   const int chunks = nks * (TK / 8);
   const unsigned t = blockIdx.x * blockDim.x + threadIdx.x;  // < nmt TM chunks, far below 2^32
   if (t >= (unsigned)(nmt * TM * chunks)) return;
@@ -344,6 +348,7 @@ __global__ void __launch_bounds__(192, 1) dst_tc_gemm_kernel(const uint8_t *__re
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+  pdl_wait();
   const uint32_t tmem = *holder;
 
   // tile t -> (parity, m tile, n tile); tiles that only hold finished right-hand sides, or lie
@@ -393,6 +398,7 @@ __global__ void __launch_bounds__(192, 1) dst_tc_gemm_kernel(const uint8_t *__re
           }
         }
       }
+      pdl_next();  // late, as in oz_wgemm_kernel
     }
   } else if (warp == 1) {
     if (lane == 0) {  // MMA issuer
@@ -497,6 +503,8 @@ __global__ void __launch_bounds__(192, 1) dst_tc_gemm_kernel(const uint8_t *__re
 __global__ void __launch_bounds__(256) butterfly_kernel(const float *__restrict__ eo, double *__restrict__ z, int rows,
                                                         int n, int ku, int kv, const KrylovScalars *__restrict__ sc,
                                                         int rpr, int rscale) {
+  pdl_next();
+  pdl_wait();
   const int row = blockIdx.x;  // one block per row, its modes over the threads
   if (row >= rows || (sc != nullptr && sc[row / rpr].state != ST_RUN)) return;
   const float *er = eo + (size_t)row * 2 * ku;
@@ -520,6 +528,8 @@ __global__ void __launch_bounds__(256) butterfly_beta_kernel(const float *__rest
                                                              const double *__restrict__ r, const double *__restrict__ q,
                                                              int n, int ku, int kv, int rpr, int flexible,
                                                              KrylovScalars *sc, Reduce red) {
+  pdl_next();
+  pdl_wait();
   const int rhs = blockIdx.y;
   if (sc[rhs].state != ST_RUN) return;
   const size_t row0 = (size_t)rhs * rpr;
@@ -614,8 +624,8 @@ static void gemm_launch_nh(const DstPlan &dp, const uint8_t *apack, const uint8_
   const int nks = dp.kpad_u, nnt = dp.npad_u * (HALF ? 2 : 1), nmt = div_up(rows, TM);
   const int ntiles = 2 * nmt * nnt;
   const int grid = std::min(ntiles, 152);
-  dst_tc_gemm_kernel<NPROD, HALF><<<grid, 192, TcCfg<NPROD, HALF>::SMEM, s>>>(
-      apack, bpack, dp.tc_bmat_bytes, nks, nmt, nnt, rows, out, ld, dp.ku, nvalid0, nvalid1, sc, rpr, err);
+  launch_chain(HALF, dst_tc_gemm_kernel<NPROD, HALF>, grid, 192, TcCfg<NPROD, HALF>::SMEM, s, apack, bpack,
+               dp.tc_bmat_bytes, nks, nmt, nnt, rows, out, ld, dp.ku, nvalid0, nvalid1, sc, rpr, err);
 }
 static int device_sms();
 // 128 x 256 tiles unless they would leave more than half the SMs idle (then 128 x 128 tiles)
@@ -653,8 +663,8 @@ void dst_apply_tc_d2f(const DstPlan &dp, const double *x, float *y, int rows, in
   {
     ProfScope prof(KC_DSTTC_FWD, s);
     const long long threads = (long long)nmt * TM * nks * (TK / 8);
-    pack_a_fwd_kernel<double><<<(unsigned)((threads + 255) / 256), 256, 0, s>>>(x, rows, dp.n, dp.ku, dp.kv, nks, nmt,
-                                                                                apack, sc, rpr, rscale ? 1 : 0);
+    launch_pdl(pack_a_fwd_kernel<double>, (unsigned)((threads + 255) / 256), 256, 0, s, x, rows, dp.n, dp.ku, dp.kv,
+               nks, nmt, apack, sc, rpr, rscale ? 1 : 0);
     count_launch();
     LAG_LAUNCH_CHECK();
     gemm_launch(dp, apack, dp.tc_b, rows, y, dp.n, dp.ku, dp.kv, sc, rpr, dp.tc_err, s);
@@ -670,12 +680,12 @@ void dst_apply_tc_f2d(const DstPlan &dp, const float *y, double *z, int rows, in
   {
     ProfScope prof(KC_DSTTC_INV, s);
     const long long threads = (long long)nmt * TM * nks * (TK / 8);
-    pack_a_inv_kernel<<<(unsigned)((threads + 255) / 256), 256, 0, s>>>(y, rows, dp.n, dp.ku, dp.kv, nks, nmt, apack,
-                                                                         sc, rpr);
+    launch_pdl(pack_a_inv_kernel, (unsigned)((threads + 255) / 256), 256, 0, s, y, rows, dp.n, dp.ku, dp.kv, nks, nmt,
+               apack, sc, rpr);
     count_launch();
     LAG_LAUNCH_CHECK();
     gemm_launch(dp, apack, dp.tc_b + 2 * dp.tc_bmat_bytes, rows, eo, 2 * dp.ku, dp.ku, dp.ku, sc, rpr, dp.tc_err, s);
-    butterfly_kernel<<<rows, 256, 0, s>>>(eo, z, rows, dp.n, dp.ku, dp.kv, sc, rpr, rscale ? 1 : 0);
+    launch_pdl(butterfly_kernel, rows, 256, 0, s, eo, z, rows, dp.n, dp.ku, dp.kv, sc, rpr, rscale ? 1 : 0);
     count_launch();
     LAG_LAUNCH_CHECK();
   }
@@ -690,8 +700,8 @@ void dst_apply_tc_f2d_beta(const DstPlan &dp, const float *y, double *z, int nrh
   const int nks = dp.kpad_u, nmt = div_up(rows, TM);
   ProfScope prof(KC_DSTTC_INV, s);
   const long long threads = (long long)nmt * TM * nks * (TK / 8);
-  pack_a_inv_kernel<<<(unsigned)((threads + 255) / 256), 256, 0, s>>>(y, rows, dp.n, dp.ku, dp.kv, nks, nmt, apack, sc,
-                                                                       rpr);
+  launch_pdl(pack_a_inv_kernel, (unsigned)((threads + 255) / 256), 256, 0, s, y, rows, dp.n, dp.ku, dp.kv, nks, nmt,
+             apack, sc, rpr);
   count_launch();
   LAG_LAUNCH_CHECK();
   gemm_launch(dp, apack, dp.tc_b + 2 * dp.tc_bmat_bytes, rows, eo, 2 * dp.ku, dp.ku, dp.ku, sc, rpr, dp.tc_err, s);
@@ -699,7 +709,7 @@ void dst_apply_tc_f2d_beta(const DstPlan &dp, const float *y, double *z, int nrh
   int blocks = std::min(std::min(rpr, 1216), red.nblk);
   if (blocks < 1) blocks = 1;
   dim3 g(blocks, nrhs);
-  butterfly_beta_kernel<<<g, 256, 0, s>>>(eo, z, r, q, dp.n, dp.ku, dp.kv, rpr, flexible, sc, red);
+  launch_pdl(butterfly_beta_kernel, g, 256, 0, s, eo, z, r, q, dp.n, dp.ku, dp.kv, rpr, flexible, sc, red);
   count_launch();
   LAG_LAUNCH_CHECK();
 }
@@ -2629,6 +2639,8 @@ size_t dst_oz_scratch_bytes(const DstPlan &dp, int rows) {
 // finished right-hand sides are left as they are (their GEMM tiles were skipped).
 __global__ void oz_butterfly_kernel(const double *__restrict__ eo, double *__restrict__ x, int rows, int n, int ku,
                                     const KrylovScalars *__restrict__ sc, int rpr) {
+  pdl_next();
+  pdl_wait();
   const int row = blockIdx.x;  // one block per row
   if (row >= rows || (sc != nullptr && sc[row / rpr].state != ST_RUN)) return;
   const double *E = eo + (size_t)row * ku, *O = eo + ((size_t)rows + row) * ku;
@@ -2727,8 +2739,9 @@ static void ow_gemm_launch(const DstPlan &dp, const uint8_t *apack, const int *e
     LAG_CUDA_CHECK(cudaFuncSetAttribute(oz_wgemm_kernel<N>, cudaFuncAttributeMaxDynamicSharedMemorySize, OwCfg<N>::SMEM));
   });
   const int tiles = ow_tiles(dp, nmt, N, inv);
-  oz_wgemm_kernel<N><<<std::min(tiles, device_sms()), 320, OwCfg<N>::SMEM, s>>>(
-      apack, inv ? dp.ow_bi : dp.ow_b, erow, dp.oz_eB, nk, nmt, nnt, rows, y, dp.n, dp.ku, dp.kv, sc, rpr, dp.tc_err, inv);
+  launch_chain(N < 64, oz_wgemm_kernel<N>, std::min(tiles, device_sms()), 320, OwCfg<N>::SMEM, s, apack,
+                inv ? dp.ow_bi : dp.ow_b, erow, dp.oz_eB, nk, nmt, nnt, rows, y, dp.n, dp.ku, dp.kv, sc, rpr, dp.tc_err,
+               inv);
 }
 
 // the weight-stacked kernel (8-bit format, no opt-in variant)
@@ -2745,8 +2758,8 @@ static void ow_apply(const DstPlan &dp, const double *x, double *y, int rows, in
   // E / O sums of the inverse: after the digits and the row exponents, 256-byte aligned
   double *eo = reinterpret_cast<double *>(
       (reinterpret_cast<uintptr_t>(erow + 2 * (size_t)nmt * TM) + 255) & ~(uintptr_t)255);
-  ow_pack_a_kernel<<<nmt * TM, OZ_PACK_THREADS, oz_pack_smem(dp.kpad_u), s>>>(x, rows, dp.n, dp.ku, dp.kv, nk, nmt,
-                                                                              apack, erow, sc, rpr, inv);
+  launch_pdl(ow_pack_a_kernel, nmt * TM, OZ_PACK_THREADS, oz_pack_smem(dp.kpad_u), s, x, rows, dp.n, dp.ku, dp.kv, nk,
+             nmt, apack, erow, sc, rpr, inv);
   count_launch();
   LAG_LAUNCH_CHECK();
   // the narrowest tiles that still run in one wave (see OwCfg)
@@ -2758,7 +2771,7 @@ static void ow_apply(const DstPlan &dp, const double *x, double *y, int rows, in
   count_launch();
   LAG_LAUNCH_CHECK();
   if (inv) {
-    oz_butterfly_kernel<<<rows, 256, 0, s>>>(eo, y, rows, dp.n, dp.ku, sc, rpr);
+    launch_pdl(oz_butterfly_kernel, rows, 256, 0, s, eo, y, rows, dp.n, dp.ku, sc, rpr);
     count_launch();
     LAG_LAUNCH_CHECK();
   }
@@ -2827,7 +2840,7 @@ static void oz_apply_fmt(const DstPlan &dp, const double *x, double *y, int rows
   count_launch();
   LAG_LAUNCH_CHECK();
   if (inv) {
-    oz_butterfly_kernel<<<rows, 256, 0, s>>>(eo, y, rows, dp.n, dp.ku, sc, rpr);
+    launch_pdl(oz_butterfly_kernel, rows, 256, 0, s, eo, y, rows, dp.n, dp.ku, sc, rpr);
     count_launch();
     LAG_LAUNCH_CHECK();
   }

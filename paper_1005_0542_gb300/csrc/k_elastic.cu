@@ -140,6 +140,8 @@ __global__ void __launch_bounds__(256) elastic_apply_kernel(const double *__rest
                                                             int nx, int nz, ElasticCoef c,
                                                             const KrylovScalars *__restrict__ sc, int mode,
                                                             const double *__restrict__ sub) {
+  pdl_next();
+  pdl_wait();
   const int b = blockIdx.z;
   if (sc != nullptr) {
     const int st = sc[b].state;
@@ -194,7 +196,7 @@ void elastic_apply(const lag_medium &m, const double *p, double *q, int nrhs, co
   }
   dim3 g((m.grid.nx + 31) / 32, (m.grid.nz + 7) / 8, nrhs);
   ProfScope prof(KC_STENCIL_E, s);
-  elastic_apply_kernel<<<g, 256, 0, s>>>(p, q, m.grid.nx, m.grid.nz, elastic_coef(m), sc, mode, sub);
+  launch_pdl(elastic_apply_kernel, g, 256, 0, s, p, q, m.grid.nx, m.grid.nz, elastic_coef(m), sc, mode, sub);
   count_launch();
   LAG_LAUNCH_CHECK();
 }
@@ -204,6 +206,8 @@ void elastic_apply(const lag_medium &m, const double *p, double *q, int nrhs, co
 __global__ void __launch_bounds__(256) gm_start_kernel(const double *__restrict__ b, double *__restrict__ w,
                                                        size_t n, int first, double tol2, int max_iter,
                                                        KrylovScalars *sc, GmresDev g, Reduce red) {
+  pdl_next();
+  pdl_wait();
   const int rhs = blockIdx.y;
   KrylovScalars &S = sc[rhs];
   if (!first && !(S.state == ST_RUN || S.state == ST_MET)) return;
@@ -240,6 +244,8 @@ __global__ void __launch_bounds__(256) gm_start_kernel(const double *__restrict_
 // v = w / ||w|| for running systems (norm taken from g[0] at a cycle start or from H at a step)
 __global__ void gm_scale_kernel(const double *__restrict__ w, double *__restrict__ v, size_t n,
                                 const KrylovScalars *sc, const double *__restrict__ nrm, int nstride) {
+  pdl_next();
+  pdl_wait();
   const int rhs = blockIdx.y;
   if (sc[rhs].state != ST_RUN) return;
   const double s = nrm[(size_t)rhs * nstride];
@@ -254,10 +260,10 @@ void gm_start(const double *b, const double *cx, double *v0, size_t n, int nrhs,
               int max_iter, KrylovScalars *sc, GmresDev &g, const Reduce &red, cudaStream_t s) {
   ProfScope prof(KC_GMRES, s);
   dim3 grid(reduce_blocks(n), nrhs);
-  gm_start_kernel<<<grid, 256, 0, s>>>(b, const_cast<double *>(cx), n, first, tol * tol, max_iter, sc, g, red);
+  launch_pdl(gm_start_kernel, grid, 256, 0, s, b, const_cast<double *>(cx), n, first, tol * tol, max_iter, sc, g, red);
   count_launch();
   LAG_LAUNCH_CHECK();
-  gm_scale_kernel<<<grid, 256, 0, s>>>(cx, v0, n, sc, g.g, g.k + 1);
+  launch_pdl(gm_scale_kernel, grid, 256, 0, s, cx, v0, n, sc, g.g, g.k + 1);
   count_launch();
   LAG_LAUNCH_CHECK();
 }
@@ -312,6 +318,8 @@ static int dots_blocks(size_t n) { return std::min(reduce_blocks(n), 4 * 152); }
 __global__ void __launch_bounds__(256) gm_dots_kernel(const double *__restrict__ w, const double *__restrict__ V,
                                                       int j, size_t n, size_t vstride, KrylovScalars *sc,
                                                       GmresDev g, Reduce red, int pass, int shifted) {
+  pdl_next();
+  pdl_wait();
   const int rhs = blockIdx.y;
   if (sc[rhs].state != ST_RUN) return;
   if (pass == 1 && sc[rhs].reorth == 0) return;
@@ -401,6 +409,8 @@ __global__ void __launch_bounds__(256) gm_dots_kernel(const double *__restrict__
 __global__ void __launch_bounds__(256) gm_axpy_kernel(double *__restrict__ w, const double *__restrict__ V, int j,
                                                       size_t n, size_t vstride, const KrylovScalars *sc, GmresDev g,
                                                       int pass) {
+  pdl_next();
+  pdl_wait();
   const int rhs = blockIdx.y;
   if (sc[rhs].state != ST_RUN) return;
   if (pass == 1 && sc[rhs].reorth == 0) return;
@@ -418,10 +428,10 @@ void gm_orthogonalize(double *w, const double *V, int j, size_t n, int nrhs, siz
   ProfScope prof(KC_GMRES, s);
   if (j + 2 > 72) throw Error(LAG_EINVAL, "GMRES restart length above 70");
   dim3 gd(dots_blocks(n), nrhs), grid(reduce_blocks(n), nrhs);
-  gm_dots_kernel<<<gd, 256, 0, s>>>(w, V, j, n, vstride, sc, g, red, pass, shifted ? 1 : 0);
+  launch_pdl(gm_dots_kernel, gd, 256, 0, s, w, V, j, n, vstride, sc, g, red, pass, shifted ? 1 : 0);
   count_launch();
   LAG_LAUNCH_CHECK();
-  gm_axpy_kernel<<<grid, 256, 0, s>>>(w, V, j, n, vstride, sc, g, pass);
+  launch_pdl(gm_axpy_kernel, grid, 256, 0, s, w, V, j, n, vstride, sc, g, pass);
   count_launch();
   LAG_LAUNCH_CHECK();
 }
@@ -429,6 +439,8 @@ void gm_orthogonalize(double *w, const double *V, int j, size_t n, int nrhs, siz
 // h_{j+1,j} = ||w||; Givens rotations on column j; g update; residual estimate -> state
 __global__ void __launch_bounds__(256) gm_norm_kernel(const double *__restrict__ w, int j, size_t n,
                                                       KrylovScalars *sc, GmresDev g, Reduce red, int max_iter) {
+  pdl_next();
+  pdl_wait();
   const int rhs = blockIdx.y;
   if (sc[rhs].state != ST_RUN) return;
   const size_t off = (size_t)rhs * n;
@@ -470,6 +482,8 @@ __global__ void __launch_bounds__(256) gm_norm_kernel(const double *__restrict__
 // V_{j+1} = w / h_{j+1,j}  (only systems still expanding)
 __global__ void gm_next_kernel(const double *__restrict__ w, double *__restrict__ v, int j, size_t n,
                                const KrylovScalars *sc, GmresDev g) {
+  pdl_next();
+  pdl_wait();
   const int rhs = blockIdx.y;
   if (sc[rhs].state != ST_RUN) return;
   const int k = g.k;
@@ -484,16 +498,18 @@ void gm_normalize(double *w, double *vnext, int j, size_t n, int nrhs, KrylovSca
                   const Reduce &red, int max_iter, cudaStream_t s) {
   ProfScope prof(KC_GMRES, s);
   dim3 grid(reduce_blocks(n), nrhs);
-  gm_norm_kernel<<<grid, 256, 0, s>>>(w, j, n, sc, g, red, max_iter);
+  launch_pdl(gm_norm_kernel, grid, 256, 0, s, w, j, n, sc, g, red, max_iter);
   count_launch();
   LAG_LAUNCH_CHECK();
-  gm_next_kernel<<<grid, 256, 0, s>>>(w, vnext, j, n, sc, g);
+  launch_pdl(gm_next_kernel, grid, 256, 0, s, w, vnext, j, n, sc, g);
   count_launch();
   LAG_LAUNCH_CHECK();
 }
 
 // end of cycle: y = R^{-1} g (R = rotated H, upper triangular), x += sum_i y_i Z_i
 __global__ void gm_tri_kernel(KrylovScalars *sc, GmresDev g, int nrhs) {
+  pdl_next();
+  pdl_wait();
   const int rhs = blockIdx.x * blockDim.x + threadIdx.x;
   if (rhs >= nrhs) return;
   const KrylovScalars &S = sc[rhs];
@@ -515,6 +531,8 @@ __global__ void gm_tri_kernel(KrylovScalars *sc, GmresDev g, int nrhs) {
 
 __global__ void __launch_bounds__(256) gm_xupd_kernel(double *__restrict__ x, const double *__restrict__ Z, size_t n,
                                                       size_t zstride, const KrylovScalars *sc, GmresDev g) {
+  pdl_next();
+  pdl_wait();
   const int rhs = blockIdx.y;
   const int st = sc[rhs].state;
   if (!(st == ST_RUN || st == ST_MET)) return;
@@ -532,11 +550,11 @@ __global__ void __launch_bounds__(256) gm_xupd_kernel(double *__restrict__ x, co
 void gm_update_x(double *x, const double *Z, int, size_t n, int nrhs, size_t zstride, const KrylovScalars *sc,
                  GmresDev &g, cudaStream_t s) {
   ProfScope prof(KC_GMRES, s);
-  gm_tri_kernel<<<(nrhs + 63) / 64, 64, 0, s>>>(const_cast<KrylovScalars *>(sc), g, nrhs);
+  launch_pdl(gm_tri_kernel, (nrhs + 63) / 64, 64, 0, s, const_cast<KrylovScalars *>(sc), g, nrhs);
   count_launch();
   LAG_LAUNCH_CHECK();
   dim3 grid(reduce_blocks(n), nrhs);
-  gm_xupd_kernel<<<grid, 256, 0, s>>>(x, Z, n, zstride, sc, g);
+  launch_pdl(gm_xupd_kernel, grid, 256, 0, s, x, Z, n, zstride, sc, g);
   count_launch();
   LAG_LAUNCH_CHECK();
 }

@@ -131,6 +131,8 @@ __global__ void __launch_bounds__(256) cyl_elastic_apply_kernel(const double *__
                                                                 int nzc, int nr, const double *__restrict__ cf,
                                                                 const KrylovScalars *__restrict__ sc, int mode,
                                                                 const double *__restrict__ sub) {
+  pdl_next();
+  pdl_wait();
   const int b = blockIdx.z;
   if (sc != nullptr) {
     const int st = sc[b].state;
@@ -221,7 +223,7 @@ void elastic_cyl_apply(const lag_medium &m, const double *p, double *q, int nrhs
   const int nzc = m.grid.nx, nr = m.grid.nz;
   dim3 g((nzc + 31) / 32, (nr + 7) / 8, nrhs);
   ProfScope prof(KC_STENCIL_E, s);
-  cyl_elastic_apply_kernel<<<g, 256, 0, s>>>(p, q, nzc, nr, m.coef.as<double>(), sc, mode, sub);
+  launch_pdl(cyl_elastic_apply_kernel, g, 256, 0, s, p, q, nzc, nr, m.coef.as<double>(), sc, mode, sub);
   count_launch();
   LAG_LAUNCH_CHECK();
 }

@@ -194,6 +194,8 @@ __global__ void __launch_bounds__(256) acoustic_apply_kernel(const double *__res
                                                              const double *__restrict__ az,
                                                              const double *__restrict__ dg, KrylovScalars *sc,
                                                              Reduce red, int mode) {
+  pdl_next();
+  pdl_wait();
   const int b = blockIdx.y;
   if (sc != nullptr && sc[b].state != ST_RUN) return;
   const int tx = (nx + 31) / 32, tz = (nz + 7) / 8;
@@ -247,6 +249,8 @@ __global__ void __launch_bounds__(256) acoustic_apply_dir_kernel(const double *_
                                                                  const double *__restrict__ az,
                                                                  const double *__restrict__ dg, KrylovScalars *sc,
                                                                  Reduce red) {
+  pdl_next();
+  pdl_wait();
   const int b = blockIdx.y;
   if (sc[b].state != ST_RUN) return;
   const double beta = sc[b].beta;
@@ -310,7 +314,7 @@ void acoustic_apply(const lag_medium &m, const double *p, double *q, int nrhs, c
   dim3 g(stencil_blocks_per_rhs(nx, nz), nrhs);
   Reduce r = red ? *red : Reduce{nullptr, nullptr, 0, 0};
   ProfScope prof(KC_STENCIL_A, s);
-  acoustic_apply_kernel<<<g, 256, 0, s>>>(p, q, nx, nz, ax, az, dg, const_cast<KrylovScalars *>(sc), r, mode);
+  launch_pdl(acoustic_apply_kernel, g, 256, 0, s, p, q, nx, nz, ax, az, dg, const_cast<KrylovScalars *>(sc), r, mode);
   count_launch();
   LAG_LAUNCH_CHECK();
 }
@@ -322,8 +326,8 @@ void acoustic_apply_dir(const lag_medium &m, const double *z, const double *pold
   const double *ax = m.coef.as<double>(), *az = ax + nax, *dg = az + naz;
   dim3 g(stencil_blocks_per_rhs(nx, nz), nrhs);
   ProfScope prof(KC_STENCIL_A, s);
-  acoustic_apply_dir_kernel<<<g, 256, 0, s>>>(z, pold, pnew, q, nx, nz, ax, az, dg, const_cast<KrylovScalars *>(sc),
-                                              red);
+  launch_pdl(acoustic_apply_dir_kernel, g, 256, 0, s, z, pold, pnew, q, nx, nz, ax, az, dg,
+             const_cast<KrylovScalars *>(sc), red);
   count_launch();
   LAG_LAUNCH_CHECK();
 }
@@ -338,6 +342,8 @@ int reduce_blocks(size_t n) {
 __global__ void __launch_bounds__(256) pcg_start_kernel(const double *__restrict__ b, double *__restrict__ x,
                                                         double *__restrict__ r, double *__restrict__ p, size_t n,
                                                         double tol2, KrylovScalars *sc, Reduce red) {
+  pdl_next();
+  pdl_wait();
   const int rhs = blockIdx.y;
   const size_t off = (size_t)rhs * n;
   double acc = 0.0;
@@ -366,7 +372,7 @@ void pcg_start(const double *b, double *x, double *r, double *p, size_t n, int n
                const Reduce &red, cudaStream_t s) {
   dim3 g(reduce_blocks(n), nrhs);
   ProfScope prof(KC_VEC, s);
-  pcg_start_kernel<<<g, 256, 0, s>>>(b, x, r, p, n, tol * tol, sc, red);
+  launch_pdl(pcg_start_kernel, g, 256, 0, s, b, x, r, p, n, tol * tol, sc, red);
   count_launch();
   LAG_LAUNCH_CHECK();
 }
@@ -376,6 +382,8 @@ __global__ void __launch_bounds__(256) pcg_update_xr_kernel(double *__restrict__
                                                             const double *__restrict__ p,
                                                             const double *__restrict__ q, size_t n, int max_iter,
                                                             KrylovScalars *sc, Reduce red) {
+  pdl_next();
+  pdl_wait();
   const int rhs = blockIdx.y;
   if (sc[rhs].state != ST_RUN) return;
   const double a = sc[rhs].alpha;
@@ -404,7 +412,7 @@ void pcg_update_xr(double *x, double *r, const double *p, const double *q, size_
                    KrylovScalars *sc, const Reduce &red, cudaStream_t s) {
   dim3 g(reduce_blocks(n), nrhs);
   ProfScope prof(KC_VEC, s);
-  pcg_update_xr_kernel<<<g, 256, 0, s>>>(x, r, p, q, n, max_iter, sc, red);
+  launch_pdl(pcg_update_xr_kernel, g, 256, 0, s, x, r, p, q, n, max_iter, sc, red);
   count_launch();
   LAG_LAUNCH_CHECK();
 }
@@ -414,6 +422,8 @@ void pcg_update_xr(double *x, double *r, const double *p, const double *q, size_
 __global__ void __launch_bounds__(256) pcg_beta_kernel(const double *__restrict__ r, const double *__restrict__ z,
                                                        const double *__restrict__ q, size_t n, int flexible,
                                                        KrylovScalars *sc, Reduce red) {
+  pdl_next();
+  pdl_wait();
   const int rhs = blockIdx.y;
   if (sc[rhs].state != ST_RUN) return;
   const size_t off = (size_t)rhs * n;
@@ -442,6 +452,8 @@ __global__ void __launch_bounds__(256) pcg_beta_kernel(const double *__restrict_
 // that the whole grid is resident at once (the sweep is one round of loads, latency-bound)
 __global__ void __launch_bounds__(256, 8) pcg_rz_beta_kernel(const double *__restrict__ r, const double *__restrict__ z,
                                                              size_t n, KrylovScalars *sc, Reduce red) {
+  pdl_next();
+  pdl_wait();
   const int rhs = blockIdx.y;
   if (sc[rhs].state != ST_RUN) return;
   const double2 *r2 = reinterpret_cast<const double2 *>(r + (size_t)rhs * n);
@@ -478,8 +490,8 @@ void pcg_beta(const double *r, const double *z, const double *q, size_t n, int n
               KrylovScalars *sc, const Reduce &red, cudaStream_t s) {
   dim3 g(reduce_blocks(n), nrhs);
   ProfScope prof(KC_VEC, s);
-  if (!flexible && (n & 1) == 0) pcg_rz_beta_kernel<<<g, 256, 0, s>>>(r, z, n, sc, red);
-  else pcg_beta_kernel<<<g, 256, 0, s>>>(r, z, q, n, flexible, sc, red);
+  if (!flexible && (n & 1) == 0) launch_pdl(pcg_rz_beta_kernel, g, 256, 0, s, r, z, n, sc, red);
+  else launch_pdl(pcg_beta_kernel, g, 256, 0, s, r, z, q, n, flexible, sc, red);
   count_launch();
   LAG_LAUNCH_CHECK();
 }
@@ -494,6 +506,8 @@ __global__ void __launch_bounds__(256) laguerre_rhs_kernel(const double *__restr
                                                            double *__restrict__ r, double *__restrict__ x,
                                                            double *__restrict__ p, double tol2, KrylovScalars *sc,
                                                            Reduce red) {
+  pdl_next();
+  pdl_wait();
   const int rhs = blockIdx.y;
   const size_t n = nplane * ncomp;
   const size_t off = (size_t)rhs * n;
@@ -528,8 +542,8 @@ void laguerre_rhs(const double *rho_h2, const double *S, double cm, const double
                   double *p, double tol, KrylovScalars *sc, const Reduce &red, cudaStream_t s) {
   dim3 g(reduce_blocks(nplane * ncomp), nrhs);
   ProfScope prof(KC_LAGUERRE, s);
-  laguerre_rhs_kernel<<<g, 256, 0, s>>>(rho_h2, S, cm, fm, m, src_idx, src_comp, inv_cell, ncomp, nplane, r, x, p,
-                                        tol * tol, sc, red);
+  launch_pdl(laguerre_rhs_kernel, g, 256, 0, s, rho_h2, S, cm, fm, m, src_idx, src_comp, inv_cell, ncomp, nplane, r, x,
+             p, tol * tol, sc, red);
   count_launch();
   LAG_LAUNCH_CHECK();
 }
@@ -537,6 +551,8 @@ void laguerre_rhs(const double *rho_h2, const double *S, double cm, const double
 // T += c^_m R_m ; S += T   (S_{m+1} = sum_{k<=m} (m+1-k) c^_k R_k)
 __global__ void __launch_bounds__(256) laguerre_acc_kernel(const double *__restrict__ x, double *__restrict__ T,
                                                            double *__restrict__ S, double chat, size_t n) {
+  pdl_next();
+  pdl_wait();
   for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
     const double t = fma(chat, x[i], T[i]);
     T[i] = t;
@@ -547,13 +563,15 @@ __global__ void __launch_bounds__(256) laguerre_acc_kernel(const double *__restr
 void laguerre_accumulate(const double *x, double *T, double *S, double chat, size_t n, int nrhs, cudaStream_t s) {
   const size_t tot = n * (size_t)nrhs;
   ProfScope prof(KC_LAGUERRE, s);
-  laguerre_acc_kernel<<<reduce_blocks(tot), 256, 0, s>>>(x, T, S, chat, tot);
+  launch_pdl(laguerre_acc_kernel, reduce_blocks(tot), 256, 0, s, x, T, S, chat, tot);
   count_launch();
   LAG_LAUNCH_CHECK();
 }
 
 __global__ void gather_kernel(const double *__restrict__ x, const int *__restrict__ idx, int nrcv, int ncomp,
                               size_t nplane, int nrhs, double *__restrict__ out) {
+  pdl_next();
+  pdl_wait();
   const int t = blockIdx.x * blockDim.x + threadIdx.x;
   const int total = nrhs * ncomp * nrcv;
   if (t >= total) return;
@@ -566,7 +584,7 @@ void gather_receivers(const double *x, const int *rcv_idx, int nrcv, int ncomp, 
   const int total = nrhs * ncomp * nrcv;
   if (total <= 0) return;
   ProfScope prof(KC_LAGUERRE, s);
-  gather_kernel<<<(total + 255) / 256, 256, 0, s>>>(x, rcv_idx, nrcv, ncomp, nplane, nrhs, out);
+  launch_pdl(gather_kernel, (total + 255) / 256, 256, 0, s, x, rcv_idx, nrcv, ncomp, nplane, nrhs, out);
   count_launch();
   LAG_LAUNCH_CHECK();
 }

@@ -315,6 +315,8 @@ __global__ void __launch_bounds__(1024) tri_solve_kernel(const T *__restrict__ d
                                                          const T *__restrict__ sw, const T *__restrict__ red,
                                                          const KrylovScalars *__restrict__ sc, int pstride, int poff,
                                                          int ncomp, int mt, int gen) {
+  pdl_next();
+  pdl_wait();
   extern __shared__ __align__(16) unsigned char smem_raw[];
   T *tile = reinterpret_cast<T *>(smem_raw);
   const int nzp = P * L;
@@ -444,6 +446,7 @@ __global__ void __launch_bounds__(RegBounds<T, L, MT, GEN>::threads, RegBounds<T
                                                                int poff, int ncomp, int nplanes, int per_cta,
                                                                KrylovScalars *scw, Reduce rz) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
+  pdl_next();
   constexpr int NCR = GEN ? 0 : 3 * L;       // staged factor rows: 3 classes x L
   T *F = reinterpret_cast<T *>(smem_raw);    // [5][NCR][MT]: fm, fa, fc, sv, sw
   T *gF = F + 5 * NCR * MT;                  // [MT][32]
@@ -485,6 +488,7 @@ __global__ void __launch_bounds__(RegBounds<T, L, MT, GEN>::threads, RegBounds<T
   const T *Sw = (GEN ? sw : F + 4 * NCR * MT) + fo;
   const int warp = tid >> 5, lane = tid & 31, nwarp = nth >> 5;
   const int n = P - 1;
+  pdl_wait();  // the factors above are the plan's own; the data come from the kernels before
   __syncthreads();
   for (int k = 0; k < per_cta; ++k) {
     const int bi = blockIdx.y * per_cta + k;
@@ -595,7 +599,8 @@ static void tri_reg_launch_rz(const TriFactors &tf, const T *d, T *y, int nrhs, 
   int per_cta = 1;
   while (per_cta < 8 && (long long)ctas_x * ((nrhs + 2 * per_cta - 1) / (2 * per_cta)) >= 152 * 8) per_cta *= 2;
   dim3 grid(ctas_x, (nrhs + per_cta - 1) / per_cta);
-  tri_solve_reg_kernel<T, L, MT, GEN, RZ><<<grid, tf.threads, tf.smem, s>>>(
+  // early only below one block per SM: more would pile up on the SMs that finish first
+  launch_chain((long long)grid.x * grid.y <= 152, tri_solve_reg_kernel<T, L, MT, GEN, RZ>, grid, tf.threads, tf.smem, s,
       d, y, tf.nz, tf.nx, tf.P, tf.levels, tf.nf, (const T *)tf.fm, (const T *)tf.fc, (const T *)tf.fa,
       (const T *)tf.sv, (const T *)tf.sw, (const T *)tf.red, sc, pstride, poff, ncomp, nrhs, per_cta,
       rz != nullptr ? rz->sc : nullptr, rz != nullptr ? rz->red : Reduce{});
@@ -661,7 +666,7 @@ static void tri_launch(const TriFactors &tf, const T *d, T *y, int nrhs, const K
   }
   if (rz != nullptr) throw Error(LAG_EINVAL, "the (d, y) dot needs the register tridiagonal kernel");
   dim3 grid((tf.nx + tf.mt - 1) / tf.mt, nrhs);
-  tri_solve_kernel<T><<<grid, tf.threads, tf.smem, s>>>(
+  launch_pdl(tri_solve_kernel<T>, grid, tf.threads, tf.smem, s,
       d, y, tf.nz, tf.nx, tf.P, tf.L, tf.levels, tf.nf, (const T *)tf.fm, (const T *)tf.fc,
       (const T *)tf.fa, (const T *)tf.sv, (const T *)tf.sw, (const T *)tf.red, sc, pstride, poff, ncomp, tf.mt,
       tf.gen ? 1 : 0);

@@ -209,6 +209,8 @@ void KrylovWork::pcg_chunk(int iters) {
 // the loop ends, for the next launch.
 __global__ void pcg_loop_kernel(const KrylovScalars *sc, int nrhs, const int *err0, const int *err1,
                                 unsigned int *count, unsigned int cap, cudaGraphConditionalHandle handle) {
+  pdl_next();
+  pdl_wait();
   bool run = false;
   for (int b = threadIdx.x; b < nrhs; b += blockDim.x) run |= (sc[b].state == ST_RUN);
   run = __any_sync(0xffffffffu, run);
@@ -225,8 +227,8 @@ __global__ void pcg_loop_kernel(const KrylovScalars *sc, int nrhs, const int *er
 
 void KrylovWork::pcg_loop_condition(unsigned long long handle) {
   const int *e0 = (p1 != nullptr && (p1->use_tc || p1->dst.oz)) ? p1->dst.tc_err : nullptr;
-  pcg_loop_kernel<<<1, 32, 0, stream>>>(sc(), nrhs, e0, nullptr, wcount.as<unsigned int>(), 1024u,
-                                        (cudaGraphConditionalHandle)handle);
+  launch_pdl(pcg_loop_kernel, 1, 32, 0, stream, sc(), nrhs, e0, nullptr, wcount.as<unsigned int>(), 1024u,
+             (cudaGraphConditionalHandle)handle);
   count_launch();
   LAG_LAUNCH_CHECK();
 }

@@ -144,6 +144,8 @@ __global__ void __launch_bounds__(OZ_PACK_THREADS) ow_pack_a_kernel(const double
                                                                     uint8_t *__restrict__ out, int *__restrict__ erow,
                                                                     const KrylovScalars *__restrict__ sc, int rpr,
                                                                     int gather) {
+  pdl_next();
+  pdl_wait();
   extern __shared__ double xs[];  // the row's n inputs at OZ_PAD(j)
   const int row = blockIdx.x;
   // rows of finished right-hand sides keep whatever digits they had (bounded integers; nothing reads
@@ -413,6 +415,7 @@ __global__ void __launch_bounds__(320, 1) oz_wgemm_kernel(const uint8_t *__restr
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+  pdl_wait();
   const uint32_t tmem = *holder;
 
   auto decode = [&](int t, int &par, int &mt, int &nt) {
@@ -463,6 +466,8 @@ __global__ void __launch_bounds__(320, 1) oz_wgemm_kernel(const uint8_t *__restr
           }
         }
       }
+      // only now: blocks of the next kernel that fit beside this one would take issue slots from the MMAs
+      pdl_next();
       // after an abort nobody has waited for the last copies: no CTA leaves with copies in flight
       if (*abort_flag)
         for (int i = max(0, it - NST); i < it; ++i) mbar_wait(full0 + 8 * (i % NST), (uint32_t)(i / NST) & 1u);
