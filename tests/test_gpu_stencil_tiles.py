@@ -1,0 +1,49 @@
+"""The direction update + stencil kernel on its 64 x 16 tiles (ragged edges, one to four right-hand sides
+per block, systems that stop at different iterations): the recursive residual of the solve must be the
+true one, formed by the oracle's operator."""
+import ctypes as C
+
+import numpy as np
+import pytest
+
+from oracle import fd
+from paper_1005_0542_gb300 import lagwave as L
+
+from gpu_util import make_ctx, dev, empty, host, medium, plan, ptr
+
+pytestmark = pytest.mark.gpu
+RNG = np.random.default_rng(4021)
+
+
+@pytest.fixture(scope="module")
+def ctx():
+    c = make_ctx()
+    yield c
+    L.lag_destroy(c)
+
+
+# tiles x right-hand sides >= 912 in every case; 1, 2 and 4 right-hand sides per block, a remainder of
+# them (17 = 4 x 4 + 1), partial tiles in both directions, a width below one tile
+@pytest.mark.parametrize("nx,nz,nrhs", [(1021, 1013, 1), (130, 517, 10), (65, 1000, 8), (193, 353, 17), (40, 2600, 7)])
+def test_residual_is_true(ctx, nx, nz, nrhs):
+    h, d, tol = 200.0, 5.0, 1e-11
+    c = RNG.uniform(1800, 2600, (nz, nx))
+    rho = 310 * c ** 0.25
+    m = medium(ctx, nx, nz, d, d, c, rho, h)
+    mid = (C.c_double * 3)()
+    L.check(L.lag_medium_midranges(m, mid))
+    p = plan(ctx, nx, nz, d, d, mid[0], mid[0], mid[1] * h * h / 4)
+    b = RNG.standard_normal((nrhs, nz, nx)) * 10.0 ** RNG.uniform(-4, 4, (nrhs, 1, 1))
+    b[nrhs // 2, :, : nx // 2] = 0.0     # another right-hand side, another iteration count
+    bd, xd = dev(b), empty(b.shape)
+    its, res = (C.c_int * nrhs)(), (C.c_double * nrhs)()
+    s = L.solver(tol=tol)
+    L.check(L.lag_solve_system(m, p, None, ptr(bd), ptr(xd), nrhs, C.byref(s), its, res), ctx)
+    kap = fd.kappa_from_velocity(c, rho)
+    x = host(xd)
+    for i in range(nrhs):
+        r = b[i] - fd.apply_A(x[i], kap, rho, h, d, d)
+        # tol plus the rounding of ~50 float64 iterations
+        assert np.linalg.norm(r) / np.linalg.norm(b[i]) < 2 * tol
+    L.lag_precond_destroy(p)
+    L.lag_medium_destroy(m)
