@@ -108,7 +108,8 @@ struct KrylovScalars {
   double tol2;    // tol^2
   int state;      // ST_* below
   int iters;
-  int jdone;      // GMRES: steps taken in the open cycle
+  int jdone;      // GMRES: steps taken in the open cycle; PCG on tensor cores: the power of two that the
+                  // packed residual is scaled by (see residual_exponent)
   int reorth;     // GMRES: 1 if this step's second Gram-Schmidt pass runs (set by the first pass)
 };
 static_assert(sizeof(KrylovScalars) == 80, "layout");

@@ -197,6 +197,17 @@ bool dst_tc_supported(int n);
 void dst_apply_tc_f2d_beta(const DstPlan &dp, const float *y, double *z, int nrhs, int rpr, const double *r,
                            const double *q, int flexible, KrylovScalars *sc, const Reduce &red, cudaStream_t s);
 size_t dst_tc_scratch_bytes(const DstPlan &dp, int rows);
+// PCG on the tensor-core transforms: the forward transform in two steps, so that the residual update can
+// write its packed operand.  packs_residual: available for this plan (split-bf16, or exact slices on the
+// weight-stacked kernel); pack_residual: the operand from r (a solve's first iteration);
+// forward_packed: the GEMM alone; pcg_update_pack: pcg_update_xr and the operand in one pass.
+// The operand lives in the plan's scratch until the plan's next transform.
+bool dst_packs_residual(const DstPlan &dp, int rows, int rpr);
+void dst_pack_residual(const DstPlan &dp, const double *r, int rows, int rpr, const KrylovScalars *sc, cudaStream_t s);
+void dst_forward_packed_f64(const DstPlan &dp, double *y, int rows, int rpr, const KrylovScalars *sc, cudaStream_t s);
+void dst_forward_packed_f32(const DstPlan &dp, float *y, int rows, int rpr, const KrylovScalars *sc, cudaStream_t s);
+void pcg_update_pack(const DstPlan &dp, double *x, double *r, const double *p, const double *q, int nrhs, int rpr,
+                     int max_iter, KrylovScalars *sc, const Reduce &red, cudaStream_t s);
 // parity permutation of a float32 spectrum: natural mode order <-> [even modes | odd modes]
 void spectrum_permute(const float *in, float *out, int rows, int n, int ku, bool to_perm, cudaStream_t s);
 void spectrum_unpermute_widen(const float *in, double *out, int rows, int n, int ku, cudaStream_t s);

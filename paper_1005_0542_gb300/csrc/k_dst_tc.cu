@@ -533,7 +533,7 @@ __global__ void __launch_bounds__(256) butterfly_beta_kernel(const float *__rest
   const int rhs = blockIdx.y;
   if (sc[rhs].state != ST_RUN) return;
   const size_t row0 = (size_t)rhs * rpr;
-  const int es = residual_exponent(sc, rhs);  // the forward pack scaled r by 2^-e
+  const int es = sc[rhs].jdone;  // the packed residual was scaled by 2^-e
   double a0 = 0.0, a1 = 0.0;
   // rows round-robin over the blocks, a row's modes over the threads (no 64-bit index division);
   // E +- O in float32 (the spectrum's precision), widened with the residual's scale by integer
@@ -655,20 +655,27 @@ size_t dst_tc_scratch_bytes(const DstPlan &dp, int rows) {
   return 2 * nmt * dp.kpad_u * 2 * A_TILE + (size_t)rows * 2 * dp.ku * sizeof(float) + 256;
 }
 
+static void tc_pack_fwd(const DstPlan &dp, const double *x, int rows, int rpr, const KrylovScalars *sc, cudaStream_t s,
+                        bool rscale) {
+  const int nks = dp.kpad_u, nmt = div_up(rows, TM);
+  const long long threads = (long long)nmt * TM * nks * (TK / 8);
+  launch_pdl(pack_a_fwd_kernel<double>, (unsigned)((threads + 255) / 256), 256, 0, s, x, rows, dp.n, dp.ku, dp.kv, nks,
+             nmt, dp.tc_scratch, sc, rpr, rscale ? 1 : 0);
+  count_launch();
+  LAG_LAUNCH_CHECK();
+}
+
 void dst_apply_tc_d2f(const DstPlan &dp, const double *x, float *y, int rows, int rpr, const KrylovScalars *sc,
                       cudaStream_t s, bool rscale) {
   if (rows <= 0) return;
-  uint8_t *apack = dp.tc_scratch;
-  const int nks = dp.kpad_u, nmt = div_up(rows, TM);
-  {
-    ProfScope prof(KC_DSTTC_FWD, s);
-    const long long threads = (long long)nmt * TM * nks * (TK / 8);
-    launch_pdl(pack_a_fwd_kernel<double>, (unsigned)((threads + 255) / 256), 256, 0, s, x, rows, dp.n, dp.ku, dp.kv,
-               nks, nmt, apack, sc, rpr, rscale ? 1 : 0);
-    count_launch();
-    LAG_LAUNCH_CHECK();
-    gemm_launch(dp, apack, dp.tc_b, rows, y, dp.n, dp.ku, dp.kv, sc, rpr, dp.tc_err, s);
-  }
+  ProfScope prof(KC_DSTTC_FWD, s);
+  tc_pack_fwd(dp, x, rows, rpr, sc, s, rscale);
+  gemm_launch(dp, dp.tc_scratch, dp.tc_b, rows, y, dp.n, dp.ku, dp.kv, sc, rpr, dp.tc_err, s);
+}
+
+void dst_forward_packed_f32(const DstPlan &dp, float *y, int rows, int rpr, const KrylovScalars *sc, cudaStream_t s) {
+  ProfScope prof(KC_DSTTC_FWD, s);
+  gemm_launch(dp, dp.tc_scratch, dp.tc_b, rows, y, dp.n, dp.ku, dp.kv, sc, rpr, dp.tc_err, s);
 }
 
 void dst_apply_tc_f2d(const DstPlan &dp, const float *y, double *z, int rows, int rpr, const KrylovScalars *sc,
@@ -2744,37 +2751,97 @@ static void ow_gemm_launch(const DstPlan &dp, const uint8_t *apack, const int *e
                inv);
 }
 
-// the weight-stacked kernel (8-bit format, no opt-in variant)
-static void ow_apply(const DstPlan &dp, const double *x, double *y, int rows, int rpr, const KrylovScalars *sc,
-                     cudaStream_t s, int inv) {
+// the weight-stacked kernel's operand areas in the plan's scratch
+struct OwArea {
+  int nk, nnt, nmt;
+  uint8_t *apack;
+  int *erow;
+  double *eo;  // E / O sums of the inverse: after the digits and the row exponents, 256-byte aligned
+};
+static OwArea ow_area(const DstPlan &dp, int rows) {
+  OwArea a;
+  a.nk = div_up(dp.ku, OW_K);
+  a.nnt = div_up(dp.ku, OW_N);
+  a.nmt = div_up(rows, TM);
+  a.apack = dp.tc_scratch + oz_sk_bytes();
+  a.erow = reinterpret_cast<int *>(a.apack + 2 * (size_t)a.nmt * a.nk * OW_A);
+  a.eo = reinterpret_cast<double *>((reinterpret_cast<uintptr_t>(a.erow + 2 * (size_t)a.nmt * TM) + 255) &
+                                    ~(uintptr_t)255);
+  return a;
+}
+
+static void ow_pack(const DstPlan &dp, const double *x, int rows, int rpr, const KrylovScalars *sc, cudaStream_t s,
+                    int inv) {
   static PerDeviceOnce attr;
   attr.run([] {
     LAG_CUDA_CHECK(cudaFuncSetAttribute(ow_pack_a_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                         (int)oz_pack_smem(OZ_PACK_MAXK / TK + 1)));
   });
-  const int nk = div_up(dp.ku, OW_K), nnt = div_up(dp.ku, OW_N), nmt = div_up(rows, TM);
-  uint8_t *apack = dp.tc_scratch + oz_sk_bytes();
-  int *erow = reinterpret_cast<int *>(apack + 2 * (size_t)nmt * nk * OW_A);
-  // E / O sums of the inverse: after the digits and the row exponents, 256-byte aligned
-  double *eo = reinterpret_cast<double *>(
-      (reinterpret_cast<uintptr_t>(erow + 2 * (size_t)nmt * TM) + 255) & ~(uintptr_t)255);
-  launch_pdl(ow_pack_a_kernel, nmt * TM, OZ_PACK_THREADS, oz_pack_smem(dp.kpad_u), s, x, rows, dp.n, dp.ku, dp.kv, nk,
-             nmt, apack, erow, sc, rpr, inv);
+  const OwArea a = ow_area(dp, rows);
+  launch_pdl(ow_pack_a_kernel, a.nmt * TM, OZ_PACK_THREADS, oz_pack_smem(dp.kpad_u), s, x, rows, dp.n, dp.ku, dp.kv,
+             a.nk, a.nmt, a.apack, a.erow, sc, rpr, inv);
   count_launch();
   LAG_LAUNCH_CHECK();
+}
+
+static void ow_gemm(const DstPlan &dp, double *y, int rows, int rpr, const KrylovScalars *sc, cudaStream_t s, int inv) {
+  const OwArea a = ow_area(dp, rows);
   // the narrowest tiles that still run in one wave (see OwCfg)
-  double *yo = inv ? eo : y;
+  double *yo = inv ? a.eo : y;
   const int sms = device_sms();
-  if (ow_tiles(dp, nmt, 16, inv) <= sms) ow_gemm_launch<16>(dp, apack, erow, nk, nmt, nnt, rows, yo, sc, rpr, inv, s);
-  else if (ow_tiles(dp, nmt, 32, inv) <= sms) ow_gemm_launch<32>(dp, apack, erow, nk, nmt, nnt, rows, yo, sc, rpr, inv, s);
-  else ow_gemm_launch<64>(dp, apack, erow, nk, nmt, nnt, rows, yo, sc, rpr, inv, s);
+  if (ow_tiles(dp, a.nmt, 16, inv) <= sms) ow_gemm_launch<16>(dp, a.apack, a.erow, a.nk, a.nmt, a.nnt, rows, yo, sc, rpr, inv, s);
+  else if (ow_tiles(dp, a.nmt, 32, inv) <= sms) ow_gemm_launch<32>(dp, a.apack, a.erow, a.nk, a.nmt, a.nnt, rows, yo, sc, rpr, inv, s);
+  else ow_gemm_launch<64>(dp, a.apack, a.erow, a.nk, a.nmt, a.nnt, rows, yo, sc, rpr, inv, s);
   count_launch();
   LAG_LAUNCH_CHECK();
   if (inv) {
-    launch_pdl(oz_butterfly_kernel, rows, 256, 0, s, eo, y, rows, dp.n, dp.ku, sc, rpr);
+    launch_pdl(oz_butterfly_kernel, rows, 256, 0, s, a.eo, y, rows, dp.n, dp.ku, sc, rpr);
     count_launch();
     LAG_LAUNCH_CHECK();
   }
+}
+
+bool dst_packs_residual(const DstPlan &dp, int rows, int rpr) {
+  if (dp.tc_b != nullptr) return oz_pack_smem(dp.kpad_u) / 2 <= 200 * 1024;  // a row as float on chip: n <= 45 k
+  return dp.ow_b != nullptr && dst_oz_gemm_variant(dp, rows, rpr, 0) == OZ_GEMM_TILES;
+}
+
+void dst_pack_residual(const DstPlan &dp, const double *r, int rows, int rpr, const KrylovScalars *sc, cudaStream_t s) {
+  if (dp.tc_b != nullptr) {
+    ProfScope prof(KC_DSTTC_FWD, s);
+    tc_pack_fwd(dp, r, rows, rpr, sc, s, true);
+  } else {
+    ProfScope prof(KC_DST64, s);
+    ow_pack(dp, r, rows, rpr, sc, s, 0);
+  }
+}
+
+void dst_forward_packed_f64(const DstPlan &dp, double *y, int rows, int rpr, const KrylovScalars *sc, cudaStream_t s) {
+  ProfScope prof(KC_DST64, s);
+  ow_gemm(dp, y, rows, rpr, sc, s, 0);
+}
+
+void pcg_update_pack(const DstPlan &dp, double *x, double *r, const double *p, const double *q, int nrhs, int rpr,
+                     int max_iter, KrylovScalars *sc, const Reduce &red, cudaStream_t s) {
+  static PerDeviceOnce attr;
+  attr.run([] {
+    LAG_CUDA_CHECK(cudaFuncSetAttribute(pcg_update_pack_kernel<0>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                        (int)oz_pack_smem(OZ_PACK_MAXK / TK + 1)));
+    LAG_CUDA_CHECK(cudaFuncSetAttribute(pcg_update_pack_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024));
+  });
+  ProfScope prof(KC_VEC, s);
+  const int rows = nrhs * rpr;
+  dim3 g(std::max(1, std::min(rpr, red.nblk)), nrhs);
+  if (dp.tc_b != nullptr) {
+    launch_pdl(pcg_update_pack_kernel<1>, g, OZ_PACK_THREADS, oz_pack_smem(dp.kpad_u) / 2, s, x, r, p, q, dp.n, rpr,
+               dp.ku, dp.kv, dp.kpad_u, div_up(rows, TM), dp.tc_scratch, (int *)nullptr, max_iter, sc, red);
+  } else {
+    const OwArea a = ow_area(dp, rows);
+    launch_pdl(pcg_update_pack_kernel<0>, g, OZ_PACK_THREADS, oz_pack_smem(dp.kpad_u), s, x, r, p, q, dp.n, rpr, dp.ku,
+               dp.kv, a.nk, a.nmt, a.apack, a.erow, max_iter, sc, red);
+  }
+  count_launch();
+  LAG_LAUNCH_CHECK();
 }
 
 template <int NB, int NS>
@@ -2852,7 +2919,8 @@ void dst_apply_oz(const DstPlan &dp, const double *x, double *y, int rows, int r
   ProfScope prof(KC_DST64, s);
   const int inv = (inverse && dp.kind == 1) ? 1 : 0;
   if (dp.ow_b != nullptr && dst_oz_gemm_variant(dp, rows, rpr, inv) == OZ_GEMM_TILES) {
-    ow_apply(dp, x, y, rows, rpr, sc, s, inv);
+    ow_pack(dp, x, rows, rpr, sc, s, inv);
+    ow_gemm(dp, y, rows, rpr, sc, s, inv);
     return;
   }
   if (dp.oz_b == nullptr) throw Error(LAG_EINVAL, "exact-slice DST: the slice tiles of this variant are not built");

@@ -513,6 +513,7 @@ __global__ void __launch_bounds__(256) pcg_start_kernel(const double *__restrict
     S.tol2 = tol2;
     S.iters = 0;
     S.rr = tot[0];
+    S.jdone = residual_exponent(sc, rhs);
     S.alpha = S.beta = S.rz = S.pq = S.zq = 0.0;
     S.state = (tot[0] == 0.0) ? ST_CONV : (isfinite(tot[0]) ? ST_RUN : ST_NAN);
   }
@@ -551,6 +552,7 @@ __global__ void __launch_bounds__(256) pcg_update_xr_kernel(double *__restrict__
   if (publish_partials<1>(red, rhs, blockIdx.x, gridDim.x, v1, tot)) {
     KrylovScalars &S = sc[rhs];
     S.rr = tot[0];
+    S.jdone = residual_exponent(sc, rhs);
     S.iters += 1;
     if (!isfinite(tot[0])) S.state = ST_NAN;
     else if (tot[0] <= S.tol2 * S.bb) S.state = ST_CONV;
@@ -680,6 +682,7 @@ __global__ void __launch_bounds__(256) laguerre_rhs_kernel(const double *__restr
     KrylovScalars &K = sc[rhs];
     K.bb = tot[0];
     K.rr = tot[0];
+    K.jdone = residual_exponent(sc, rhs);
     K.tol2 = tol2;
     K.iters = 0;
     K.alpha = K.beta = K.rz = K.pq = K.zq = 0.0;

@@ -81,6 +81,7 @@ void KrylovWork::setup(lag_ctx *c, lag_medium *med, lag_precond *q1, lag_precond
   }
   eager_done = false;
   pcur = 0;
+  r_packed = false;
   ctx = c;
   m = med;
   p1 = q1;
@@ -96,10 +97,10 @@ void KrylovWork::setup(lag_ctx *c, lag_medium *med, lag_precond *q1, lag_precond
   const int nvec = elastic ? (3 + (s.restart_k + 1) + s.restart_k) : 7;
   vecs.alloc(ctx, (size_t)nvec * n * nrhs * sizeof(double));
   scal.alloc(ctx, (size_t)nrhs * sizeof(KrylovScalars), true);
-  // blocks per right-hand side of the reductions: the vector kernels, the stencil, and the float64
-  // tridiagonal solve that also forms (r, z) (one CTA per 4 modes at most)
+  // blocks per right-hand side of the reductions: the vector kernels, the stencil, the update that packs
+  // (a block per row) and the float64 tridiagonal solve that also forms (r, z) (one CTA per 4 modes at most)
   const int cap = std::max(std::max(std::max(reduce_blocks(n), stencil_blocks(med->grid)), 1),
-                           elastic ? 1 : (med->grid.nx + 3) / 4);
+                           elastic ? 1 : std::max((med->grid.nx + 3) / 4, std::min(med->grid.nz, 1216)));
   red.ensure(ctx, nrhs, cap, elastic ? s.restart_k + 1 : 2);
   if (elastic) {
     gk = s.restart_k;
@@ -156,6 +157,7 @@ void KrylovWork::start_from_r() {
   // PCG: x = 0, r = b and p = 0 were set by the right-hand side kernel; the first iteration takes
   // beta = 0, so its direction is z = B^{-1} r
   pcur = 0;
+  r_packed = false;
 }
 
 // One PCG iteration (Sec. 2.3), in the order z = B^{-1} r, beta, p = z + beta p with q = A p and
@@ -167,30 +169,43 @@ void KrylovWork::pcg_iteration() {
   Reduce rd = red.get();
   const int flexible = s.prec == LAG_MIXED ? 1 : 0;
   const int rpr = p1->grid.nz;
+  const int rows = nrhs * rpr;
+  p1->ensure_scratch(nrhs);
+  // on the tensor-core transforms the previous iteration's update has packed r already
+  const bool packs = dst_packs_residual(p1->dst, rows, rpr);
+  if (packs && !r_packed) dst_pack_residual(p1->dst, r(), rows, rpr, sc(), stream);
   if (p1->use_tc) {
     // mixed path: forward DST, tridiagonal solve, then the inverse DST whose butterfly also forms
     // (r, z), (z, q) and beta
-    const int rows = nrhs * rpr;
-    p1->ensure_scratch(nrhs);
     float *w = p1->scratch.as<float>();
-    dst_apply_tc_d2f(p1->dst, r(), w, rows, rpr, sc(), stream, true);
+    if (packs) dst_forward_packed_f32(p1->dst, w, rows, rpr, sc(), stream);
+    else dst_apply_tc_d2f(p1->dst, r(), w, rows, rpr, sc(), stream, true);
     tri_solve_f32(p1->tri32, w, w, nrhs, sc(), stream);
     dst_apply_tc_f2d_beta(p1->dst, w, z, nrhs, rpr, r(), q, flexible, sc(), rd, stream);
-  } else if (p1->prec == LAG_FP64 && p1->dst.kind == 0 && tri_rz_fusable(p1->tri64, rd)) {
-    // float64 path: one symmetric DST-I S serves both transforms, so (r, z) = (S r, T^{-1} S r) and
-    // the tridiagonal solve forms it from its input and output, with beta.  Its output goes to q,
-    // whose previous content only the flexible beta reads; the direction update rewrites it.
-    p1->ensure_scratch(nrhs);
+  } else if (packs || (p1->prec == LAG_FP64 && p1->dst.kind == 0 && tri_rz_fusable(p1->tri64, rd))) {
     double *w = p1->scratch.as<double>();
-    dst_apply_f64(p1->dst, r(), w, nrhs * rpr, rpr, sc(), stream);
-    tri_solve_f64_rz(p1->tri64, w, q, nrhs, sc(), rd, stream);
-    dst_inverse_f64(p1->dst, q, z, nrhs * rpr, rpr, sc(), stream);
+    if (packs) dst_forward_packed_f64(p1->dst, w, rows, rpr, sc(), stream);
+    else dst_apply_f64(p1->dst, r(), w, rows, rpr, sc(), stream);
+    if (p1->dst.kind == 0 && tri_rz_fusable(p1->tri64, rd)) {
+      // one symmetric DST-I S serves both transforms, so (r, z) = (S r, T^{-1} S r) and the tridiagonal
+      // solve forms it from its input and output, with beta.  Its output goes to q, whose previous
+      // content only the flexible beta reads; the direction update rewrites it.
+      tri_solve_f64_rz(p1->tri64, w, q, nrhs, sc(), rd, stream);
+      dst_inverse_f64(p1->dst, q, z, rows, rpr, sc(), stream);
+    } else {
+      tri_solve_f64(p1->tri64, w, w, nrhs, sc(), stream);
+      dst_inverse_f64(p1->dst, w, z, rows, rpr, sc(), stream);
+      pcg_beta(r(), z, q, n, nrhs, flexible, sc(), rd, stream);
+    }
   } else {
     precond(r(), z);                                                 // z = B^{-1} r
     pcg_beta(r(), z, q, n, nrhs, flexible, sc(), rd, stream);
   }
   acoustic_apply_dir(*m, z, pold, pnew, q, nrhs, sc(), rd, stream);   // p = z + beta p, q = A p, alpha
-  pcg_update_xr(x(), r(), pnew, q, n, nrhs, s.max_iter, sc(), rd, stream);  // x, r, ||r||, state
+  // x, r, ||r||, state (and the next iteration's packed r)
+  if (packs) pcg_update_pack(p1->dst, x(), r(), pnew, q, nrhs, rpr, s.max_iter, sc(), rd, stream);
+  else pcg_update_xr(x(), r(), pnew, q, n, nrhs, s.max_iter, sc(), rd, stream);
+  r_packed = packs;
   pcur ^= 1;
 }
 
@@ -236,7 +251,11 @@ void KrylovWork::pcg_loop_condition(unsigned long long handle) {
 void KrylovWork::pcg_while() {
   p1->ensure_scratch(nrhs);
   const void *key[4] = {p1->scratch.ptr, p1->tc_scratch.ptr, vecs.ptr, red.part.ptr};
-  const int prod = p1->dst.tc_products;
+  const int rpr = p1->grid.nz;
+  const bool packs = dst_packs_residual(p1->dst, nrhs * rpr, rpr);
+  if (packs && !r_packed) dst_pack_residual(p1->dst, r(), nrhs * rpr, rpr, sc(), stream);
+  r_packed = packs;  // as the body finds and leaves it
+  const int prod = p1->dst.tc_products | (packs ? 16 : 0);
   if (wexec != nullptr && (std::memcmp(key, wkey, sizeof(key)) != 0 || prod != wprod)) {
     cudaGraphExecDestroy(wexec);
     wexec = nullptr;

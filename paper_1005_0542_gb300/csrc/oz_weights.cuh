@@ -136,43 +136,14 @@ __global__ void ow_pack_b_kernel(const double *m0, int k0n, int n0n, int ld0, co
   ow_store_digits<OW_BSL>(T, base + ow_swz(n % OW_N, ch & 1));
 }
 
-// A digits per apply: one CTA per row, both parities, as oz_pack_a_kernel (row staged in shared memory,
-// row exponent from the largest |input|, fold as exact integer sums).
-// Layout [parity][m tile][K stage][digit][128 x 16]; erow[parity][row].
-__global__ void __launch_bounds__(OZ_PACK_THREADS) ow_pack_a_kernel(const double *__restrict__ x, int rows, int n,
-                                                                    int ku, int kv, int nk, int nmt,
-                                                                    uint8_t *__restrict__ out, int *__restrict__ erow,
-                                                                    const KrylovScalars *__restrict__ sc, int rpr,
-                                                                    int gather) {
-  pdl_next();
-  pdl_wait();
-  extern __shared__ double xs[];  // the row's n inputs at OZ_PAD(j)
-  const int row = blockIdx.x;
-  // rows of finished right-hand sides keep whatever digits they had (bounded integers; nothing reads
-  // those rows' outputs any more)
-  if (row < rows && sc != nullptr && sc[row / rpr].state != ST_RUN) return;
-  const bool live = row < rows;  // the padding rows of the last tile pack as zeros
-  const double *xr = x + (size_t)(live ? row : 0) * n;
-  unsigned long long b0 = 0, b1 = 0;
-  constexpr int PB = 16;  // a batch of loads all issue before any is used
-  for (int jb = 0; jb < n; jb += PB * OZ_PACK_THREADS) {
-    double vb[PB];
-#pragma unroll
-    for (int u = 0; u < PB; ++u) {
-      const int j = jb + u * OZ_PACK_THREADS + threadIdx.x;
-      vb[u] = (live && j < n) ? __ldg(xr + j) : 0.0;
-    }
-#pragma unroll
-    for (int u = 0; u < PB; ++u) {
-      const int j = jb + u * OZ_PACK_THREADS + threadIdx.x;
-      if (j < n) {
-        xs[OZ_PAD(j)] = vb[u];
-        const unsigned long long m = (unsigned long long)__double_as_longlong(vb[u]) & 0x7fffffffffffffffull;
-        if (gather && (j & 1)) b1 = max(b1, m);
-        else b0 = max(b0, m);
-      }
-    }
-  }
+// The digits of one row staged in shared memory (its n inputs at OZ_PAD(j)), both parities: the row
+// exponent from the largest |input| (b0, b1: this thread's largest bit patterns with the sign cleared, b1
+// the odd entries' when gathered), the fold u_j = x_j + x_{n-1-j}, v_j = x_j - x_{n-1-j} as exact integer sums,
+// or (gather, the DCT-II inverse) u = the even entries and v = the odd ones.  By all OZ_PACK_THREADS
+// threads of a CTA; layout [parity][m tile][K stage][digit][128 x 16], erow[parity][row].
+__device__ __forceinline__ void ow_pack_row(const double *xs, unsigned long long b0, unsigned long long b1, int row,
+                                            bool live, int n, int ku, int kv, int nk, int nmt, uint8_t *out, int *erow,
+                                            bool gather) {
   __shared__ unsigned long long red[2][OZ_PACK_THREADS / 32];
   for (int o = 16; o > 0; o >>= 1) {
     b0 = max(b0, __shfl_xor_sync(0xffffffffu, b0, o));
@@ -224,6 +195,142 @@ __global__ void __launch_bounds__(OZ_PACK_THREADS) ow_pack_a_kernel(const double
     uint8_t *t0 = out + ((size_t)mt * nk + (ch >> 1)) * OW_A + ow_swz(r, ch & 1);
     ow_store_digits<OW_ASL>(U, t0);
     ow_store_digits<OW_ASL>(W, t0 + (size_t)nmt * nk * OW_A);
+  }
+}
+
+// A digits per apply: one CTA per row, both parities
+__global__ void __launch_bounds__(OZ_PACK_THREADS) ow_pack_a_kernel(const double *__restrict__ x, int rows, int n,
+                                                                    int ku, int kv, int nk, int nmt,
+                                                                    uint8_t *__restrict__ out, int *__restrict__ erow,
+                                                                    const KrylovScalars *__restrict__ sc, int rpr,
+                                                                    int gather) {
+  pdl_next();
+  pdl_wait();
+  extern __shared__ double xs[];  // the row's n inputs at OZ_PAD(j)
+  const int row = blockIdx.x;
+  // rows of finished right-hand sides keep whatever digits they had (bounded integers; nothing reads
+  // those rows' outputs any more)
+  if (row < rows && sc != nullptr && sc[row / rpr].state != ST_RUN) return;
+  const bool live = row < rows;  // the padding rows of the last tile pack as zeros
+  const double *xr = x + (size_t)(live ? row : 0) * n;
+  unsigned long long b0 = 0, b1 = 0;
+  constexpr int PB = 16;  // a batch of loads all issue before any is used
+  for (int jb = 0; jb < n; jb += PB * OZ_PACK_THREADS) {
+    double vb[PB];
+#pragma unroll
+    for (int u = 0; u < PB; ++u) {
+      const int j = jb + u * OZ_PACK_THREADS + threadIdx.x;
+      vb[u] = (live && j < n) ? __ldg(xr + j) : 0.0;
+    }
+#pragma unroll
+    for (int u = 0; u < PB; ++u) {
+      const int j = jb + u * OZ_PACK_THREADS + threadIdx.x;
+      if (j < n) {
+        xs[OZ_PAD(j)] = vb[u];
+        const unsigned long long m = (unsigned long long)__double_as_longlong(vb[u]) & 0x7fffffffffffffffull;
+        if (gather && (j & 1)) b1 = max(b1, m);
+        else b0 = max(b0, m);
+      }
+    }
+  }
+  ow_pack_row(xs, b0, b1, row, live, n, ku, kv, nk, nmt, out, erow, gather != 0);
+}
+
+// PCG's x += alpha p, r -= alpha q and (r, r) -> convergence state, and the operand of the next
+// iteration's forward transform packed from the new r while its row is on chip: MODE 0 the exact-slice
+// digits (one launch and one pass over r less per iteration), MODE 1 the split-bf16 tiles of the mixed
+// path (scaled by the power of two of the OLD (r, r), the one known here; recorded in jdone for
+// the inverse transform).  A CTA takes whole rows of its right-hand side, grid-stride.  Bound by HBM
+// / L2: 48 B a point plus the operand (14 or 4 B).  2048 x 1024: update and pack 22 + 16 us as two
+// kernels, 33 us as one (mixed 22 + 9, 24 us; 32 right-hand sides 560 + 170, 510 us).
+template <int MODE>
+__global__ void __launch_bounds__(OZ_PACK_THREADS) pcg_update_pack_kernel(
+    double *__restrict__ x, double *__restrict__ r, const double *__restrict__ p, const double *__restrict__ q, int n,
+    int rpr, int ku, int kv, int nk, int nmt, uint8_t *__restrict__ out, int *__restrict__ erow, int max_iter,
+    KrylovScalars *sc, Reduce red) {
+  pdl_next();
+  pdl_wait();
+  extern __shared__ double xs[];  // MODE 0: the row at OZ_PAD(j); MODE 1: as float, scaled
+  float *xf = reinterpret_cast<float *>(xs);
+  const int rhs = blockIdx.y;
+  if (sc[rhs].state != ST_RUN) return;
+  const double a = sc[rhs].alpha;
+  const int es = residual_exponent(sc, rhs);
+  double acc = 0.0;
+  constexpr int PB = 4;
+  for (int row = blockIdx.x; row < rpr; row += gridDim.x) {
+    const int g = rhs * rpr + row;
+    const size_t o = (size_t)g * n;
+    unsigned long long b0 = 0;
+    for (int jb = 0; jb < n; jb += PB * OZ_PACK_THREADS) {
+      double xv[PB], rv[PB], pv[PB], qv[PB];
+#pragma unroll
+      for (int u = 0; u < PB; ++u) {
+        const int j = jb + u * OZ_PACK_THREADS + threadIdx.x;
+        const bool in = j < n;
+        xv[u] = in ? x[o + j] : 0.0;
+        rv[u] = in ? r[o + j] : 0.0;
+        pv[u] = in ? p[o + j] : 0.0;
+        qv[u] = in ? q[o + j] : 0.0;
+      }
+#pragma unroll
+      for (int u = 0; u < PB; ++u) {
+        const int j = jb + u * OZ_PACK_THREADS + threadIdx.x;
+        if (j >= n) continue;
+        x[o + j] = fma(a, pv[u], xv[u]);
+        const double v = fma(-a, qv[u], rv[u]);
+        r[o + j] = v;
+        acc = fma(v, v, acc);
+        if (MODE == 0) {
+          xs[OZ_PAD(j)] = v;
+          b0 = max(b0, (unsigned long long)__double_as_longlong(v) & 0x7fffffffffffffffull);
+        } else {
+          xf[OZ_PAD(j)] = narrow_pow2(v, -es);
+        }
+      }
+    }
+    if (MODE == 0) {
+      ow_pack_row(xs, b0, 0, g, true, n, ku, kv, nk, nmt, out, erow, false);
+    } else {
+      __syncthreads();
+      const int mt = g / TM, rr = g % TM;
+      for (int ch = threadIdx.x; ch < nk * (TK / 8); ch += OZ_PACK_THREADS) {
+        alignas(16) uint16_t uh[8], ul[8], vh[8], vl[8];
+#pragma unroll
+        for (int e = 0; e < 8; ++e) {
+          const int j = ch * 8 + e;
+          float u = 0.f, w = 0.f;
+          if (j < kv) {
+            const float f1 = xf[OZ_PAD(j)], f2 = xf[OZ_PAD(n - 1 - j)];
+            u = f1 + f2;
+            w = f1 - f2;
+          } else if (j < ku) {
+            u = xf[OZ_PAD(j)];  // middle element of an odd-length row
+          }
+          split2f(u, uh[e], ul[e]);
+          split2f(w, vh[e], vl[e]);
+        }
+        const uint32_t off = swz(rr, (ch * 8) % TK);
+        for (int par = 0; par < 2; ++par) {
+          uint8_t *tile = out + (((size_t)par * nmt + mt) * nk + (ch * 8) / TK) * 2 * A_TILE;
+          *reinterpret_cast<uint4 *>(tile + off) = *reinterpret_cast<const uint4 *>(par ? vh : uh);
+          *reinterpret_cast<uint4 *>(tile + A_TILE + off) = *reinterpret_cast<const uint4 *>(par ? vl : ul);
+        }
+      }
+    }
+    __syncthreads();  // the row's stage is reused
+  }
+  double v1[1] = {acc}, tot[1];
+  __shared__ double sh[32];
+  block_sum<1>(v1, sh);
+  if (publish_partials<1>(red, rhs, blockIdx.x, gridDim.x, v1, tot)) {
+    KrylovScalars &S = sc[rhs];
+    S.rr = tot[0];
+    S.jdone = es;
+    S.iters += 1;
+    if (!isfinite(tot[0])) S.state = ST_NAN;
+    else if (tot[0] <= S.tol2 * S.bb) S.state = ST_CONV;
+    else if (S.iters >= max_iter) S.state = ST_STOP;
   }
 }
 

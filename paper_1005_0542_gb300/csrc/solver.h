@@ -59,6 +59,7 @@ struct KrylovWork {
   DevBuf wcount;             // the loop's repeat counter (a bound on one launch) and its body total
   unsigned long long wbodies_seen = 0;
   bool eager_done = false;
+  bool r_packed = false;     // PCG: the plan's scratch holds the packed operand of the current r
   int pcur = 0;              // which of the two direction buffers holds the current p
 
   ~KrylovWork();
