@@ -93,8 +93,9 @@ void lag_precond::apply(const double *r, double *z, int nrhs, const KrylovScalar
     float *w = scratch.as<float>();
     if (use_tc) dst_apply_tc_d2f(dst, r, w, rows, grid.nz, sc, s, rscale);
     else dst_apply_f32_d2f(dst, r, w, rows, grid.nz, sc, s, rscale);
-    tri_solve_f32(tri32, w, w, nrhs, sc, s);
-    if (use_tc) dst_apply_tc_f2d(dst, w, z, rows, grid.nz, sc, s, rscale);
+    const bool packed = use_tc && tri_solve_f32_packed(tri32, w, dst_tc_operand(dst, rows), nrhs, sc, s);
+    if (!packed) tri_solve_f32(tri32, w, w, nrhs, sc, s);
+    if (use_tc) dst_apply_tc_f2d(dst, packed ? nullptr : w, z, rows, grid.nz, sc, s, rscale);
     else dst_inverse_f32_f2d(dst, w, z, rows, grid.nz, sc, s, rscale);
   }
 }

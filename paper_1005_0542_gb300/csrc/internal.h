@@ -12,6 +12,7 @@
 
 #include "../../include/lagwave.h"
 #include "common.cuh"
+#include "tc_layout.cuh"
 
 // ----------------------------------------------------------------------------- context
 struct lag_ctx {
@@ -107,6 +108,12 @@ void tri_solve_f64(const TriFactors &tf, const double *d, double *y, int nplanes
 void tri_solve_f32(const TriFactors &tf, const float *d, float *y, int nplanes,
                    const KrylovScalars *sc, cudaStream_t s, int pstride = 1, int poff = 0,
                    int ncomp = 1);
+// the same on a parity-permuted spectrum (mixed tensor-core plans), the result written as the inverse
+// transform's split-bf16 operand instead of a spectrum; d is left as it is.  False where !tri_packs (constant
+// coefficients on the register kernel only): nothing is launched then.
+bool tri_packs(const TriFactors &tf);
+bool tri_solve_f32_packed(const TriFactors &tf, const float *d, const TcOperand &out, int nplanes,
+                          const KrylovScalars *sc, cudaStream_t s, int pstride = 1, int poff = 0, int ncomp = 1);
 // y = T^{-1} d for nrhs one-component planes (d != y) and, per plane b, (d, y) summed in a fixed
 // order into rz_new, then PCG's Fletcher-Reeves beta = rz_new / sc[b].rz (0 on a solve's first
 // iteration) and sc[b].rz = rz_new.  Between z = S T^{-1} S r and d = S r with one symmetric S
@@ -193,6 +200,8 @@ void dst_apply_tc_d2f(const DstPlan &dp, const double *x, float *y, int rows, in
 void dst_apply_tc_f2d(const DstPlan &dp, const float *x, double *y, int rows, int rows_per_rhs,
                       const KrylovScalars *sc, cudaStream_t s, bool rscale = false);
 bool dst_tc_supported(int n);
+// dst_apply_tc_f2d[_beta] take y = null where the tridiagonal solve has packed its result (tri_solve_f32_packed)
+TcOperand dst_tc_operand(const DstPlan &dp, int rows);
 // inverse tensor-core DST fused with the CG beta of the next step (per rhs: rpr rows)
 void dst_apply_tc_f2d_beta(const DstPlan &dp, const float *y, double *z, int nrhs, int rpr, const double *r,
                            const double *q, int flexible, KrylovScalars *sc, const Reduce &red, cudaStream_t s);

@@ -32,6 +32,7 @@
 #include <cstdint>
 
 #include "internal.h"
+#include "tc_layout.cuh"
 
 #include <utility>
 #include <vector>
@@ -40,23 +41,10 @@ namespace lag {
 
 namespace {
 
-constexpr int TM = 128;          // rows per tile (MMA M)
 constexpr int TN = 256;          // output columns per tile (MMA N)
-constexpr int TK = 64;           // K per stage (one 128-byte swizzle atom of bf16)
-constexpr int A_TILE = TM * TK * 2;   // 16 KB
 constexpr int B_TILE = TN * TK * 2;   // 32 KB
 constexpr uint32_t TMEM_COLS = 256;
 constexpr long long WAIT_LIMIT = 1LL << 26;
-
-// element (r, k) of a rows x 64 tile in the K-major SWIZZLE_128B layout (byte offset)
-__host__ __device__ __forceinline__ uint32_t swz(int r, int k) {
-  return (uint32_t)r * 128u + ((uint32_t)((k >> 3) ^ (r & 7)) << 4) + (uint32_t)(k & 7) * 2u;
-}
-
-__device__ __forceinline__ uint16_t bf16_bits(float f) {
-  __nv_bfloat16 b = __float2bfloat16_rn(f);
-  return *reinterpret_cast<uint16_t *>(&b);
-}
 
 // split v into bf16 hi + bf16 lo (float64 arithmetic: used once per plan for S)
 __device__ __forceinline__ void split2(double v, uint16_t &hi, uint16_t &lo) {
@@ -65,14 +53,6 @@ __device__ __forceinline__ void split2(double v, uint16_t &hi, uint16_t &lo) {
   const float r = (float)(v - (double)__bfloat162float(h));
   hi = *reinterpret_cast<uint16_t *>(&h);
   lo = bf16_bits(r);
-}
-
-// the same split in float32 arithmetic (per apply: FP64 throughput is 1/61 of FP32 on this part;
-// hi + lo keeps 16 significant bits, far inside float32 rounding)
-__device__ __forceinline__ void split2f(float f, uint16_t &hi, uint16_t &lo) {
-  __nv_bfloat16 h = __float2bfloat16_rn(f);
-  hi = *reinterpret_cast<uint16_t *>(&h);
-  lo = bf16_bits(f - __bfloat162float(h));
 }
 
 __device__ __forceinline__ uint32_t smem_u32(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
@@ -592,7 +572,6 @@ __global__ void unpermute_widen_kernel(const float *in, double *out, int rows, i
 
 // ------------------------------------------------------------------------------ host side
 static int div_up(int a, int b) { return (a + b - 1) / b; }
-
 bool dst_tc_supported(int n) { return n >= 16; }
 
 size_t dst_tc_bytes(int n) {
@@ -678,45 +657,58 @@ void dst_forward_packed_f32(const DstPlan &dp, float *y, int rows, int rpr, cons
   gemm_launch(dp, dp.tc_scratch, dp.tc_b, rows, y, dp.n, dp.ku, dp.kv, sc, rpr, dp.tc_err, s);
 }
 
-void dst_apply_tc_f2d(const DstPlan &dp, const float *y, double *z, int rows, int rpr, const KrylovScalars *sc,
-                      cudaStream_t s, bool rscale) {
-  if (rows <= 0) return;
-  uint8_t *apack = dp.tc_scratch;
-  float *eo = reinterpret_cast<float *>(apack + 2 * (size_t)div_up(rows, TM) * dp.kpad_u * 2 * A_TILE);
+TcOperand dst_tc_operand(const DstPlan &dp, int rows) {
+  TcOperand t;
+  t.a = dp.tc_scratch;
+  t.ku = dp.ku;
+  t.nks = dp.kpad_u;
+  t.nmt = div_up(rows, TM);
+  return t;
+}
+
+// the inverse's sums E [ku] | O [ku] per row: z[k] = E[k] + O[k], z[n-1-k] = E[k] - O[k]
+static float *dst_tc_eo(const DstPlan &dp, int rows) {
+  return reinterpret_cast<float *>(dp.tc_scratch + 2 * (size_t)div_up(rows, TM) * dp.kpad_u * 2 * A_TILE);
+}
+
+// the inverse's E / O sums, from the spectrum y (null: its operand has been packed by the tridiagonal solve)
+static void tc_inverse_eo(const DstPlan &dp, const float *y, int rows, int rpr, const KrylovScalars *sc,
+                          cudaStream_t s) {
   const int nks = dp.kpad_u, nmt = div_up(rows, TM);
-  {
-    ProfScope prof(KC_DSTTC_INV, s);
+  if (y != nullptr) {
     const long long threads = (long long)nmt * TM * nks * (TK / 8);
     launch_pdl(pack_a_inv_kernel, (unsigned)((threads + 255) / 256), 256, 0, s, y, rows, dp.n, dp.ku, dp.kv, nks, nmt,
-               apack, sc, rpr);
-    count_launch();
-    LAG_LAUNCH_CHECK();
-    gemm_launch(dp, apack, dp.tc_b + 2 * dp.tc_bmat_bytes, rows, eo, 2 * dp.ku, dp.ku, dp.ku, sc, rpr, dp.tc_err, s);
-    launch_pdl(butterfly_kernel, rows, 256, 0, s, eo, z, rows, dp.n, dp.ku, dp.kv, sc, rpr, rscale ? 1 : 0);
+               dp.tc_scratch, sc, rpr);
     count_launch();
     LAG_LAUNCH_CHECK();
   }
+  gemm_launch(dp, dp.tc_scratch, dp.tc_b + 2 * dp.tc_bmat_bytes, rows, dst_tc_eo(dp, rows), 2 * dp.ku, dp.ku, dp.ku, sc,
+              rpr, dp.tc_err, s);
+}
+
+void dst_apply_tc_f2d(const DstPlan &dp, const float *y, double *z, int rows, int rpr, const KrylovScalars *sc,
+                      cudaStream_t s, bool rscale) {
+  if (rows <= 0) return;
+  ProfScope prof(KC_DSTTC_INV, s);
+  tc_inverse_eo(dp, y, rows, rpr, sc, s);
+  launch_pdl(butterfly_kernel, rows, 256, 0, s, dst_tc_eo(dp, rows), z, rows, dp.n, dp.ku, dp.kv, sc, rpr,
+             rscale ? 1 : 0);
+  count_launch();
+  LAG_LAUNCH_CHECK();
 }
 
 void dst_apply_tc_f2d_beta(const DstPlan &dp, const float *y, double *z, int nrhs, int rpr, const double *r,
                            const double *q, int flexible, KrylovScalars *sc, const Reduce &red, cudaStream_t s) {
   const int rows = nrhs * rpr;
   if (rows <= 0) return;
-  uint8_t *apack = dp.tc_scratch;
-  float *eo = reinterpret_cast<float *>(apack + 2 * (size_t)div_up(rows, TM) * dp.kpad_u * 2 * A_TILE);
-  const int nks = dp.kpad_u, nmt = div_up(rows, TM);
   ProfScope prof(KC_DSTTC_INV, s);
-  const long long threads = (long long)nmt * TM * nks * (TK / 8);
-  launch_pdl(pack_a_inv_kernel, (unsigned)((threads + 255) / 256), 256, 0, s, y, rows, dp.n, dp.ku, dp.kv, nks, nmt,
-             apack, sc, rpr);
-  count_launch();
-  LAG_LAUNCH_CHECK();
-  gemm_launch(dp, apack, dp.tc_b + 2 * dp.tc_bmat_bytes, rows, eo, 2 * dp.ku, dp.ku, dp.ku, sc, rpr, dp.tc_err, s);
+  tc_inverse_eo(dp, y, rows, rpr, sc, s);
   // rows per right-hand side over at most min(1216, the reduction's block capacity) blocks
   int blocks = std::min(std::min(rpr, 1216), red.nblk);
   if (blocks < 1) blocks = 1;
   dim3 g(blocks, nrhs);
-  launch_pdl(butterfly_beta_kernel, g, 256, 0, s, eo, z, r, q, dp.n, dp.ku, dp.kv, rpr, flexible, sc, red);
+  launch_pdl(butterfly_beta_kernel, g, 256, 0, s, dst_tc_eo(dp, rows), z, r, q, dp.n, dp.ku, dp.kv, rpr, flexible, sc,
+             red);
   count_launch();
   LAG_LAUNCH_CHECK();
 }

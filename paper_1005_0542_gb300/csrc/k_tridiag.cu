@@ -433,10 +433,12 @@ struct RegBounds {
   static constexpr int blocks = per_sm / threads > 0 ? per_sm / threads : 1;
 };
 
+// PK (float32): the result goes out as the inverse transform's split-bf16 operand (see tc_layout.cuh) instead
+// of a spectrum: one pass over it and one launch less.
 // RZ (float64, one component, din != yout): also the dot (d, y) of each plane, summed over the CTAs
 // of its modes (block sums published into rz, the last CTA combining them in CTA order), and PCG's
 // beta from it into scw (see tri_solve_f64_rz)
-template <typename T, int L, int MT, bool GEN, bool RZ>
+template <typename T, int L, int MT, bool GEN, bool RZ, bool PK>
 __global__ void __launch_bounds__(RegBounds<T, L, MT, GEN>::threads, RegBounds<T, L, MT, GEN>::blocks) tri_solve_reg_kernel(const T *__restrict__ din, T *__restrict__ yout, int nz,
                                                                int nx, int P, int levels, int nf,
                                                                const T *__restrict__ fm, const T *__restrict__ fc,
@@ -444,7 +446,7 @@ __global__ void __launch_bounds__(RegBounds<T, L, MT, GEN>::threads, RegBounds<T
                                                                const T *__restrict__ sw, const T *__restrict__ red,
                                                                const KrylovScalars *__restrict__ sc, int pstride,
                                                                int poff, int ncomp, int nplanes, int per_cta,
-                                                               KrylovScalars *scw, Reduce rz) {
+                                                               KrylovScalars *scw, Reduce rz, TcOperand pk) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   pdl_next();
   constexpr int NCR = GEN ? 0 : 3 * L;       // staged factor rows: 3 classes x L
@@ -497,7 +499,7 @@ __global__ void __launch_bounds__(RegBounds<T, L, MT, GEN>::threads, RegBounds<T
     if (sc != nullptr && sc[b / ncomp].state != ST_RUN) continue;  // uniform over the CTA
     const bool live = col_ok;
     const T *src = din + (size_t)b * nz * nx + j;
-    T *dst = yout + (size_t)b * nz * nx + j;
+    T *dst = PK ? nullptr : yout + (size_t)b * nz * nx + j;
     T v[L];
 #pragma unroll
     for (int i = 0; i < L; ++i) {
@@ -554,11 +556,24 @@ __global__ void __launch_bounds__(RegBounds<T, L, MT, GEN>::threads, RegBounds<T
       // correction with the spike vectors, store
       const T xa = xi[c * 33 + p];
       const T xb = (p + 1 <= P - 1) ? xi[c * 33 + p + 1] : T(0);
+      // PK: this thread's operand column, the row parts added below
+      const int par = (PK && j >= pk.ku) ? 1 : 0, kc = j - par * pk.ku, mstep = pk.nks * 2 * A_TILE;
+      uint8_t *pc = PK ? pk.a + ((size_t)par * pk.nmt * pk.nks + kc / TK) * 2 * A_TILE + (kc & 7) * 2 : nullptr;
+      const int kx = (kc >> 3) & 7, g0 = b * nz + p * L;
 #pragma unroll
       for (int i = 0; i < L; ++i) {
         const int r = p * L + i;
         const T y = (i < i0) ? xa : v[i] - xa * Sv[i * FS] - xb * Sw[i * FS];
-        if (r < nz) {
+        if (PK) {
+          if (r < nz) {
+            const int g = g0 + i;  // swz(g % TM, kc % TK) of m tile g / TM
+            uint8_t *t = pc + (size_t)(g / TM) * mstep + (g % TM) * 128 + ((kx ^ (g & 7)) << 4);
+            uint16_t hi, lo;
+            split2f((float)y, hi, lo);
+            *reinterpret_cast<uint16_t *>(t) = hi;
+            *reinterpret_cast<uint16_t *>(t + A_TILE) = lo;
+          }
+        } else if (r < nz) {
           dst[(size_t)r * nx] = y;
           if constexpr (RZ) dot = fma(src[(size_t)r * nx], y, dot);  // d is still intact (din != yout)
         }
@@ -586,12 +601,12 @@ struct TriRz {
   Reduce red;
 };
 
-template <typename T, int L, int MT, bool GEN, bool RZ>
+template <typename T, int L, int MT, bool GEN, bool RZ, bool PK>
 static void tri_reg_launch_rz(const TriFactors &tf, const T *d, T *y, int nrhs, const KrylovScalars *sc,
-                              cudaStream_t s, int pstride, int poff, int ncomp, const TriRz *rz) {
+                              cudaStream_t s, int pstride, int poff, int ncomp, const TriRz *rz, const TcOperand *pk) {
   static PerDeviceOnce attr_done;
   attr_done.run([] {
-    LAG_CUDA_CHECK(cudaFuncSetAttribute(tri_solve_reg_kernel<T, L, MT, GEN, RZ>,
+    LAG_CUDA_CHECK(cudaFuncSetAttribute(tri_solve_reg_kernel<T, L, MT, GEN, RZ, PK>,
                                         cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024));
   });
   // several right-hand sides per CTA when there are plenty of CTAs anyway (factor reuse)
@@ -600,51 +615,57 @@ static void tri_reg_launch_rz(const TriFactors &tf, const T *d, T *y, int nrhs, 
   while (per_cta < 8 && (long long)ctas_x * ((nrhs + 2 * per_cta - 1) / (2 * per_cta)) >= 152 * 8) per_cta *= 2;
   dim3 grid(ctas_x, (nrhs + per_cta - 1) / per_cta);
   // early only below one block per SM: more would pile up on the SMs that finish first
-  launch_chain((long long)grid.x * grid.y <= 152, tri_solve_reg_kernel<T, L, MT, GEN, RZ>, grid, tf.threads, tf.smem, s,
+  launch_chain((long long)grid.x * grid.y <= 152, tri_solve_reg_kernel<T, L, MT, GEN, RZ, PK>, grid, tf.threads, tf.smem, s,
       d, y, tf.nz, tf.nx, tf.P, tf.levels, tf.nf, (const T *)tf.fm, (const T *)tf.fc, (const T *)tf.fa,
       (const T *)tf.sv, (const T *)tf.sw, (const T *)tf.red, sc, pstride, poff, ncomp, nrhs, per_cta,
-      rz != nullptr ? rz->sc : nullptr, rz != nullptr ? rz->red : Reduce{});
+      rz != nullptr ? rz->sc : nullptr, rz != nullptr ? rz->red : Reduce{}, pk != nullptr ? *pk : TcOperand{});
 }
 
 template <typename T, int L, int MT, bool GEN>
 static void tri_reg_launch_mt(const TriFactors &tf, const T *d, T *y, int nrhs, const KrylovScalars *sc,
-                              cudaStream_t s, int pstride, int poff, int ncomp, const TriRz *rz) {
+                              cudaStream_t s, int pstride, int poff, int ncomp, const TriRz *rz, const TcOperand *pk) {
   if constexpr (sizeof(T) == 8) {
     if (rz != nullptr) {
-      tri_reg_launch_rz<T, L, MT, GEN, true>(tf, d, y, nrhs, sc, s, pstride, poff, ncomp, rz);
+      tri_reg_launch_rz<T, L, MT, GEN, true, false>(tf, d, y, nrhs, sc, s, pstride, poff, ncomp, rz, nullptr);
+      return;
+    }
+  } else if constexpr (!GEN) {
+    if (pk != nullptr) {
+      tri_reg_launch_rz<T, L, MT, GEN, false, true>(tf, d, y, nrhs, sc, s, pstride, poff, ncomp, nullptr, pk);
       return;
     }
   }
-  tri_reg_launch_rz<T, L, MT, GEN, false>(tf, d, y, nrhs, sc, s, pstride, poff, ncomp, nullptr);
+  tri_reg_launch_rz<T, L, MT, GEN, false, false>(tf, d, y, nrhs, sc, s, pstride, poff, ncomp, nullptr, nullptr);
 }
 
 template <typename T, int L, int MT>
 static void tri_reg_launch_gen(const TriFactors &tf, const T *d, T *y, int nrhs, const KrylovScalars *sc,
-                               cudaStream_t s, int pstride, int poff, int ncomp, const TriRz *rz) {
-  if (tf.gen) tri_reg_launch_mt<T, L, MT, true>(tf, d, y, nrhs, sc, s, pstride, poff, ncomp, rz);
-  else tri_reg_launch_mt<T, L, MT, false>(tf, d, y, nrhs, sc, s, pstride, poff, ncomp, rz);
+                               cudaStream_t s, int pstride, int poff, int ncomp, const TriRz *rz, const TcOperand *pk) {
+  if (tf.gen) tri_reg_launch_mt<T, L, MT, true>(tf, d, y, nrhs, sc, s, pstride, poff, ncomp, rz, pk);
+  else tri_reg_launch_mt<T, L, MT, false>(tf, d, y, nrhs, sc, s, pstride, poff, ncomp, rz, pk);
 }
 
 template <typename T, int L>
 static void tri_reg_launch(const TriFactors &tf, const T *d, T *y, int nrhs, const KrylovScalars *sc, cudaStream_t s,
-                           int pstride, int poff, int ncomp, const TriRz *rz) {
+                           int pstride, int poff, int ncomp, const TriRz *rz, const TcOperand *pk) {
   if constexpr (sizeof(T) == 4) {
-    if (tf.mt == 8) tri_reg_launch_gen<T, L, 8>(tf, d, y, nrhs, sc, s, pstride, poff, ncomp, rz);
+    if (tf.mt == 8) tri_reg_launch_gen<T, L, 8>(tf, d, y, nrhs, sc, s, pstride, poff, ncomp, rz, pk);
     else if constexpr (L <= 32) {
-      if (tf.mt == 32) tri_reg_launch_gen<T, L, 32>(tf, d, y, nrhs, sc, s, pstride, poff, ncomp, rz);
-      else tri_reg_launch_gen<T, L, 16>(tf, d, y, nrhs, sc, s, pstride, poff, ncomp, rz);
+      if (tf.mt == 32) tri_reg_launch_gen<T, L, 32>(tf, d, y, nrhs, sc, s, pstride, poff, ncomp, rz, pk);
+      else tri_reg_launch_gen<T, L, 16>(tf, d, y, nrhs, sc, s, pstride, poff, ncomp, rz, pk);
     } else {
-      tri_reg_launch_gen<T, L, 16>(tf, d, y, nrhs, sc, s, pstride, poff, ncomp, rz);
+      tri_reg_launch_gen<T, L, 16>(tf, d, y, nrhs, sc, s, pstride, poff, ncomp, rz, pk);
     }
   } else {
-    if (tf.mt == 8) tri_reg_launch_gen<T, L, 8>(tf, d, y, nrhs, sc, s, pstride, poff, ncomp, rz);
-    else tri_reg_launch_gen<T, L, 4>(tf, d, y, nrhs, sc, s, pstride, poff, ncomp, rz);
+    if (tf.mt == 8) tri_reg_launch_gen<T, L, 8>(tf, d, y, nrhs, sc, s, pstride, poff, ncomp, rz, pk);
+    else tri_reg_launch_gen<T, L, 4>(tf, d, y, nrhs, sc, s, pstride, poff, ncomp, rz, pk);
   }
 }
 
 template <typename T>
 static void tri_launch(const TriFactors &tf, const T *d, T *y, int nrhs, const KrylovScalars *sc,
-                       cudaStream_t s, int pstride, int poff, int ncomp, const TriRz *rz = nullptr) {
+                       cudaStream_t s, int pstride, int poff, int ncomp, const TriRz *rz = nullptr,
+                       const TcOperand *pk = nullptr) {
   if (nrhs <= 0) return;
   static PerDeviceOnce attr_done;
   attr_done.run([] {
@@ -653,18 +674,19 @@ static void tri_launch(const TriFactors &tf, const T *d, T *y, int nrhs, const K
   ProfScope prof(sizeof(T) == 8 ? KC_TRI64 : KC_TRI32, s);
   if (tf.reg) {
     switch (tf.L) {
-      case 2: tri_reg_launch<T, 2>(tf, d, y, nrhs, sc, s, pstride, poff, ncomp, rz); break;
-      case 4: tri_reg_launch<T, 4>(tf, d, y, nrhs, sc, s, pstride, poff, ncomp, rz); break;
-      case 8: tri_reg_launch<T, 8>(tf, d, y, nrhs, sc, s, pstride, poff, ncomp, rz); break;
-      case 16: tri_reg_launch<T, 16>(tf, d, y, nrhs, sc, s, pstride, poff, ncomp, rz); break;
-      case 32: tri_reg_launch<T, 32>(tf, d, y, nrhs, sc, s, pstride, poff, ncomp, rz); break;
-      default: tri_reg_launch<T, 64>(tf, d, y, nrhs, sc, s, pstride, poff, ncomp, rz); break;
+      case 2: tri_reg_launch<T, 2>(tf, d, y, nrhs, sc, s, pstride, poff, ncomp, rz, pk); break;
+      case 4: tri_reg_launch<T, 4>(tf, d, y, nrhs, sc, s, pstride, poff, ncomp, rz, pk); break;
+      case 8: tri_reg_launch<T, 8>(tf, d, y, nrhs, sc, s, pstride, poff, ncomp, rz, pk); break;
+      case 16: tri_reg_launch<T, 16>(tf, d, y, nrhs, sc, s, pstride, poff, ncomp, rz, pk); break;
+      case 32: tri_reg_launch<T, 32>(tf, d, y, nrhs, sc, s, pstride, poff, ncomp, rz, pk); break;
+      default: tri_reg_launch<T, 64>(tf, d, y, nrhs, sc, s, pstride, poff, ncomp, rz, pk); break;
     }
     count_launch();
     LAG_LAUNCH_CHECK();
     return;
   }
-  if (rz != nullptr) throw Error(LAG_EINVAL, "the (d, y) dot needs the register tridiagonal kernel");
+  if (rz != nullptr || pk != nullptr)
+    throw Error(LAG_EINVAL, "the (d, y) dot and the packed result need the register tridiagonal kernel");
   dim3 grid((tf.nx + tf.mt - 1) / tf.mt, nrhs);
   launch_pdl(tri_solve_kernel<T>, grid, tf.threads, tf.smem, s,
       d, y, tf.nz, tf.nx, tf.P, tf.L, tf.levels, tf.nf, (const T *)tf.fm, (const T *)tf.fc,
@@ -681,6 +703,17 @@ void tri_solve_f64(const TriFactors &tf, const double *d, double *y, int nrhs, c
 void tri_solve_f32(const TriFactors &tf, const float *d, float *y, int nrhs, const KrylovScalars *sc,
                    cudaStream_t s, int pstride, int poff, int ncomp) {
   tri_launch<float>(tf, d, y, nrhs, sc, s, pstride, poff, ncomp);
+}
+
+// Constant coefficients only: 2048 modes x 1024 rows 13.6 + 4.7 us as two kernels, 15.8 us as one (32
+// right-hand sides 171 + 81, 209 us); with a factor set per partition the addresses of both do not
+// fit the registers (512 modes x 768 radii: 18.4 + 3.4 against 30 us)
+bool tri_packs(const TriFactors &tf) { return tf.reg && !tf.gen; }
+bool tri_solve_f32_packed(const TriFactors &tf, const float *d, const TcOperand &out, int nplanes,
+                          const KrylovScalars *sc, cudaStream_t s, int pstride, int poff, int ncomp) {
+  if (!tri_packs(tf)) return false;
+  tri_launch<float>(tf, d, nullptr, nplanes, sc, s, pstride, poff, ncomp, nullptr, &out);
+  return true;
 }
 
 bool tri_rz_fusable(const TriFactors &tf, const Reduce &red) {

@@ -60,9 +60,14 @@ void precond_apply_multi(lag_precond *p1, lag_precond *p2, const double *r, doub
     float *w = p1->scratch.as<float>();
     if (p1->use_tc) dst_apply_tc_d2f(p1->dst, r, w, rows, rpr, sc, s);
     else dst_apply_f32_d2f(p1->dst, r, w, rows, rpr, sc, s);
-    tri_solve_f32(p1->tri32, w, w, nrhs, sc, s, ncomp, 0, ncomp);
-    tri_solve_f32(p2->tri32, w, w, nrhs, sc, s, ncomp, 1, ncomp);
-    if (p1->use_tc) dst_apply_tc_f2d(p1->dst, w, z, rows, rpr, sc, s);
+    const lag_precond *pc[2] = {p1, p2};
+    const TcOperand op = p1->use_tc ? dst_tc_operand(p1->dst, rows) : TcOperand{};
+    const bool packed = p1->use_tc && tri_packs(p1->tri32) && tri_packs(p2->tri32);
+    for (int c = 0; c < 2; ++c) {
+      if (packed) tri_solve_f32_packed(pc[c]->tri32, w, op, nrhs, sc, s, ncomp, c, ncomp);
+      else tri_solve_f32(pc[c]->tri32, w, w, nrhs, sc, s, ncomp, c, ncomp);
+    }
+    if (p1->use_tc) dst_apply_tc_f2d(p1->dst, packed ? nullptr : w, z, rows, rpr, sc, s);
     else dst_inverse_f32_f2d(p1->dst, w, z, rows, rpr, sc, s);
   }
 }
@@ -180,8 +185,9 @@ void KrylovWork::pcg_iteration() {
     float *w = p1->scratch.as<float>();
     if (packs) dst_forward_packed_f32(p1->dst, w, rows, rpr, sc(), stream);
     else dst_apply_tc_d2f(p1->dst, r(), w, rows, rpr, sc(), stream, true);
-    tri_solve_f32(p1->tri32, w, w, nrhs, sc(), stream);
-    dst_apply_tc_f2d_beta(p1->dst, w, z, nrhs, rpr, r(), q, flexible, sc(), rd, stream);
+    const bool packed = tri_solve_f32_packed(p1->tri32, w, dst_tc_operand(p1->dst, rows), nrhs, sc(), stream);
+    if (!packed) tri_solve_f32(p1->tri32, w, w, nrhs, sc(), stream);
+    dst_apply_tc_f2d_beta(p1->dst, packed ? nullptr : w, z, nrhs, rpr, r(), q, flexible, sc(), rd, stream);
   } else if (packs || (p1->prec == LAG_FP64 && p1->dst.kind == 0 && tri_rz_fusable(p1->tri64, rd))) {
     double *w = p1->scratch.as<double>();
     if (packs) dst_forward_packed_f64(p1->dst, w, rows, rpr, sc(), stream);
