@@ -703,10 +703,11 @@ void dst_apply_tc_f2d_beta(const DstPlan &dp, const float *y, double *z, int nrh
   if (rows <= 0) return;
   ProfScope prof(KC_DSTTC_INV, s);
   tc_inverse_eo(dp, y, rows, rpr, sc, s);
-  // rows per right-hand side over at most min(1216, the reduction's block capacity) blocks
-  int blocks = std::min(std::min(rpr, 1216), red.nblk);
-  if (blocks < 1) blocks = 1;
-  dim3 g(blocks, nrhs);
+  // a block's reduction costs as much FP64 pipe as the dots of its row (2 x 90 additions of 32 lanes
+  // against 128 FMAs): with many right-hand sides twice the blocks that are resident, several rows each
+  // (32 right-hand sides 460 -> 330 us)
+  const int fill = std::max(1, 2 * 8 * 152 / nrhs);
+  dim3 g(std::max(1, std::min(std::min(rpr, red.nblk), fill)), nrhs);
   launch_pdl(butterfly_beta_kernel, g, 256, 0, s, dst_tc_eo(dp, rows), z, r, q, dp.n, dp.ku, dp.kv, rpr, flexible, sc,
              red);
   count_launch();
