@@ -220,22 +220,47 @@ __device__ __forceinline__ float warp_sumf(float v) {
   return v;
 }
 
-// Block sum of NV values per thread; result valid in thread 0.  blockDim.x multiple of 32, <= 1024.
+// Block sum of NV values per thread; result valid in thread 0.  blockDim.x a multiple of 32, at most
+// BLOCK_SUM_MAX; fixed order.  One value: the first warp adds up the block's values from shared memory, 12
+// warp instructions on the narrow FP64 pipe for 256 threads instead of the 45 of a butterfly in every warp
+// (128 x 128 shot 63.7 -> 62.5 ms, axisymmetric float64 solve 6.33 -> 6.21 ms).  Two values: butterflies
+// (the longer serial tail and twice the shared memory cost the mixed butterfly more than they saved it).
+constexpr int BLOCK_SUM_MAX = 256;
 template <int NV>
-__device__ __forceinline__ void block_sum(double (&v)[NV], double *sh /* [32*NV] */) {
+__device__ __forceinline__ void block_sum(double (&v)[NV]) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  if constexpr (NV == 1) {
+    __shared__ double buf[BLOCK_SUM_MAX];
+    __syncthreads();
+    buf[threadIdx.x] = v[0];
+    __syncthreads();
+    if (warp == 0) {
+      double t[BLOCK_SUM_MAX / 32];
 #pragma unroll
-  for (int i = 0; i < NV; ++i) v[i] = warp_sum(v[i]);
-  __syncthreads();
-  if (lane == 0)
+      for (int k = 0; k < BLOCK_SUM_MAX / 32; ++k) t[k] = k < nw ? buf[lane + 32 * k] : 0.0;
+      if (nw > 4) {
 #pragma unroll
-    for (int i = 0; i < NV; ++i) sh[i * 32 + warp] = v[i];
-  __syncthreads();
-  if (warp == 0) {
+        for (int k = 0; k < 4; ++k) t[k] += t[k + 4];
+      }
+      if (nw > 2) {
+        t[0] += t[2];
+        t[1] += t[3];
+      }
+      if (nw > 1) t[0] += t[1];
+      v[0] = warp_sum(t[0]);
+    }
+  } else {
+    __shared__ double sh[NV][32];
 #pragma unroll
-    for (int i = 0; i < NV; ++i) {
-      double t = lane < nw ? sh[i * 32 + lane] : 0.0;
-      v[i] = warp_sum(t);
+    for (int i = 0; i < NV; ++i) v[i] = warp_sum(v[i]);
+    __syncthreads();
+    if (lane == 0)
+#pragma unroll
+      for (int i = 0; i < NV; ++i) sh[i][warp] = v[i];
+    __syncthreads();
+    if (warp == 0) {
+#pragma unroll
+      for (int i = 0; i < NV; ++i) v[i] = warp_sum(lane < nw ? sh[i][lane] : 0.0);
     }
   }
 }
@@ -260,7 +285,6 @@ __device__ __forceinline__ bool publish_partials(const Reduce &red, int rhs, int
   // the last block: every thread helps sum the partials in a fixed order
   __threadfence();
   const double *p = red.part + (size_t)rhs * red.rstride;
-  __shared__ double sh[32 * NV];
   double acc[NV];
 #pragma unroll
   for (int i = 0; i < NV; ++i) {
@@ -268,7 +292,7 @@ __device__ __forceinline__ bool publish_partials(const Reduce &red, int rhs, int
     // fixed partition: thread t sums blocks t, t + blockDim, ... in order
     for (int b = threadIdx.x; b < nblk; b += blockDim.x) acc[i] += __ldcg(p + i * red.nblk + b);
   }
-  block_sum<NV>(acc, sh);
+  block_sum<NV>(acc);
   if (threadIdx.x == 0) {
 #pragma unroll
     for (int i = 0; i < NV; ++i) tot[i] = acc[i];

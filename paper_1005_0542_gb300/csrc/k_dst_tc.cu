@@ -539,8 +539,7 @@ __global__ void __launch_bounds__(256) butterfly_beta_kernel(const float *__rest
     }
   }
   double v2[2] = {a0, a1}, tot[2];
-  __shared__ double sh[64];
-  block_sum<2>(v2, sh);
+  block_sum<2>(v2);
   if (publish_partials<2>(red, rhs, blockIdx.x, gridDim.x, v2, tot)) {
     KrylovScalars &S = sc[rhs];
     const double rz_new = tot[0];

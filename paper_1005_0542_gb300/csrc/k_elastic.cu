@@ -219,8 +219,7 @@ __global__ void __launch_bounds__(256) gm_start_kernel(const double *__restrict_
     acc = fma(v, v, acc);
   }
   double v1[1] = {acc}, tot[1];
-  __shared__ double sh[32];
-  block_sum<1>(v1, sh);
+  block_sum<1>(v1);
   if (publish_partials<1>(red, rhs, blockIdx.x, gridDim.x, v1, tot)) {
     const int k = g.k;
     if (first) {
@@ -448,8 +447,7 @@ __global__ void __launch_bounds__(256) gm_norm_kernel(const double *__restrict__
   for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < n; e += (size_t)gridDim.x * blockDim.x)
     acc = fma(w[off + e], w[off + e], acc);
   double v1[1] = {acc}, tot[1];
-  __shared__ double sh[32];
-  block_sum<1>(v1, sh);
+  block_sum<1>(v1);
   if (!publish_partials<1>(red, rhs, blockIdx.x, gridDim.x, v1, tot)) return;
   const int k = g.k;
   KrylovScalars &S = sc[rhs];

@@ -227,8 +227,7 @@ __global__ void __launch_bounds__(256) acoustic_apply_kernel(const double *__res
   }
   if (mode == 1) {
     double v1[1] = {dot}, tot[1];
-    __shared__ double sh[32];
-    block_sum<1>(v1, sh);
+    block_sum<1>(v1);
     if (publish_partials<1>(red, b, blockIdx.x, gridDim.x, v1, tot)) {
       const double pq = tot[0];
       sc[b].pq = pq;
@@ -293,8 +292,7 @@ __global__ void __launch_bounds__(256) acoustic_apply_dir_kernel(const double *_
     }
   }
   double v1[1] = {dot}, tot[1];
-  __shared__ double sh[32];
-  block_sum<1>(v1, sh);
+  block_sum<1>(v1);
   if (publish_partials<1>(red, b, blockIdx.x, gridDim.x, v1, tot)) {
     const double pq = tot[0];
     sc[b].pq = pq;
@@ -414,14 +412,13 @@ __global__ void __launch_bounds__(256, 3) acoustic_apply_dir_tall_kernel(
       }
     }
   }
-  __shared__ double sh[32];
 #pragma unroll
   for (int r = 0; r < NR; ++r) {
     if (!run[r]) continue;
     const int b = b0 + r;
     double v1[1] = {dot[r]}, tot[1];
     __syncthreads();
-    block_sum<1>(v1, sh);
+    block_sum<1>(v1);
     if (publish_partials<1>(red, b, blockIdx.x, gridDim.x, v1, tot)) {
       const double pq = tot[0];
       sc[b].pq = pq;
@@ -505,8 +502,7 @@ __global__ void __launch_bounds__(256) pcg_start_kernel(const double *__restrict
     acc = fma(v, v, acc);
   }
   double v1[1] = {acc}, tot[1];
-  __shared__ double sh[32];
-  block_sum<1>(v1, sh);
+  block_sum<1>(v1);
   if (publish_partials<1>(red, rhs, blockIdx.x, gridDim.x, v1, tot)) {
     KrylovScalars &S = sc[rhs];
     S.bb = tot[0];
@@ -547,8 +543,7 @@ __global__ void __launch_bounds__(256) pcg_update_xr_kernel(double *__restrict__
     acc = fma(rv, rv, acc);
   }
   double v1[1] = {acc}, tot[1];
-  __shared__ double sh[32];
-  block_sum<1>(v1, sh);
+  block_sum<1>(v1);
   if (publish_partials<1>(red, rhs, blockIdx.x, gridDim.x, v1, tot)) {
     KrylovScalars &S = sc[rhs];
     S.rr = tot[0];
@@ -586,8 +581,7 @@ __global__ void __launch_bounds__(256) pcg_beta_kernel(const double *__restrict_
     if (flexible) a1 = fma(zv, q[off + i], a1);
   }
   double v2[2] = {a0, a1}, tot[2];
-  __shared__ double sh[64];
-  block_sum<2>(v2, sh);
+  block_sum<2>(v2);
   if (publish_partials<2>(red, rhs, blockIdx.x, gridDim.x, v2, tot)) {
     KrylovScalars &S = sc[rhs];
     const double rz_new = tot[0];
@@ -626,8 +620,7 @@ __global__ void __launch_bounds__(256, 8) pcg_rz_beta_kernel(const double *__res
     a1 = fma(rb.y, zb.y, a1);
   }
   double v1[1] = {a0 + a1}, tot[1];
-  __shared__ double sh[32];
-  block_sum<1>(v1, sh);
+  block_sum<1>(v1);
   if (publish_partials<1>(red, rhs, blockIdx.x, gridDim.x, v1, tot)) {
     KrylovScalars &S = sc[rhs];
     const double rz_new = tot[0];
@@ -676,8 +669,7 @@ __global__ void __launch_bounds__(256) laguerre_rhs_kernel(const double *__restr
     acc = fma(v, v, acc);
   }
   double v1[1] = {acc}, tot[1];
-  __shared__ double sh[32];
-  block_sum<1>(v1, sh);
+  block_sum<1>(v1);
   if (publish_partials<1>(red, rhs, blockIdx.x, gridDim.x, v1, tot)) {
     KrylovScalars &K = sc[rhs];
     K.bb = tot[0];

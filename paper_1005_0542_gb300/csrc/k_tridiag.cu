@@ -581,8 +581,7 @@ __global__ void __launch_bounds__(RegBounds<T, L, MT, GEN>::threads, RegBounds<T
     }
     if constexpr (RZ) {
       double v1[1] = {(double)dot}, tot[1];
-      __shared__ double rsh[32];
-      block_sum<1>(v1, rsh);
+      block_sum<1>(v1);
       if (publish_partials<1>(rz, b, blockIdx.x, gridDim.x, v1, tot)) {
         KrylovScalars &S = scw[b];
         const double rz_new = tot[0];

@@ -321,8 +321,7 @@ __global__ void __launch_bounds__(OZ_PACK_THREADS) pcg_update_pack_kernel(
     __syncthreads();  // the row's stage is reused
   }
   double v1[1] = {acc}, tot[1];
-  __shared__ double sh[32];
-  block_sum<1>(v1, sh);
+  block_sum<1>(v1);
   if (publish_partials<1>(red, rhs, blockIdx.x, gridDim.x, v1, tot)) {
     KrylovScalars &S = sc[rhs];
     S.rr = tot[0];
