@@ -249,8 +249,9 @@ struct lag_precond {
 
 namespace lag {
 // K^{-1} for ncomp interleaved components ([rhs][comp][nz][nx]): component 0 with p1, 1 with p2.
+// r_packed: p1's scratch holds r as the mixed forward transform's operand (gm_scale_pack).
 void precond_apply_multi(lag_precond *p1, lag_precond *p2, const double *r, double *z, int nrhs,
-                         int ncomp, const KrylovScalars *sc, cudaStream_t s);
+                         int ncomp, const KrylovScalars *sc, cudaStream_t s, bool r_packed = false);
 }
 
 // ----------------------------------------------------------------------------- medium
@@ -329,15 +330,19 @@ struct GmresDev {
   double *hcol;                  // per rhs: [k+1] current column (Gram-Schmidt coefficients)
   int k;
 };
-void gm_start(const double *b, const double *cx, double *v0, size_t n, int nrhs, int first,
-              double tol, int max_iter, KrylovScalars *sc, GmresDev &g, const Reduce &red,
+void gm_start(const double *b, const double *cx, size_t n, int nrhs, int first, double tol, int max_iter,
+              KrylovScalars *sc, GmresDev &g, const Reduce &red, cudaStream_t s);
+// v = w / nrm[rhs nstride] for running systems; gm_scale_pack also packs v as the operand of the mixed
+// forward transform (rows: planes of all components and right-hand sides, rpr per right-hand side)
+void gm_scale(const double *w, double *v, size_t n, int nrhs, const KrylovScalars *sc, const double *nrm, int nstride,
               cudaStream_t s);
+void gm_scale_pack(const DstPlan &dp, const double *w, double *v, int nrhs, int rpr, const KrylovScalars *sc,
+                   const double *nrm, int nstride, cudaStream_t s);
+// one Gram-Schmidt pass; the last one of a step also takes ||w||, rotates column j and updates the state.
 // shifted: w holds C z_j - V_j (the shifted Arnoldi step); h_jj gets the 1 back
 void gm_orthogonalize(double *w, const double *V, int j, size_t n, int nrhs, size_t vstride,
                       KrylovScalars *sc, GmresDev &g, const Reduce &red, int pass, bool shifted,
-                      cudaStream_t s);
-void gm_normalize(double *w, double *vnext, int j, size_t n, int nrhs, KrylovScalars *sc,
-                  GmresDev &g, const Reduce &red, int max_iter, cudaStream_t s);
+                      int max_iter, cudaStream_t s);
 void gm_update_x(double *x, const double *Z, int jdone, size_t n, int nrhs, size_t zstride,
                  const KrylovScalars *sc, GmresDev &g, cudaStream_t s);
 

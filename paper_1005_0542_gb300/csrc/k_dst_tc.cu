@@ -147,6 +147,11 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float (&v)[16]) {
 
 }  // namespace
 
+// index j of a row staged in shared memory at j + j / 8: a thread's 8 consecutive values (or the mirrored
+// ones) then sit 9 apart from its neighbour's, so their reads hit every bank once (unpadded doubles,
+// lanes 64 bytes apart, fell on two banks: 16-way conflicts)
+#define OZ_PAD(j) ((j) + ((j) >> 3))
+
 // ------------------------------------------------------------------------------ packing
 // B operands, once per plan.  which: 0 fwd even (B[n][k] = S[k][2n]), 1 fwd odd (S[k][2n+1]),
 // 2 inv E (S[n][2k]), 3 inv O (S[n][2k+1], zero row at n = kv for odd n).  Layout per matrix:
@@ -215,6 +220,73 @@ __global__ void __launch_bounds__(256) pack_a_fwd_kernel(const TI *__restrict__ 
     *reinterpret_cast<uint4 *>(tile + off) = *reinterpret_cast<const uint4 *>(par ? vh : uh);
     *reinterpret_cast<uint4 *>(tile + A_TILE + off) = *reinterpret_cast<const uint4 *>(par ? vl : ul);
   }
+}
+
+// the operand chunks of one row staged as float (index j at OZ_PAD(j)), by all threads of the CTA
+__device__ __forceinline__ void tc_pack_row(const float *xf, int row, int n, int ku, int kv, int nks, int nmt,
+                                            uint8_t *out) {
+  const int mt = row / TM, r = row % TM;
+  for (int ch = threadIdx.x; ch < nks * (TK / 8); ch += blockDim.x) {
+    alignas(16) uint16_t uh[8], ul[8], vh[8], vl[8];
+#pragma unroll
+    for (int e = 0; e < 8; ++e) {
+      const int j = ch * 8 + e;
+      float u = 0.f, w = 0.f;
+      if (j < kv) {
+        const float f1 = xf[OZ_PAD(j)], f2 = xf[OZ_PAD(n - 1 - j)];
+        u = f1 + f2;
+        w = f1 - f2;
+      } else if (j < ku) {
+        u = xf[OZ_PAD(j)];  // middle element of an odd-length row
+      }
+      split2f(u, uh[e], ul[e]);
+      split2f(w, vh[e], vl[e]);
+    }
+    const uint32_t off = swz(r, (ch * 8) % TK);
+    for (int par = 0; par < 2; ++par) {
+      uint8_t *tile = out + (((size_t)par * nmt + mt) * nks + (ch * 8) / TK) * 2 * A_TILE;
+      *reinterpret_cast<uint4 *>(tile + off) = *reinterpret_cast<const uint4 *>(par ? vh : uh);
+      *reinterpret_cast<uint4 *>(tile + A_TILE + off) = *reinterpret_cast<const uint4 *>(par ? vl : ul);
+    }
+  }
+}
+
+// FGMRES: v = w / nrm, the next basis vector, with the operand of its forward transform (one pass over w
+// instead of two and one over v).  A CTA per row of the running right-hand sides; grid (rows, nrhs).
+__global__ void __launch_bounds__(128) gm_scale_pack_kernel(const double *__restrict__ w, double *__restrict__ v, int n,
+                                                            int rpr, int ku, int kv, int nks, int nmt,
+                                                            uint8_t *__restrict__ out,
+                                                            const KrylovScalars *__restrict__ sc,
+                                                            const double *__restrict__ nrm, int nstride) {
+  pdl_next();
+  pdl_wait();
+  extern __shared__ float gmx[];
+  const int rhs = blockIdx.y;
+  if (sc[rhs].state != ST_RUN) return;
+  const double s = nrm[(size_t)rhs * nstride];
+  if (!(s > 0.0)) return;
+  const double inv = 1.0 / s;
+  const int row = rhs * rpr + blockIdx.x;
+  const size_t o = (size_t)row * n;
+  constexpr int PB = 8;
+  for (int jb = 0; jb < n; jb += PB * 128) {
+    double wv[PB];
+#pragma unroll
+    for (int u = 0; u < PB; ++u) {
+      const int j = jb + u * 128 + threadIdx.x;
+      wv[u] = j < n ? w[o + j] : 0.0;
+    }
+#pragma unroll
+    for (int u = 0; u < PB; ++u) {
+      const int j = jb + u * 128 + threadIdx.x;
+      if (j >= n) continue;
+      const double x = wv[u] * inv;
+      v[o + j] = x;
+      gmx[OZ_PAD(j)] = narrow_pow2(x, 0);
+    }
+  }
+  __syncthreads();
+  tc_pack_row(gmx, row, n, ku, kv, nks, nmt, out);
 }
 
 // A operand of the inverse transform from the parity-permuted spectrum (no fold)
@@ -944,10 +1016,6 @@ __global__ void oz_pack_b_kernel(const double *m0, int k0n, int n0n, int ld0, co
 // Layout [parity][slice][m tile][k stage][TM x TK]; erow[parity][row] = e_r with |values| < 2^e_r.
 constexpr int OZ_PACK_THREADS = 128;  // 62 registers: 128-thread CTAs keep every row of a shot resident at once
 constexpr int OZ_PACK_MAXK = 4224;  // ceil(n / 2) bound of the exact-slice path (K pad <= 4224)
-// the staged row's index j at j + j / 8: a thread's 8 consecutive values (or the mirrored ones)
-// then sit 9 doubles from its neighbour's, so a half-warp's 8-byte reads hit every bank once
-// (unpadded, lanes 64 bytes apart fell on two banks: 16-way conflicts)
-#define OZ_PAD(j) ((j) + ((j) >> 3))
 static size_t oz_pack_smem(int nks) { return (size_t)(2 * nks * TK + (2 * nks * TK) / 8 + 8) * sizeof(double); }
 // gather (DCT-II inverse): u = the even entries x[2j], v = the odd ones x[2j+1] instead of the fold.
 template <int NB, int NS>
@@ -2811,6 +2879,19 @@ void dst_pack_residual(const DstPlan &dp, const double *r, int rows, int rpr, co
 void dst_forward_packed_f64(const DstPlan &dp, double *y, int rows, int rpr, const KrylovScalars *sc, cudaStream_t s) {
   ProfScope prof(KC_DST64, s);
   ow_gemm(dp, y, rows, rpr, sc, s, 0);
+}
+
+void gm_scale_pack(const DstPlan &dp, const double *w, double *v, int nrhs, int rpr, const KrylovScalars *sc,
+                   const double *nrm, int nstride, cudaStream_t s) {
+  static PerDeviceOnce attr;
+  attr.run([] {
+    LAG_CUDA_CHECK(cudaFuncSetAttribute(gm_scale_pack_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024));
+  });
+  ProfScope prof(KC_GMRES, s);
+  launch_pdl(gm_scale_pack_kernel, dim3(rpr, nrhs), 128, oz_pack_smem(dp.kpad_u) / 2, s, w, v, dp.n, rpr, dp.ku, dp.kv,
+             dp.kpad_u, div_up(nrhs * rpr, TM), dp.tc_scratch, sc, nrm, nstride);
+  count_launch();
+  LAG_LAUNCH_CHECK();
 }
 
 void pcg_update_pack(const DstPlan &dp, double *x, double *r, const double *p, const double *q, int nrhs, int rpr,

@@ -255,14 +255,20 @@ __global__ void gm_scale_kernel(const double *__restrict__ w, double *__restrict
     v[off + i] = w[off + i] * inv;
 }
 
-void gm_start(const double *b, const double *cx, double *v0, size_t n, int nrhs, int first, double tol,
-              int max_iter, KrylovScalars *sc, GmresDev &g, const Reduce &red, cudaStream_t s) {
+void gm_scale(const double *w, double *v, size_t n, int nrhs, const KrylovScalars *sc, const double *nrm, int nstride,
+              cudaStream_t s) {
+  ProfScope prof(KC_GMRES, s);
+  dim3 grid(reduce_blocks(n), nrhs);
+  launch_pdl(gm_scale_kernel, grid, 256, 0, s, w, v, n, sc, nrm, nstride);
+  count_launch();
+  LAG_LAUNCH_CHECK();
+}
+
+void gm_start(const double *b, const double *cx, size_t n, int nrhs, int first, double tol, int max_iter,
+              KrylovScalars *sc, GmresDev &g, const Reduce &red, cudaStream_t s) {
   ProfScope prof(KC_GMRES, s);
   dim3 grid(reduce_blocks(n), nrhs);
   launch_pdl(gm_start_kernel, grid, 256, 0, s, b, const_cast<double *>(cx), n, first, tol * tol, max_iter, sc, g, red);
-  count_launch();
-  LAG_LAUNCH_CHECK();
-  launch_pdl(gm_scale_kernel, grid, 256, 0, s, cx, v0, n, sc, g.g, g.k + 1);
   count_launch();
   LAG_LAUNCH_CHECK();
 }
@@ -385,18 +391,18 @@ __global__ void __launch_bounds__(256) gm_dots_kernel(const double *__restrict__
     if (lane == 0) tot[v] = a;
   }
   __syncthreads();
-  if (threadIdx.x == 0) {
-    const int k = g.k;
+  // a thread per coefficient (one thread alone spent longer on the loads than the dots take on small grids)
+  const int k = g.k, t = threadIdx.x;
+  if (t <= j) {
     double *hc = g.hcol + (size_t)rhs * (k + 1);
-    double *tmp = g.y + (size_t)rhs * k;  // this pass's coefficients
-    double hsum = 0.0;
-    for (int i = 0; i <= j; ++i) {
-      const double h = tot[i];
-      tmp[i] = h;
-      hc[i] = pass == 0 ? (shifted && i == j ? h + 1.0 : h) : hc[i] + h;
-      hsum = fma(h, h, hsum);
-    }
+    const double h = tot[t];
+    g.y[(size_t)rhs * k + t] = h;  // this pass's coefficients
+    hc[t] = pass == 0 ? (shifted && t == j ? h + 1.0 : h) : hc[t] + h;
+  }
+  if (t == 0) {
     if (pass == 0) {
+      double hsum = 0.0;
+      for (int i = 0; i <= j; ++i) hsum = fma(tot[i], tot[i], hsum);
       const double wnorm2 = tot[j + 1], rest = wnorm2 - hsum;
       sc[rhs].reorth = (rest > 0.5 * wnorm2 && isfinite(rest)) ? 0 : 1;
     }
@@ -404,102 +410,92 @@ __global__ void __launch_bounds__(256) gm_dots_kernel(const double *__restrict__
   }
 }
 
-// w -= sum_i tmp_i V_i
+// w -= sum_i tmp_i V_i; in the step's last pass (the second one, or the first where that is skipped) also
+// (w, w), from which the last block finishes the step: h_{j+1,j} = ||w||, the Givens rotations of column j,
+// the update of g and the residual estimate -> state.  The block loads the column's coefficients and
+// rotations at once; one thread applies them.
 __global__ void __launch_bounds__(256) gm_axpy_kernel(double *__restrict__ w, const double *__restrict__ V, int j,
-                                                      size_t n, size_t vstride, const KrylovScalars *sc, GmresDev g,
-                                                      int pass) {
+                                                      size_t n, size_t vstride, KrylovScalars *sc, GmresDev g,
+                                                      Reduce red, int pass, int max_iter) {
   pdl_next();
   pdl_wait();
   const int rhs = blockIdx.y;
   if (sc[rhs].state != ST_RUN) return;
-  if (pass == 1 && sc[rhs].reorth == 0) return;
+  const bool again = sc[rhs].reorth != 0;
+  if (pass == 1 && !again) return;
+  const bool last_pass = pass == 1 || !again;
   const size_t off = (size_t)rhs * n;
   const double *tmp = g.y + (size_t)rhs * g.k;
-  for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < n; e += (size_t)gridDim.x * blockDim.x) {
-    double v = w[off + e];
-    for (int i = 0; i <= j; ++i) v = fma(-tmp[i], V[(size_t)i * vstride + off + e], v);
-    w[off + e] = v;
+  double acc = 0.0;
+  if (last_pass) {
+    for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < n; e += (size_t)gridDim.x * blockDim.x) {
+      double v = w[off + e];
+      for (int i = 0; i <= j; ++i) v = fma(-tmp[i], V[(size_t)i * vstride + off + e], v);
+      w[off + e] = v;
+      acc = fma(v, v, acc);
+    }
+  } else {
+    for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < n; e += (size_t)gridDim.x * blockDim.x) {
+      double v = w[off + e];
+      for (int i = 0; i <= j; ++i) v = fma(-tmp[i], V[(size_t)i * vstride + off + e], v);
+      w[off + e] = v;
+    }
+    return;
   }
+  double v1[1] = {acc}, tot[1];
+  block_sum<1>(v1);
+  __shared__ bool finish;
+  __shared__ double hs[72], cv[72], sv[72];
+  const bool mine = publish_partials<1>(red, rhs, blockIdx.x, gridDim.x, v1, tot);
+  if (threadIdx.x == 0) finish = mine;
+  __syncthreads();
+  if (!finish) return;
+  const int k = g.k, t = threadIdx.x;
+  double *cs = g.cs + (size_t)rhs * k, *sn = g.sn + (size_t)rhs * k, *gg = g.g + (size_t)rhs * (k + 1);
+  double *col = g.H + (size_t)rhs * (k + 1) * k + (size_t)j * (k + 1);  // column-major: H[col * (k+1) + row]
+  if (t <= j) hs[t] = g.hcol[(size_t)rhs * (k + 1) + t];
+  if (t < j) {
+    cv[t] = cs[t];
+    sv[t] = sn[t];
+  }
+  __syncthreads();
+  if (t == 0) {
+    KrylovScalars &S = sc[rhs];
+    const double hnext = sqrt(tot[0]);
+    double c0 = hs[0];
+    for (int i = 0; i < j; ++i) {
+      const double c1 = hs[i + 1];
+      hs[i] = cv[i] * c0 + sv[i] * c1;
+      c0 = -sv[i] * c0 + cv[i] * c1;
+    }
+    const double den = hypot(c0, hnext), g0 = gg[j];
+    const double c = c0 / den, sj = hnext / den;
+    cs[j] = c;
+    sn[j] = sj;
+    hs[j] = den;
+    hs[j + 1] = hnext;  // kept for the scaling of V_{j+1}; not part of the triangular factor
+    const double g1 = -sj * g0;
+    gg[j + 1] = g1;
+    gg[j] = c * g0;
+    S.iters += 1;
+    S.jdone = j + 1;
+    S.rr = g1 * g1;
+    if (!isfinite(S.rr) || !isfinite(den)) S.state = ST_NAN;
+    else if (S.rr <= S.tol2 * S.bb || hnext == 0.0 || S.iters >= max_iter || j + 1 >= k) S.state = ST_MET;
+  }
+  __syncthreads();
+  if (t <= j + 1) col[t] = hs[t];
 }
 
 void gm_orthogonalize(double *w, const double *V, int j, size_t n, int nrhs, size_t vstride, KrylovScalars *sc,
-                      GmresDev &g, const Reduce &red, int pass, bool shifted, cudaStream_t s) {
+                      GmresDev &g, const Reduce &red, int pass, bool shifted, int max_iter, cudaStream_t s) {
   ProfScope prof(KC_GMRES, s);
   if (j + 2 > 72) throw Error(LAG_EINVAL, "GMRES restart length above 70");
   dim3 gd(dots_blocks(n), nrhs), grid(reduce_blocks(n), nrhs);
   launch_pdl(gm_dots_kernel, gd, 256, 0, s, w, V, j, n, vstride, sc, g, red, pass, shifted ? 1 : 0);
   count_launch();
   LAG_LAUNCH_CHECK();
-  launch_pdl(gm_axpy_kernel, grid, 256, 0, s, w, V, j, n, vstride, sc, g, pass);
-  count_launch();
-  LAG_LAUNCH_CHECK();
-}
-
-// h_{j+1,j} = ||w||; Givens rotations on column j; g update; residual estimate -> state
-__global__ void __launch_bounds__(256) gm_norm_kernel(const double *__restrict__ w, int j, size_t n,
-                                                      KrylovScalars *sc, GmresDev g, Reduce red, int max_iter) {
-  pdl_next();
-  pdl_wait();
-  const int rhs = blockIdx.y;
-  if (sc[rhs].state != ST_RUN) return;
-  const size_t off = (size_t)rhs * n;
-  double acc = 0.0;
-  for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < n; e += (size_t)gridDim.x * blockDim.x)
-    acc = fma(w[off + e], w[off + e], acc);
-  double v1[1] = {acc}, tot[1];
-  block_sum<1>(v1);
-  if (!publish_partials<1>(red, rhs, blockIdx.x, gridDim.x, v1, tot)) return;
-  const int k = g.k;
-  KrylovScalars &S = sc[rhs];
-  double *H = g.H + (size_t)rhs * (k + 1) * k;  // column-major: H[col * (k+1) + row]
-  double *cs = g.cs + (size_t)rhs * k, *sn = g.sn + (size_t)rhs * k, *gg = g.g + (size_t)rhs * (k + 1);
-  const double *hc = g.hcol + (size_t)rhs * (k + 1);
-  double *col = H + (size_t)j * (k + 1);
-  const double hnext = sqrt(tot[0]);
-  for (int i = 0; i <= j; ++i) col[i] = hc[i];
-  col[j + 1] = hnext;
-  for (int i = 0; i < j; ++i) {
-    const double t = cs[i] * col[i] + sn[i] * col[i + 1];
-    col[i + 1] = -sn[i] * col[i] + cs[i] * col[i + 1];
-    col[i] = t;
-  }
-  const double den = hypot(col[j], col[j + 1]);
-  cs[j] = col[j] / den;
-  sn[j] = col[j + 1] / den;
-  col[j] = den;
-  col[j + 1] = hnext;  // kept for the scaling of V_{j+1}; not part of the triangular factor
-  gg[j + 1] = -sn[j] * gg[j];
-  gg[j] = cs[j] * gg[j];
-  S.iters += 1;
-  S.jdone = j + 1;
-  S.rr = gg[j + 1] * gg[j + 1];
-  if (!isfinite(S.rr) || !isfinite(den)) S.state = ST_NAN;
-  else if (S.rr <= S.tol2 * S.bb || hnext == 0.0 || S.iters >= max_iter || j + 1 >= k) S.state = ST_MET;
-}
-
-// V_{j+1} = w / h_{j+1,j}  (only systems still expanding)
-__global__ void gm_next_kernel(const double *__restrict__ w, double *__restrict__ v, int j, size_t n,
-                               const KrylovScalars *sc, GmresDev g) {
-  pdl_next();
-  pdl_wait();
-  const int rhs = blockIdx.y;
-  if (sc[rhs].state != ST_RUN) return;
-  const int k = g.k;
-  const double h = g.H[(size_t)rhs * (k + 1) * k + (size_t)j * (k + 1) + j + 1];
-  const double inv = 1.0 / h;
-  const size_t off = (size_t)rhs * n;
-  for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < n; e += (size_t)gridDim.x * blockDim.x)
-    v[off + e] = w[off + e] * inv;
-}
-
-void gm_normalize(double *w, double *vnext, int j, size_t n, int nrhs, KrylovScalars *sc, GmresDev &g,
-                  const Reduce &red, int max_iter, cudaStream_t s) {
-  ProfScope prof(KC_GMRES, s);
-  dim3 grid(reduce_blocks(n), nrhs);
-  launch_pdl(gm_norm_kernel, grid, 256, 0, s, w, j, n, sc, g, red, max_iter);
-  count_launch();
-  LAG_LAUNCH_CHECK();
-  launch_pdl(gm_next_kernel, grid, 256, 0, s, w, vnext, j, n, sc, g);
+  launch_pdl(gm_axpy_kernel, grid, 256, 0, s, w, V, j, n, vstride, sc, g, red, pass, max_iter);
   count_launch();
   LAG_LAUNCH_CHECK();
 }

@@ -40,7 +40,7 @@ void check_solver(const lag_solver &s, bool elastic) {
 }
 
 void precond_apply_multi(lag_precond *p1, lag_precond *p2, const double *r, double *z, int nrhs, int ncomp,
-                         const KrylovScalars *sc, cudaStream_t s) {
+                         const KrylovScalars *sc, cudaStream_t s, bool r_packed) {
   if (ncomp == 1) {  // PCG: r is the residual whose norm sc[b].rr holds
     p1->apply(r, z, nrhs, sc, s, true);
     return;
@@ -58,7 +58,8 @@ void precond_apply_multi(lag_precond *p1, lag_precond *p2, const double *r, doub
     dst_inverse_f64(p1->dst, w, z, rows, rpr, sc, s);
   } else {
     float *w = p1->scratch.as<float>();
-    if (p1->use_tc) dst_apply_tc_d2f(p1->dst, r, w, rows, rpr, sc, s);
+    if (r_packed) dst_forward_packed_f32(p1->dst, w, rows, rpr, sc, s);
+    else if (p1->use_tc) dst_apply_tc_d2f(p1->dst, r, w, rows, rpr, sc, s);
     else dst_apply_f32_d2f(p1->dst, r, w, rows, rpr, sc, s);
     const lag_precond *pc[2] = {p1, p2};
     const TcOperand op = p1->use_tc ? dst_tc_operand(p1->dst, rows) : TcOperand{};
@@ -445,7 +446,8 @@ void KrylovWork::gmres_begin_cycle(bool first) {
   double *V0 = vec(3);
   Reduce rd = red.get();
   if (!first) m->apply(x(), w, nrhs, sc(), nullptr, 2, stream);  // w = C x for systems still open
-  gm_start(b(), w, V0, n, nrhs, first ? 1 : 0, s.tol, s.max_iter, sc(), gdev, rd, stream);
+  gm_start(b(), w, n, nrhs, first ? 1 : 0, s.tol, s.max_iter, sc(), gdev, rd, stream);
+  gmres_basis(w, V0, gdev.g, gk + 1);
   gj = 0;
   cycle_open = true;
 }
@@ -455,16 +457,26 @@ void KrylovWork::gmres_step() {
   double *V = vec(3), *Z = vec(3 + k + 1), *w = r();
   const size_t vs = n * (size_t)nrhs;
   Reduce rd = red.get();
-  precond(V + (size_t)j * vs, Z + (size_t)j * vs);               // Z_j = K^{-1} V_j
+  // Z_j = K^{-1} V_j
+  precond_apply_multi(p1, p2, V + (size_t)j * vs, Z + (size_t)j * vs, nrhs, ncomp, sc(), stream, r_packed);
   // shifted Arnoldi step: w = C Z_j - V_j spans the same Krylov space (C K^{-1} - I has the
   // Hessenberg matrix H - I), but for a good preconditioner C K^{-1} V_j lies close to V_j and the
   // shift removes that component before the projections, so the first Gram-Schmidt pass cancels
   // less and the second one (selective) is often skipped
   m->apply(Z + (size_t)j * vs, w, nrhs, sc(), nullptr, 0, stream, V + (size_t)j * vs);
-  gm_orthogonalize(w, V, j, n, nrhs, vs, sc(), gdev, rd, 0, true, stream);
-  gm_orthogonalize(w, V, j, n, nrhs, vs, sc(), gdev, rd, 1, true, stream);
-  gm_normalize(w, V + (size_t)(j + 1) * vs, j, n, nrhs, sc(), gdev, rd, s.max_iter, stream);
+  gm_orthogonalize(w, V, j, n, nrhs, vs, sc(), gdev, rd, 0, true, s.max_iter, stream);
+  gm_orthogonalize(w, V, j, n, nrhs, vs, sc(), gdev, rd, 1, true, s.max_iter, stream);
+  // V_{j+1} = w / h_{j+1,j} (only systems still expanding)
+  gmres_basis(w, V + (size_t)(j + 1) * vs, gdev.H + (size_t)j * (k + 1) + j + 1, (k + 1) * k);
   gj = j + 1;
+}
+
+void KrylovWork::gmres_basis(const double *w, double *v, const double *nrm, int nstride) {
+  const int rpr = p1->grid.nz * ncomp;
+  p1->ensure_scratch(nrhs * ncomp);
+  r_packed = p1->use_tc && dst_packs_residual(p1->dst, nrhs * rpr, rpr);
+  if (r_packed) gm_scale_pack(p1->dst, w, v, nrhs, rpr, sc(), nrm, nstride, stream);
+  else gm_scale(w, v, n, nrhs, sc(), nrm, nstride, stream);
 }
 
 void KrylovWork::gmres_end_cycle() {

@@ -293,30 +293,7 @@ __global__ void __launch_bounds__(OZ_PACK_THREADS) pcg_update_pack_kernel(
       ow_pack_row(xs, b0, 0, g, true, n, ku, kv, nk, nmt, out, erow, false);
     } else {
       __syncthreads();
-      const int mt = g / TM, rr = g % TM;
-      for (int ch = threadIdx.x; ch < nk * (TK / 8); ch += OZ_PACK_THREADS) {
-        alignas(16) uint16_t uh[8], ul[8], vh[8], vl[8];
-#pragma unroll
-        for (int e = 0; e < 8; ++e) {
-          const int j = ch * 8 + e;
-          float u = 0.f, w = 0.f;
-          if (j < kv) {
-            const float f1 = xf[OZ_PAD(j)], f2 = xf[OZ_PAD(n - 1 - j)];
-            u = f1 + f2;
-            w = f1 - f2;
-          } else if (j < ku) {
-            u = xf[OZ_PAD(j)];  // middle element of an odd-length row
-          }
-          split2f(u, uh[e], ul[e]);
-          split2f(w, vh[e], vl[e]);
-        }
-        const uint32_t off = swz(rr, (ch * 8) % TK);
-        for (int par = 0; par < 2; ++par) {
-          uint8_t *tile = out + (((size_t)par * nmt + mt) * nk + (ch * 8) / TK) * 2 * A_TILE;
-          *reinterpret_cast<uint4 *>(tile + off) = *reinterpret_cast<const uint4 *>(par ? vh : uh);
-          *reinterpret_cast<uint4 *>(tile + A_TILE + off) = *reinterpret_cast<const uint4 *>(par ? vl : ul);
-        }
-      }
+      tc_pack_row(xf, g, n, ku, kv, nk, nmt, out);
     }
     __syncthreads();  // the row's stage is reused
   }

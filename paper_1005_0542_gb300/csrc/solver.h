@@ -59,7 +59,7 @@ struct KrylovWork {
   DevBuf wcount;             // the loop's repeat counter (a bound on one launch) and its body total
   unsigned long long wbodies_seen = 0;
   bool eager_done = false;
-  bool r_packed = false;     // PCG: the plan's scratch holds the packed operand of the current r
+  bool r_packed = false;     // the plan's scratch holds the packed operand of the current r (GMRES: of V_gj)
   int pcur = 0;              // which of the two direction buffers holds the current p
 
   ~KrylovWork();
@@ -91,6 +91,7 @@ struct KrylovWork {
   void mirror_state();        // async copy of the scalars and the plans' error words + event
   void gmres_begin_cycle(bool first);
   void gmres_step();
+  void gmres_basis(const double *w, double *v, const double *nrm, int nstride);  // v = w / nrm, packed if mixed
   void gmres_end_cycle();
 };
 
