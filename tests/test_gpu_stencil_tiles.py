@@ -77,3 +77,23 @@ def test_packed_update(ctx, nx, nz, nrhs, prec):
             assert np.linalg.norm(r) / np.linalg.norm(b[i]) < 2 * tol
     L.lag_precond_destroy(p)
     L.lag_medium_destroy(m)
+
+
+# the elastic operator on its 64 x 16 tiles (456 or more of them): ragged in both directions, a width
+# below one tile, several right-hand sides
+@pytest.mark.parametrize("nx,nz,nrhs", [(1000, 517, 1), (130, 333, 8), (65, 17, 230), (37, 1030, 9)])
+def test_elastic_operator(ctx, nx, nz, nrhs):
+    h, dx, dz = 300.0, 2.5, 3.5
+    vp = RNG.uniform(2000, 5000, (nz, nx))
+    vs, rho = vp / 1.73, RNG.uniform(1800, 2600, (nz, nx))
+    m = medium(ctx, nx, nz, dx, dz, vp, rho, h, vs=vs)
+    p = RNG.standard_normal((nrhs, 2, nz, nx))
+    pd, qd = dev(p), empty(p.shape)
+    L.check(L.lag_apply_operator(m, ptr(pd), ptr(qd), nrhs), ctx)
+    mu = rho * vs * vs
+    lam = rho * (vp * vp - 2 * vs * vs)
+    q = host(qd)
+    for i in range(nrhs):
+        ref = np.stack(fd.apply_C(p[i, 0], p[i, 1], lam, mu, rho, h, dx, dz))
+        assert np.abs(q[i] - ref).max() < 1e-14 * np.abs(ref).max()  # some 30 roundings of 1.1e-16 a node
+    L.lag_medium_destroy(m)
