@@ -2834,12 +2834,18 @@ static void ow_pack(const DstPlan &dp, const double *x, int rows, int rpr, const
                     int inv) {
   static PerDeviceOnce attr;
   attr.run([] {
-    LAG_CUDA_CHECK(cudaFuncSetAttribute(ow_pack_a_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    LAG_CUDA_CHECK(cudaFuncSetAttribute(ow_pack_a_kernel<OZ_PACK_THREADS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                         (int)oz_pack_smem(OZ_PACK_MAXK / TK + 1)));
   });
   const OwArea a = ow_area(dp, rows);
-  launch_pdl(ow_pack_a_kernel, a.nmt * TM, OZ_PACK_THREADS, oz_pack_smem(dp.kpad_u), s, x, rows, dp.n, dp.ku, dp.kv,
-             a.nk, a.nmt, a.apack, a.erow, sc, rpr, inv);
+  const size_t row_smem = oz_pack_smem(dp.kpad_u);
+  const int stage = (int)(row_smem / sizeof(double));
+  if (2 * a.nk <= 64)
+    launch_pdl(ow_pack_a_kernel<64>, a.nmt * TM / 2, OZ_PACK_THREADS, 2 * row_smem, s, x, rows, dp.n, dp.ku, dp.kv, a.nk,
+               a.nmt, a.apack, a.erow, sc, rpr, inv, stage);
+  else
+    launch_pdl(ow_pack_a_kernel<OZ_PACK_THREADS>, a.nmt * TM, OZ_PACK_THREADS, row_smem, s, x, rows, dp.n, dp.ku, dp.kv,
+               a.nk, a.nmt, a.apack, a.erow, sc, rpr, inv, stage);
   count_launch();
   LAG_LAUNCH_CHECK();
 }

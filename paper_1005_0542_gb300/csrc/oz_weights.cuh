@@ -139,10 +139,12 @@ __global__ void ow_pack_b_kernel(const double *m0, int k0n, int n0n, int ld0, co
 // The digits of one row staged in shared memory (its n inputs at OZ_PAD(j)), both parities: the row
 // exponent from the largest |input| (b0, b1: this thread's largest bit patterns with the sign cleared, b1
 // the odd entries' when gathered), the fold u_j = x_j + x_{n-1-j}, v_j = x_j - x_{n-1-j} as exact integer sums,
-// or (gather, the DCT-II inverse) u = the even entries and v = the odd ones.  By all OZ_PACK_THREADS
-// threads of a CTA; layout [parity][m tile][K stage][digit][128 x 16], erow[parity][row].
-__device__ __forceinline__ void ow_pack_row(const double *xs, unsigned long long b0, unsigned long long b1, int row,
-                                            bool live, int n, int ku, int kv, int nk, int nmt, uint8_t *out, int *erow,
+// or (gather, the DCT-II inverse) u = the even entries and v = the odd ones.  By NT threads of the CTA, whole
+// warps, tid of them (every thread of the CTA calls it, for its own row); layout [parity][m tile][K
+// stage][digit][128 x 16], erow[parity][row].
+template <int NT>
+__device__ __forceinline__ void ow_pack_row(int tid, const double *xs, unsigned long long b0, unsigned long long b1,
+                                            int row, bool live, int n, int ku, int kv, int nk, int nmt, uint8_t *out, int *erow,
                                             bool gather) {
   __shared__ unsigned long long red[2][OZ_PACK_THREADS / 32];
   for (int o = 16; o > 0; o >>= 1) {
@@ -154,12 +156,13 @@ __device__ __forceinline__ void ow_pack_row(const double *xs, unsigned long long
     red[1][threadIdx.x >> 5] = b1;
   }
   __syncthreads();
+  const int w0 = (threadIdx.x >> 5) - (tid >> 5);  // first warp of the row's threads
   int e[2];
 #pragma unroll
   for (int par = 0; par < 2; ++par) {
     unsigned long long m = 0;
 #pragma unroll
-    for (int w = 0; w < OZ_PACK_THREADS / 32; ++w) m = max(m, red[gather ? par : 0][w]);
+    for (int w = 0; w < NT / 32; ++w) m = max(m, red[gather ? par : 0][w0 + w]);
     const int E = (int)(m >> 52);
     // |inputs| <= m < 2^(E - 1022) for normal m, < 2^-1022 for subnormal m; 0 for a zero row; the
     // fold's sums and differences of two inputs stay below 2^(that + 1)
@@ -167,11 +170,10 @@ __device__ __forceinline__ void ow_pack_row(const double *xs, unsigned long long
   }
   // a non-finite value anywhere in the row makes every output of the row non-finite
   const bool bad = e[0] == OZ_EXP_NAN || e[1] == OZ_EXP_NAN;
-  if (threadIdx.x < 2 && live)
-    erow[threadIdx.x * (nmt * TM) + row] = bad ? OZ_EXP_NAN : (threadIdx.x ? e[1] : e[0]);
+  if (tid < 2 && live) erow[tid * (nmt * TM) + row] = bad ? OZ_EXP_NAN : (tid ? e[1] : e[0]);
   const int mt = row / TM, r = row % TM;
   const bool odd_n = (n & 1) != 0;
-  for (int ch = threadIdx.x; ch < 2 * nk; ch += OZ_PACK_THREADS) {
+  for (int ch = tid; ch < 2 * nk; ch += NT) {
     long long U[8], W[8];
 #pragma unroll
     for (int q = 0; q < 8; ++q) {
@@ -198,33 +200,45 @@ __device__ __forceinline__ void ow_pack_row(const double *xs, unsigned long long
   }
 }
 
-// A digits per apply: one CTA per row, both parities
+// A digits per apply, both parities: NT threads per row (64 for rows of up to 1024 values, whose 64 chunks
+// would leave half of 128 threads idle), OZ_PACK_THREADS / NT rows per CTA.  HBM-bound: 22 B a point;
+// 262144 rows of 1024: 1.28 -> 1.01 ms with two rows per CTA, 5.9 TB/s.
+template <int NT>
 __global__ void __launch_bounds__(OZ_PACK_THREADS) ow_pack_a_kernel(const double *__restrict__ x, int rows, int n,
                                                                     int ku, int kv, int nk, int nmt,
                                                                     uint8_t *__restrict__ out, int *__restrict__ erow,
                                                                     const KrylovScalars *__restrict__ sc, int rpr,
-                                                                    int gather) {
+                                                                    int gather, int stage) {
   pdl_next();
   pdl_wait();
-  extern __shared__ double xs[];  // the row's n inputs at OZ_PAD(j)
-  const int row = blockIdx.x;
+  extern __shared__ double xs_all[];
+  const int tid = threadIdx.x % NT, sub = threadIdx.x / NT;
+  double *xs = xs_all + sub * stage;  // the row's n inputs at OZ_PAD(j)
+  const int row = blockIdx.x * (OZ_PACK_THREADS / NT) + sub;
   // rows of finished right-hand sides keep whatever digits they had (bounded integers; nothing reads
-  // those rows' outputs any more)
-  if (row < rows && sc != nullptr && sc[row / rpr].state != ST_RUN) return;
+  // those rows' outputs any more); a CTA of two rows packs both if either runs
+  if (sc != nullptr) {
+    bool any = false;
+    for (int q = 0; q < OZ_PACK_THREADS / NT; ++q) {
+      const int g = blockIdx.x * (OZ_PACK_THREADS / NT) + q;
+      any = any || g >= rows || sc[g / rpr].state == ST_RUN;
+    }
+    if (!any) return;
+  }
   const bool live = row < rows;  // the padding rows of the last tile pack as zeros
   const double *xr = x + (size_t)(live ? row : 0) * n;
   unsigned long long b0 = 0, b1 = 0;
   constexpr int PB = 16;  // a batch of loads all issue before any is used
-  for (int jb = 0; jb < n; jb += PB * OZ_PACK_THREADS) {
+  for (int jb = 0; jb < n; jb += PB * NT) {
     double vb[PB];
 #pragma unroll
     for (int u = 0; u < PB; ++u) {
-      const int j = jb + u * OZ_PACK_THREADS + threadIdx.x;
+      const int j = jb + u * NT + tid;
       vb[u] = (live && j < n) ? __ldg(xr + j) : 0.0;
     }
 #pragma unroll
     for (int u = 0; u < PB; ++u) {
-      const int j = jb + u * OZ_PACK_THREADS + threadIdx.x;
+      const int j = jb + u * NT + tid;
       if (j < n) {
         xs[OZ_PAD(j)] = vb[u];
         const unsigned long long m = (unsigned long long)__double_as_longlong(vb[u]) & 0x7fffffffffffffffull;
@@ -233,7 +247,7 @@ __global__ void __launch_bounds__(OZ_PACK_THREADS) ow_pack_a_kernel(const double
       }
     }
   }
-  ow_pack_row(xs, b0, b1, row, live, n, ku, kv, nk, nmt, out, erow, gather != 0);
+  ow_pack_row<NT>(tid, xs, b0, b1, row, live, n, ku, kv, nk, nmt, out, erow, gather != 0);
 }
 
 // PCG's x += alpha p, r -= alpha q and (r, r) -> convergence state, and the operand of the next
@@ -290,7 +304,7 @@ __global__ void __launch_bounds__(OZ_PACK_THREADS) pcg_update_pack_kernel(
       }
     }
     if (MODE == 0) {
-      ow_pack_row(xs, b0, 0, g, true, n, ku, kv, nk, nmt, out, erow, false);
+      ow_pack_row<OZ_PACK_THREADS>(threadIdx.x, xs, b0, 0, g, true, n, ku, kv, nk, nmt, out, erow, false);
     } else {
       __syncthreads();
       tc_pack_row(xf, g, n, ku, kv, nk, nmt, out);
