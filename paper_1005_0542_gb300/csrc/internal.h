@@ -363,8 +363,8 @@ void gather_receivers(const double *x, const int *rcv_idx, int nrcv, int ncomp, 
                       int nrhs, double *out, cudaStream_t s);
 void inverse_sum(const double *rrcv, const double *tab, int nharm, int nrows, int nt,
                  double *traces, cudaStream_t s);
-void midrange_device(const double *f, size_t n, double *minmax_dev, cudaStream_t s);
-// per-row min/max of f [nz][nx] -> minmax_dev [nz][2]
+// per-row min/max of f [nz][nx] -> minmax_dev [nz][2], and the whole array's from them -> minmax_dev [2]
 void row_minmax_device(const double *f, int nx, int nz, double *minmax_dev, cudaStream_t s);
+void midrange_device(const double *row_minmax, int nz, double *minmax_dev, cudaStream_t s);
 
 }  // namespace lag

@@ -207,9 +207,13 @@ void medium_build_elastic_cylindrical(lag_medium &m, const double *vp_host, cons
   count_launch();
   LAG_LAUNCH_CHECK();
   // whole-medium midranges (l+2m)~, m~, rho~ (footnote to Eq. 21; Eq. 22 puts the r weights in the plan)
-  midrange_device(p2m, n, mm, s);
-  midrange_device(mun, n, mm + 2, s);
-  midrange_device(drho, n, mm + 4, s);
+  m.rowmm.alloc(m.ctx, 6 * (size_t)nr * sizeof(double));
+  const double *fields[3] = {p2m, mun, drho};
+  for (int f = 0; f < 3; ++f) {
+    double *rmm = m.rowmm.as<double>() + 2 * (size_t)f * nr;
+    row_minmax_device(fields[f], nzc, nr, rmm, s);
+    midrange_device(rmm, nr, mm + 2 * f, s);
+  }
   double h_mm[6];
   LAG_CUDA_CHECK(cudaMemcpyAsync(h_mm, mm, 6 * sizeof(double), cudaMemcpyDeviceToHost, s));
   LAG_CUDA_CHECK(cudaStreamSynchronize(s));

@@ -97,3 +97,17 @@ def test_elastic_operator(ctx, nx, nz, nrhs):
         ref = np.stack(fd.apply_C(p[i, 0], p[i, 1], lam, mu, rho, h, dx, dz))
         assert np.abs(q[i] - ref).max() < 1e-14 * np.abs(ref).max()  # some 30 roundings of 1.1e-16 a node
     L.lag_medium_destroy(m)
+
+
+# whole-medium extremes from the rows' own: one row, one column, more rows than threads; whichever row
+# holds them
+@pytest.mark.parametrize("nx,nz", [(1, 1), (37, 1), (1, 300), (5, 256), (3, 1025)])
+def test_midranges(ctx, nx, nz):
+    for row in (0, nz // 2, nz - 1):
+        c, rho = RNG.uniform(2000, 3000, (nz, nx)), RNG.uniform(1000, 2000, (nz, nx))
+        rho[row, nx - 1], rho[nz - 1 - row, 0] = 2500.0, 500.0 if nx * nz > 1 else 2500.0
+        m = medium(ctx, nx, nz, 5.0, 5.0, c, rho, 200.0)
+        mid = (C.c_double * 3)()
+        L.check(L.lag_medium_midranges(m, mid))
+        assert mid[1] == 0.5 * (rho.min() + rho.max())
+        L.lag_medium_destroy(m)
