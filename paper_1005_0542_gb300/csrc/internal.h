@@ -213,6 +213,10 @@ size_t dst_tc_scratch_bytes(const DstPlan &dp, int rows);
 // The operand lives in the plan's scratch until the plan's next transform.
 bool dst_packs_residual(const DstPlan &dp, int rows, int rpr);
 void dst_pack_residual(const DstPlan &dp, const double *r, int rows, int rpr, const KrylovScalars *sc, cudaStream_t s);
+// float64 DCT-II plans for which dst_packs_residual holds: z = the inverse transform of x with (r, z) and the
+// Fletcher-Reeves beta
+void dst_inverse_f64_beta(const DstPlan &dp, const double *x, double *z, int nrhs, int rpr, const double *r,
+                          KrylovScalars *sc, const Reduce &red, cudaStream_t s);
 void dst_forward_packed_f64(const DstPlan &dp, double *y, int rows, int rpr, const KrylovScalars *sc, cudaStream_t s);
 void dst_forward_packed_f32(const DstPlan &dp, float *y, int rows, int rpr, const KrylovScalars *sc, cudaStream_t s);
 void pcg_update_pack(const DstPlan &dp, double *x, double *r, const double *p, const double *q, int nrhs, int rpr,

@@ -201,8 +201,12 @@ void KrylovWork::pcg_iteration() {
       dst_inverse_f64(p1->dst, q, z, rows, rpr, sc(), stream);
     } else {
       tri_solve_f64(p1->tri64, w, w, nrhs, sc(), stream);
-      dst_inverse_f64(p1->dst, w, z, rows, rpr, sc(), stream);
-      pcg_beta(r(), z, q, n, nrhs, flexible, sc(), rd, stream);
+      if (p1->dst.kind == 1 && !flexible) {
+        dst_inverse_f64_beta(p1->dst, w, z, nrhs, rpr, r(), sc(), rd, stream);
+      } else {
+        dst_inverse_f64(p1->dst, w, z, rows, rpr, sc(), stream);
+        pcg_beta(r(), z, q, n, nrhs, flexible, sc(), rd, stream);
+      }
     }
   } else {
     precond(r(), z);                                                 // z = B^{-1} r

@@ -6,7 +6,7 @@ import ctypes as C
 import numpy as np
 import pytest
 
-from oracle import fd
+from oracle import cyl, fd, krylov
 from paper_1005_0542_gb300 import lagwave as L
 
 from gpu_util import make_ctx, dev, empty, host, medium, plan, ptr
@@ -96,6 +96,39 @@ def test_elastic_operator(ctx, nx, nz, nrhs):
     for i in range(nrhs):
         ref = np.stack(fd.apply_C(p[i, 0], p[i, 1], lam, mu, rho, h, dx, dz))
         assert np.abs(q[i] - ref).max() < 1e-14 * np.abs(ref).max()  # some 30 roundings of 1.1e-16 a node
+    L.lag_medium_destroy(m)
+
+
+# the DCT-II's last pass that also forms (r, z) and beta: an odd length's middle value, more rows than
+# blocks, several right-hand sides of which one stops first; a wrong beta costs iterations, so the count
+# is the oracle's up to the rounding that moves the last residual across the tolerance
+@pytest.mark.parametrize("nr,nz,nrhs", [(20, 16, 1), (33, 257, 3), (1300, 17, 2)])
+def test_cylindrical_beta(ctx, nr, nz, nrhs):
+    hr, hz, h, tol = 5.0, 4.0, 300.0, 1e-10
+    c = RNG.uniform(1800, 2600, (nr, nz))
+    rho = 310 * c ** 0.25
+    kap = fd.kappa_from_velocity(c, rho)
+    kt, dt = cyl.precond_params(kap, rho, h)
+    g = L.grid(nr, nz, hr, hz, cylindrical=True)
+    m, p = C.c_void_p(), C.c_void_p()
+    (c_, pc), (r_, pr) = L.f64(c), L.f64(rho)
+    L.check(L.lag_medium_create_acoustic(ctx, C.byref(g), pc, pr, h, C.byref(m)), ctx)
+    L.check(L.lag_precond_create_sep(ctx, C.byref(g), kt, kt, dt, L.LAG_FP64, 0, C.byref(p)), ctx)
+    b = RNG.standard_normal((nrhs, nr, nz)) * (10.0 ** np.linspace(-6, 6, nrhs))[:, None, None]
+    b[-1, nr // 3:] = 0.0
+    bd, xd = dev(b), empty(b.shape)
+    its, res = (C.c_int * nrhs)(), (C.c_double * nrhs)()
+    s = L.solver(tol=tol)
+    L.check(L.lag_solve_system(m, p, None, ptr(bd), ptr(xd), nrhs, C.byref(s), its, res), ctx)
+    a1, a2, w = cyl.coefficients(kap, rho, hr, hz, h)
+    x = host(xd)
+    for i in range(nrhs):
+        A = lambda v: cyl.apply_A(v.reshape(nr, nz), a1, a2, w, hr, hz).ravel()
+        B = lambda v: cyl.apply_inverse(v.reshape(nr, nz), hr, hz, kt, dt).ravel()
+        _, n, _ = krylov.pcg(A, B, b[i].ravel(), tol)
+        assert abs(its[i] - n) <= 1
+        assert np.linalg.norm(b[i].ravel() - A(x[i].ravel())) / np.linalg.norm(b[i]) < 2 * tol
+    L.lag_precond_destroy(p)
     L.lag_medium_destroy(m)
 
 
