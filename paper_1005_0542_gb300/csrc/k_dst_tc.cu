@@ -2983,7 +2983,8 @@ static void oz_apply_fmt(const DstPlan &dp, const double *x, double *y, int rows
                          cudaStream_t s, int inv) {
   static PerDeviceOnce attr;
   attr.run([] {
-    LAG_CUDA_CHECK(cudaFuncSetAttribute(oz_gemm_kernel<NB, NS>, cudaFuncAttributeMaxDynamicSharedMemorySize, OZT_SMEM));
+    if constexpr (NB != 8)  // 8-bit plans: the weight-stacked GEMM in place of the tiles
+      LAG_CUDA_CHECK(cudaFuncSetAttribute(oz_gemm_kernel<NB, NS>, cudaFuncAttributeMaxDynamicSharedMemorySize, OZT_SMEM));
     LAG_CUDA_CHECK(cudaFuncSetAttribute(oz_gemm2_kernel<NB, NS>, cudaFuncAttributeMaxDynamicSharedMemorySize, OZ2_SMEM));
     LAG_CUDA_CHECK(cudaFuncSetAttribute(oz_gemm_sk_kernel<NB, NS>, cudaFuncAttributeMaxDynamicSharedMemorySize, OZ_SMEM));
     LAG_CUDA_CHECK(cudaFuncSetAttribute(oz_pack_a_kernel<NB, NS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -3000,8 +3001,6 @@ static void oz_apply_fmt(const DstPlan &dp, const double *x, double *y, int rows
   LAG_LAUNCH_CHECK();
   const int variant = dst_oz_gemm_variant(dp, rows, rpr, inv);
   const OzSched sch = oz_schedule(nks * TK, OzFmt{NB, NS}, variant == OZ_GEMM_TILES || variant == OZ_GEMM_PAIRS);
-  const int ntiles = 2 * nmt * nnt;
-  const int grid = std::min(ntiles, 152);
   // E / O sums of the inverse: after the packed A slices and the row exponents, 256-byte aligned
   double *eo = reinterpret_cast<double *>(
       (reinterpret_cast<uintptr_t>(erow + 2 * (size_t)nmt * TM) + 255) & ~(uintptr_t)255);
@@ -3033,7 +3032,8 @@ static void oz_apply_fmt(const DstPlan &dp, const double *x, double *y, int rows
     oz_gemm_sk_kernel<NB, NS><<<gsk, 320, OZ_SMEM, s>>>(apack, a_slice, dp.oz_b, dp.oz_slice_bytes, erow, dp.oz_eB,
                                                         nks, nmt, nnt, rows, y, dp.n, dp.ku, dp.kv, sch, sc,
                                                         dp.tc_err, ska);
-  } else {
+  } else if constexpr (NB != 8) {
+    const int grid = std::min(2 * nmt * nnt, 152);
     oz_gemm_kernel<NB, NS><<<grid, 320, OZT_SMEM, s>>>(apack, a_slice, inv ? dp.oz_bi : dp.oz_b, dp.oz_slice_bytes,
                                                       erow, dp.oz_eB, nks, nmt, nnt, rows, inv ? eo : y, dp.n, dp.ku,
                                                       dp.kv, sch, sc, rpr, dp.tc_err, inv);
