@@ -38,10 +38,9 @@ WORKLOAD = ("random_layered_2048x1024 acoustic FP64 single shot: 5 m, 20 layers 
 # dram__bytes_read.sum + dram__bytes_write.sum per launch from ncu captures, with the sha1 of the
 # kernel source file at capture time (null when the kernel changed since).  See profiles/.
 NCU_TRAFFIC = {
-    # oz_pack_a_kernel<8, 7> (16.83 MB) + oz_gemm_kernel<8, 7> (58.85 MB), one 2048-mode x 1024-row
-    # launch each (bench.py --capture-kernels; profiles/launches_dst_f64_random_layered_2048x1024.md)
-    "dst_f64_oz": {"bytes": 75.68e6, "sha1": "78396d00351a",
-                   "section": "// ============================================================================ exact-slice FP64 DST"},
+    # ow_pack_a_kernel (16.83 MB) + oz_wgemm_kernel<64> (62.47 MB), one 2048-mode x 1024-row launch each
+    # (bench.py --capture-kernels; profiles/launches_dst_f64_random_layered_2048x1024.md)
+    "dst_f64_oz": {"bytes": 79.30e6, "sha1": "fd272ca8c0d9"},
 }
 
 
@@ -50,22 +49,12 @@ def sha1_of(path):
         return hashlib.sha1(f.read()).hexdigest()[:12]
 
 
-def section_sha1(path, marker):
-    """sha1 of the source from the line holding `marker` to the end of the file (the kernels the
-    counters were taken on; edits elsewhere in the file do not void them)."""
-    with open(path, "rb") as f:
-        data = f.read()
-    i = data.find(marker.encode())
-    return hashlib.sha1(data[i:] if i >= 0 else data).hexdigest()[:12]
-
-
 def traffic_for(kernel_file, key):
     rec = NCU_TRAFFIC.get(key)
     if not rec:
         return None
     path = os.path.join(ROOT, "paper_1005_0542_gb300", "csrc", kernel_file)
-    digest = section_sha1(path, rec["section"]) if "section" in rec else sha1_of(path)
-    if digest != rec["sha1"]:
+    if sha1_of(path) != rec["sha1"]:
         return None
     return rec["bytes"]
 
@@ -394,10 +383,11 @@ def gpu_arm(args, rank, world, local_rank):
         achieved = fp64_equiv * npair if fp64_equiv else None
         peak = peaks["bf16_tflops_sustained"]
         roofline = {"bound": "tensor",
-                    "kernel": "oz_gemm_kernel + oz_pack_a_kernel (float64 DST as exact bf16 slice products, tcgen05)",
+                    "kernel": "oz_wgemm_kernel + ow_pack_a_kernel (float64 DST as exact bf16 slice products, tcgen05; "
+                              "the forward operand is packed by the residual update, outside this time)",
                     "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
                     "frac": (achieved / peak) if achieved else None,
-                    "traffic": traffic_for("k_dst_tc.cu", "dst_f64_oz"),
+                    "traffic": traffic_for("oz_weights.cuh", "dst_f64_oz"),
                     "flops_per_launch": flops_launch * npair, "slice_products": npair,
                     "fp64_equivalent_tflops": fp64_equiv, "fp64_alu_peak_tflops": FP64_PEAK_TFLOPS,
                     "launches_timed": n_dst, "launches_real": real,
