@@ -691,6 +691,17 @@ static void tri_launch(const TriFactors &tf, const T *d, T *y, int nrhs, const K
   attr_done.run([] {
     LAG_CUDA_CHECK(cudaFuncSetAttribute(tri_solve_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024));
   });
+  if (sizeof(T) == 4 && tf.reg && tf.gen && tf.mt == 16 && 2 * ((tf.nx + 15) / 16) * (long long)nrhs <= 152) {
+    // general systems on few CTAs: half the mode tile while every CTA still has an SM of its own (the factors
+    // come from L2, so nothing is staged twice; same arithmetic per mode): 768 x 512 axisymmetric
+    // elastic solve 11.40 -> 11.27 ms; with more CTAs 16 modes measured best
+    TriFactors half = tf;
+    half.mt = 8;
+    half.threads = (8 * tf.P + 31) / 32 * 32;
+    half.smem = tf.smem / 2;
+    tri_launch<T>(half, d, y, nrhs, sc, s, pstride, poff, ncomp, rz, pk);
+    return;
+  }
   ProfScope prof(sizeof(T) == 8 ? KC_TRI64 : KC_TRI32, s);
   if (tf.reg) {
     switch (tf.L) {

@@ -164,3 +164,25 @@ def test_packed_tridiagonal(ctx, nx, nz, nrhs):
         ref = host(zo)[0]
         assert np.linalg.norm(z[i] - ref) / np.linalg.norm(ref) < 1e-5
     L.lag_precond_destroy(p)
+
+
+# general float32 systems: the half mode tile of small launches (ragged last tile, one partition, 64-row
+# partitions) against the full tile that a larger batch takes; float32 sums in the same order per mode,
+# contraction apart: partition length x 2^-24 < 1e-5
+@pytest.mark.parametrize("nx,nz", [(17, 40), (100, 1), (39, 1000), (300, 2000)])
+def test_general_systems_on_few_blocks(ctx, nx, nz):
+    rows = np.concatenate([RNG.uniform(2e9, 4e9, 2 * nz), RNG.uniform(1e7, 2e7, nz)])
+    ax, az, d = (np.ascontiguousarray(v) for v in rows.reshape(3, nz))
+    p = C.c_void_p()
+    g = L.grid(nx, nz, 5.0, 4.0)
+    (_, pa), (_, pz), (_, pd) = L.f64(ax), L.f64(az), L.f64(d)
+    L.check(L.lag_precond_create_layered(ctx, C.byref(g), pa, pz, pd, L.LAG_MIXED, 0, C.byref(p)), ctx)
+    nrhs = 160 // (2 * ((nx + 15) // 16)) + 1
+    r = RNG.standard_normal((nrhs, nz, nx)).astype(np.float32)
+    rd, zd = dev(r), dev(np.zeros_like(r))
+    L.check(L.lag_precond_tridiag_f32(p, ptr(rd), ptr(zd), nrhs), ctx)
+    one, zo = dev(r[-1:]), dev(np.zeros_like(r[-1:]))
+    L.check(L.lag_precond_tridiag_f32(p, ptr(one), ptr(zo), 1), ctx)
+    a, b = host(zd)[-1], host(zo)[0]
+    assert np.linalg.norm(a - b) <= 1e-5 * np.linalg.norm(a)
+    L.lag_precond_destroy(p)
