@@ -227,8 +227,8 @@ int  lag_dst_f64_slice_products(int n);
  *                           per SM (LAGWAVE_OZ_SK=1, opt-in: one right-hand side whose tile count is
  *                           not a multiple of the SM count)
  *   LAG_GEMM_SLICE_PAIRS    float64 exact slices on two-SM pairs (LAGWAVE_OZ_PAIR=1, opt-in)
- *   LAG_GEMM_SLICE_CLUSTER  float64 exact slices on clusters of 2 x 2, 1 x 2 or 2 x 1 tiles whose
- *                           shared operand tiles are read once and multicast (LAGWAVE_OZ_CLUSTER)
+ *   LAG_GEMM_SLICE_CLUSTER  float64 exact slices on clusters of 2 x 2, 1 x 2 or 2 x 1 tiles that read
+ *                           the same operand tiles side by side (LAGWAVE_OZ_CLUSTER, opt-in)
  * A negative LAG_E* code for a null plan or nrhs < 1. */
 #define LAG_GEMM_SIMT 0
 #define LAG_GEMM_SPLIT_BF16 1

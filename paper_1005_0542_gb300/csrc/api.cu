@@ -426,7 +426,7 @@ int lag_precond_status(lag_precond *p) {
     if (h != 0)
       throw Error(LAG_ETIMEDOUT, "tensor-core DST: a bounded pipeline wait gave up (code " + std::to_string(h) +
                                      ": 1-4 split-bf16 GEMM, 11-14 exact-slice GEMM, 21-24 its two-SM pairs, "
-                                     "31-36 its stream-K variant)");
+                                     "31-36 its stream-K variant, 41-44 its cluster variant)");
   });
 }
 

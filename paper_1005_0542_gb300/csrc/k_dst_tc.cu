@@ -2132,38 +2132,17 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(320, 1)
     asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(OZ2_NACC * OZ_TN) : "memory");
 }
 
-// ---------------------------------------------------------------- cluster-multicast variant
-// The tile kernel's GEMM with the CTAs of a CM x CN cluster on a CM x CN block of output tiles:
-// the CN CTAs of a cluster row compute tiles of the same m tile and need the same A slice tiles,
-// the CM CTAs of a column the same B slice tiles.  Each K tile of a stage is read from L2 once per
-// row (A) or column (B), by one of its CTAs, and multicast into the shared memory of every CTA that
-// needs it (cp.async.bulk .multicast::cluster), so the cluster reads (CM + CN) / (2 CM CN) of the
-// tile kernel's operand bytes from L2.  Every SM still receives a full stage per step.
-// Pipeline: each CTA's "full" barrier expects the whole stage (its own copies and its peers'); its
-// "empty" barrier counts the releases of every CTA its copies write into (itself, its row and its
-// column: CM + CN - 1), and each CTA's MMA commit releases the stage in those same CTAs.  All CTAs
-// of a cluster run the same sequence of stages (the block of tiles, its units and K tiles), so the
-// stages line up; a block is skipped only when none of its tiles has work, and a CTA whose own tile
-// lies outside the valid tiles (an odd column-tile count) still copies its share and stores nothing.
-// Every wait is bounded; the cluster meets at a barrier before any CTA frees its tensor memory and
-// exits, so no CTA leaves while a peer may still copy into it or release a stage there.
-__device__ __forceinline__ void bulk_g2s_mc(uint32_t dst, const void *src, uint32_t bytes, uint32_t bar,
-                                            uint16_t mask) {
-  asm volatile(
-      "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes.multicast::cluster [%0], [%1], %2, [%3], %4;" ::"r"(
-          dst),
-      "l"(src), "r"(bytes), "r"(bar), "h"(mask)
-      : "memory");
-}
-__device__ __forceinline__ void commit_mc(uint32_t bar, uint16_t mask) {
-  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;" ::"r"(
-                   bar),
-               "h"(mask)
-               : "memory");
-}
-
+// ---------------------------------------------------------------- cluster variant
+// The pair-product GEMM with the CTAs of a CM x CN cluster on a CM x CN block of output tiles: the
+// CN CTAs of a cluster row compute tiles of the same m tile and read the same A slice tiles, the CM
+// CTAs of a column the same B slice tiles, side by side on neighbouring SMs, so that a tile one of
+// them has read is in L2 for the others.  Every CTA copies its own stages with plain bulk copies:
+// the library also runs as replicas on several GPUs, and a copy that writes into the shared memory
+// of other CTAs (a multicast load) belongs only in programs that use one GPU.  Every barrier is
+// therefore the CTA's own, every wait is bounded, and no CTA leaves with copies of its own in
+// flight.
 template <int NB, int NS, int CM, int CN>
-__global__ void __launch_bounds__(320, 1) oz_gemm_mc_kernel(const uint8_t *__restrict__ apack, size_t a_slice_bytes,
+__global__ void __launch_bounds__(320, 1) oz_gemm_cluster_kernel(const uint8_t *__restrict__ apack, size_t a_slice_bytes,
                                                             const uint8_t *__restrict__ bpack, size_t b_slice_bytes,
                                                             const int *__restrict__ erow, int eB, int nks, int nmt,
                                                             int nnt, int rows, double *__restrict__ y, int ld, int ku,
@@ -2182,11 +2161,6 @@ __global__ void __launch_bounds__(320, 1) oz_gemm_mc_kernel(const uint8_t *__res
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int rank = (int)cluster_rank();
   const int ci = rank / CN, cj = rank % CN;  // this CTA's row (m) and column (n) in the block
-  // multicast masks: the CTAs of this row (same A), of this column (same B), and both (releases)
-  uint16_t row_mask = 0, col_mask = 0;
-  for (int q = 0; q < CN; ++q) row_mask |= (uint16_t)(1u << (ci * CN + q));
-  for (int q = 0; q < CM; ++q) col_mask |= (uint16_t)(1u << (q * CN + cj));
-  const uint16_t rel_mask = row_mask | col_mask;
   const int cluster = blockIdx.x / CS, nclusters = gridDim.x / CS;
   const int nbm = nmt / CM, nbn = (nnt + CN - 1) / CN;  // blocks of tiles per parity (nmt is even)
   const int nblocks = 2 * nbm * nbn;
@@ -2199,8 +2173,8 @@ __global__ void __launch_bounds__(320, 1) oz_gemm_mc_kernel(const uint8_t *__res
   }
   if (tid == 32) {
     for (int s = 0; s < OZ_NST; ++s) {
-      mbar_init(full0 + 8 * s, 1);            // this CTA's expect-tx arrive; the bytes of every copy
-      mbar_init(empty0 + 8 * s, CM + CN - 1);  // releases by every CTA this CTA's copies write into
+      mbar_init(full0 + 8 * s, 1);
+      mbar_init(empty0 + 8 * s, 1);
     }
     for (int a = 0; a < OZ_NACC; ++a) {
       mbar_init(tfull0 + 8 * a, 1);
@@ -2210,7 +2184,7 @@ __global__ void __launch_bounds__(320, 1) oz_gemm_mc_kernel(const uint8_t *__res
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-  cluster_sync_all();  // every CTA's barriers initialised before any copy or release reaches them
+  __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   const uint32_t tmem = *holder;
 
@@ -2229,20 +2203,15 @@ __global__ void __launch_bounds__(320, 1) oz_gemm_mc_kernel(const uint8_t *__res
       if (sc[r].state == ST_RUN) return true;
     return false;
   };
-  auto block_wanted = [&](int par, int bm, int bn) -> bool {
-    for (int q = 0; q < CS; ++q)
-      if (wanted(par, bm * CM + q / CN, bn * CN + q % CN)) return true;
-    return false;
-  };
 
   if (warp == 0) {
-    if (lane == 0) {  // producer: this CTA's share of each stage, multicast to the CTAs that need it
+    if (lane == 0) {  // producer
       int it = 0;
       for (int b = cluster; b < nblocks && !*abort_flag; b += nclusters) {
         int par, bm, bn;
         decode(b, par, bm, bn);
-        if (!block_wanted(par, bm, bn)) continue;
-        const int mt = bm * CM + ci, nt = min(bn * CN + cj, nnt - 1);  // copies stay inside the slices
+        const int mt = bm * CM + ci, nt = bn * CN + cj;
+        if (!wanted(par, mt, nt)) continue;
         for (int pr = 0; pr < sch.nunits && !*abort_flag; ++pr) {
           const uint8_t *at = apack + ((size_t)par * NS + (sch.si[pr] - 1)) * a_slice_bytes + (size_t)mt * nks * A_TILE;
           const uint8_t *bt = bpack + ((size_t)par * NS + (sch.sj[pr] - 1)) * b_slice_bytes + (size_t)nt * nks * OZ_BT;
@@ -2250,7 +2219,7 @@ __global__ void __launch_bounds__(320, 1) oz_gemm_mc_kernel(const uint8_t *__res
           for (int kk = sch.k0[pr]; kk < ke; kk += OZ_KT, ++it) {
             const int kt = min(OZ_KT, ke - kk);  // K tiles in this stage
             const int s = it % OZ_NST, use = it / OZ_NST;
-            if (it >= OZ_NST && !mbar_wait_cluster(empty0 + 8 * s, (use - 1) & 1)) {
+            if (it >= OZ_NST && !mbar_wait(empty0 + 8 * s, (use - 1) & 1)) {
               atomicExch(err, 41);
               *abort_flag = 1;
               break;
@@ -2259,19 +2228,15 @@ __global__ void __launch_bounds__(320, 1) oz_gemm_mc_kernel(const uint8_t *__res
             const uint32_t fb = full0 + 8 * s;
             mbar_expect_tx(fb, (uint32_t)(kt * (A_TILE + OZ_BT)));
             for (int t = 0; t < kt; ++t) {
-              if (t % CN == cj) {  // A K tile t: one copy per row
-                if (CN == 1) bulk_g2s(st + t * A_TILE, at + (size_t)(kk + t) * A_TILE, A_TILE, fb);
-                else bulk_g2s_mc(st + t * A_TILE, at + (size_t)(kk + t) * A_TILE, A_TILE, fb, row_mask);
-              }
-              if (t % CM == ci) {  // B K tile t: one copy per column
-                const uint32_t dst = st + OZ_KT * A_TILE + t * OZ_BT;
-                if (CM == 1) bulk_g2s(dst, bt + (size_t)(kk + t) * OZ_BT, OZ_BT, fb);
-                else bulk_g2s_mc(dst, bt + (size_t)(kk + t) * OZ_BT, OZ_BT, fb, col_mask);
-              }
+              bulk_g2s(st + t * A_TILE, at + (size_t)(kk + t) * A_TILE, A_TILE, fb);
+              bulk_g2s(st + OZ_KT * A_TILE + t * OZ_BT, bt + (size_t)(kk + t) * OZ_BT, OZ_BT, fb);
             }
           }
         }
       }
+      // after an abort nobody has waited for the last copies
+      if (*abort_flag)
+        for (int i = max(0, it - OZ_NST); i < it; ++i) mbar_wait(full0 + 8 * (i % OZ_NST), (uint32_t)(i / OZ_NST) & 1u);
     }
   } else if (warp == 1) {
     if (lane == 0) {  // MMA issuer
@@ -2279,7 +2244,7 @@ __global__ void __launch_bounds__(320, 1) oz_gemm_mc_kernel(const uint8_t *__res
       for (int b = cluster; b < nblocks && !*abort_flag; b += nclusters) {
         int par, bm, bn;
         decode(b, par, bm, bn);
-        if (!block_wanted(par, bm, bn)) continue;
+        if (!wanted(par, bm * CM + ci, bn * CN + cj)) continue;
         uint32_t d = 0;
         for (int pr = 0; pr < sch.nunits && !*abort_flag; ++pr) {
           if (sch.first[pr]) {
@@ -2296,7 +2261,7 @@ __global__ void __launch_bounds__(320, 1) oz_gemm_mc_kernel(const uint8_t *__res
           for (int kk = kb; kk < ke; kk += OZ_KT, ++it) {
             const int kt = min(OZ_KT, ke - kk);
             const int s = it % OZ_NST, use = it / OZ_NST;
-            if (!mbar_wait_cluster(full0 + 8 * s, use & 1)) {
+            if (!mbar_wait(full0 + 8 * s, use & 1)) {
               atomicExch(err, 43);
               *abort_flag = 1;
               break;
@@ -2311,13 +2276,9 @@ __global__ void __launch_bounds__(320, 1) oz_gemm_mc_kernel(const uint8_t *__res
                               (sch.first[pr] && kk == kb && t == 0 && sub == 0) ? 0u : 1u);
               }
             }
-            // the stage is free again in this CTA and in the CTAs whose copies wrote into it
-            if (CS == 1)
-              asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
-                               empty0 + 8 * s)
-                           : "memory");
-            else
-              commit_mc(empty0 + 8 * s, rel_mask);
+            asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
+                             empty0 + 8 * s)
+                         : "memory");
           }
           if (sch.last[pr]) {
             asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
@@ -2334,11 +2295,10 @@ __global__ void __launch_bounds__(320, 1) oz_gemm_mc_kernel(const uint8_t *__res
     for (int b = cluster; b < nblocks; b += nclusters) {
       int par, bm, bn;
       decode(b, par, bm, bn);
-      if (!block_wanted(par, bm, bn)) continue;
       const int mt = bm * CM + ci, nt = bn * CN + cj;
-      const bool mine = wanted(par, mt, nt);
+      if (!wanted(par, mt, nt)) continue;
       const int row = mt * TM + lg * 32 + lane;
-      const bool rok = mine && row < rows;
+      const bool rok = row < rows;
       const int e = rok ? erow[par * (nmt * TM) + row] : 0;
       long long acci[64];
 #pragma unroll
@@ -2391,7 +2351,6 @@ __global__ void __launch_bounds__(320, 1) oz_gemm_mc_kernel(const uint8_t *__res
   }
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
-  cluster_sync_all();  // no CTA leaves while a peer may still copy into it or release a stage there
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(OZ_NACC * OZ_TN) : "memory");
 }
@@ -2760,7 +2719,7 @@ __global__ void __launch_bounds__(256) oz_butterfly_beta_kernel(const double *__
   }
 }
 
-// cluster shape of the multicast kernel: LAGWAVE_OZ_CLUSTER=2x2 / 1x2 / 2x1 (rows x columns of
+// cluster shape of the cluster kernel: LAGWAVE_OZ_CLUSTER=2x2 / 1x2 / 2x1 (rows x columns of
 // tiles), else 0 x 0 (not used)
 static void oz_cluster_shape(int &cm, int &cn) {
   cm = cn = 0;
@@ -2796,10 +2755,10 @@ int dst_oz_gemm_variant(const DstPlan &dp, int rows, int rpr, int inv) {
   return OZ_GEMM_TILES;
 }
 
-// the multicast kernel on CM x CN clusters: as many clusters as fit at once (at most one per block
+// the cluster kernel on CM x CN clusters: as many clusters as fit at once (at most one per block
 // of tiles), each walking the blocks persistently
 template <int NB, int NS, int CM, int CN>
-static void oz_launch_mc(const uint8_t *apack, size_t a_slice, const uint8_t *bpack, const DstPlan &dp, const int *erow,
+static void oz_launch_cluster(const uint8_t *apack, size_t a_slice, const uint8_t *bpack, const DstPlan &dp, const int *erow,
                          int nks, int nmt, int nnt, int rows, double *y, const OzSched &sch, const KrylovScalars *sc,
                          int rpr, int inv, cudaStream_t s) {
   static PerDeviceOnce attr;
@@ -2819,19 +2778,19 @@ static void oz_launch_mc(const uint8_t *apack, size_t a_slice, const uint8_t *bp
   cfg.attrs = at;
   cfg.numAttrs = 1;
   attr.run([&] {
-    LAG_CUDA_CHECK(cudaFuncSetAttribute(oz_gemm_mc_kernel<NB, NS, CM, CN>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    LAG_CUDA_CHECK(cudaFuncSetAttribute(oz_gemm_cluster_kernel<NB, NS, CM, CN>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                         OZ_SMEM));
   });
   if (fit[dev].load() == 0) {
     int n = 0;
     cfg.gridDim = dim3(CM * CN, 1, 1);
-    LAG_CUDA_CHECK(cudaOccupancyMaxActiveClusters(&n, oz_gemm_mc_kernel<NB, NS, CM, CN>, &cfg));
+    LAG_CUDA_CHECK(cudaOccupancyMaxActiveClusters(&n, oz_gemm_cluster_kernel<NB, NS, CM, CN>, &cfg));
     if (n < 1) throw Error(LAG_ECUDA, "exact-slice GEMM: no cluster of this shape fits on the device");
     fit[dev].store(n);
   }
   const int nblocks = 2 * (nmt / CM) * ((nnt + CN - 1) / CN);
   cfg.gridDim = dim3(CM * CN * std::min(nblocks, fit[dev].load()), 1, 1);
-  LAG_CUDA_CHECK(cudaLaunchKernelEx(&cfg, oz_gemm_mc_kernel<NB, NS, CM, CN>, apack, a_slice, bpack, dp.oz_slice_bytes,
+  LAG_CUDA_CHECK(cudaLaunchKernelEx(&cfg, oz_gemm_cluster_kernel<NB, NS, CM, CN>, apack, a_slice, bpack, dp.oz_slice_bytes,
                                     erow, dp.oz_eB, nks, nmt, nnt, rows, y, dp.n, dp.ku, dp.kv, sch, sc, rpr, dp.tc_err,
                                     inv));
 }
@@ -3017,11 +2976,11 @@ static void oz_apply_fmt(const DstPlan &dp, const double *x, double *y, int rows
     const uint8_t *bp = inv ? dp.oz_bi : dp.oz_b;
     double *yo = inv ? eo : y;
     if (cm == 2 && cn == 2)
-      oz_launch_mc<NB, NS, 2, 2>(apack, a_slice, bp, dp, erow, nks, nmt, nnt, rows, yo, sch, sc, rpr, inv, s);
+      oz_launch_cluster<NB, NS, 2, 2>(apack, a_slice, bp, dp, erow, nks, nmt, nnt, rows, yo, sch, sc, rpr, inv, s);
     else if (cm == 1)
-      oz_launch_mc<NB, NS, 1, 2>(apack, a_slice, bp, dp, erow, nks, nmt, nnt, rows, yo, sch, sc, rpr, inv, s);
+      oz_launch_cluster<NB, NS, 1, 2>(apack, a_slice, bp, dp, erow, nks, nmt, nnt, rows, yo, sch, sc, rpr, inv, s);
     else
-      oz_launch_mc<NB, NS, 2, 1>(apack, a_slice, bp, dp, erow, nks, nmt, nnt, rows, yo, sch, sc, rpr, inv, s);
+      oz_launch_cluster<NB, NS, 2, 1>(apack, a_slice, bp, dp, erow, nks, nmt, nnt, rows, yo, sch, sc, rpr, inv, s);
   } else if (variant == OZ_GEMM_STREAMK) {
     const int gsk = oz_sk_ctas();
     uint8_t *area = dp.tc_scratch;
