@@ -221,23 +221,29 @@ __device__ __forceinline__ float warp_sumf(float v) {
 }
 
 // Block sum of NV values per thread; result valid in thread 0.  blockDim.x a multiple of 32, at most
-// BLOCK_SUM_MAX; fixed order.  One value: the first warp adds up the block's values from shared memory, 12
+// 1024; fixed order.  One value: the first warp adds up the block's values from shared memory, 12
 // warp instructions on the narrow FP64 pipe for 256 threads instead of the 45 of a butterfly in every warp
-// (128 x 128 shot 63.7 -> 62.5 ms, axisymmetric float64 solve 6.33 -> 6.21 ms).  Two values: butterflies
-// (the longer serial tail and twice the shared memory cost the mixed butterfly more than they saved it).
-constexpr int BLOCK_SUM_MAX = 256;
+// (128 x 128 shot 63.7 -> 62.5 ms, axisymmetric float64 solve 6.33 -> 6.21 ms); the threads of a block beyond
+// the buffer's 256 entries first add theirs to it.  Two values: butterflies (the longer serial tail and
+// twice the shared memory cost the mixed butterfly more than they saved it).
+constexpr int BLOCK_SUM_BUF = 256;
 template <int NV>
 __device__ __forceinline__ void block_sum(double (&v)[NV]) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
   if constexpr (NV == 1) {
-    __shared__ double buf[BLOCK_SUM_MAX];
+    __shared__ double buf[BLOCK_SUM_BUF];
     __syncthreads();
-    buf[threadIdx.x] = v[0];
+    if (threadIdx.x < BLOCK_SUM_BUF) buf[threadIdx.x] = v[0];
     __syncthreads();
+    for (int lo = BLOCK_SUM_BUF; lo < (int)blockDim.x; lo += BLOCK_SUM_BUF) {
+      const int i = (int)threadIdx.x - lo;
+      if (i >= 0 && i < BLOCK_SUM_BUF) buf[i] += v[0];
+      __syncthreads();
+    }
     if (warp == 0) {
-      double t[BLOCK_SUM_MAX / 32];
+      double t[BLOCK_SUM_BUF / 32];
 #pragma unroll
-      for (int k = 0; k < BLOCK_SUM_MAX / 32; ++k) t[k] = k < nw ? buf[lane + 32 * k] : 0.0;
+      for (int k = 0; k < BLOCK_SUM_BUF / 32; ++k) t[k] = k < nw ? buf[lane + 32 * k] : 0.0;
       if (nw > 4) {
 #pragma unroll
         for (int k = 0; k < 4; ++k) t[k] += t[k + 4];
