@@ -263,7 +263,8 @@ size_t lag_precond_static_capacity(void);
 /* Layout of the partitioned tridiagonal solve (Sec. 1; partitions are the paper's subdomains, here
  * threads of one CTA): partitions 1..32 (0 = automatic, the largest count with >= 2 rows each) and
  * the register kernel's mode tile, the x-modes one CTA solves together (float32 plans 8, 16, 32
- * (the last only with partition length <= 32), float64 plans 4, 8; 0 = default 16 / 4).  Rebuilds
+ * (the last only with partition length <= 32), float64 plans 4, 8; 0 = default 16 / 4, of which
+ * launches of float32 layered or cylindrical plans on few CTAs take 8).  Rebuilds
  * the factors (blocking).  LAG_EINVAL for values outside those sets or a tile the layout cannot
  * use (partition length > 64, which takes the shared-memory kernel). */
 int  lag_precond_set_layout(lag_precond *p, int partitions, int modes_per_cta);
@@ -278,6 +279,10 @@ int  lag_precond_autotune(lag_precond *p, int nrhs, int *partitions_out, int *mo
                           int *products_out, double *ms_per_apply_out);
 /* plan facts: partitions P, partition length L, modes per CTA of the tridiagonal kernel */
 int  lag_precond_info(const lag_precond *p, int *partitions, int *part_len, int *modes_per_cta);
+/* Modes per CTA that the tridiagonal solve of nrhs right-hand sides launches: the plan's, or fewer
+ * where the plan leaves the tile to its default (see lag_precond_set_layout).  A negative LAG_E*
+ * code for a null plan or nrhs < 1. */
+int  lag_precond_tri_modes(lag_precond *p, int nrhs);
 /* Waits for the context's stream, then reports the plan's device error word: LAG_OK, or
  * LAG_ETIMEDOUT when a bounded pipeline wait inside the tensor-core DST gave up since the plan was
  * created (sticky; that apply's output is invalid and the plan should be rebuilt).  Krylov solves

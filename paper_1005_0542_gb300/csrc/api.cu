@@ -524,6 +524,17 @@ int lag_precond_info(const lag_precond *p, int *P, int *L, int *mt) {
   return LAG_OK;
 }
 
+int lag_precond_tri_modes(lag_precond *p, int nrhs) {
+  if (!p || nrhs < 1) return LAG_EINVAL;
+  const bool f64 = p->prec == LAG_FP64;
+  int v = 0;
+  const int rc = guarded(p->ctx, [&] {
+    set_device(p->ctx);
+    v = tri_launch_modes(f64 ? p->tri64 : p->tri32, f64 ? 8 : 4, nrhs);
+  });
+  return rc == LAG_OK ? v : rc;
+}
+
 int lag_dst_f64_slice_products(int n) {
   if (!dst_oz_supported(n)) return 0;
   return dst_oz_products(n);

@@ -62,6 +62,8 @@ struct DevBuf {
   template <typename T> T *as() const { return static_cast<T *>(ptr); }
 };
 
+int device_sms();  // SMs of the current device, read once per device
+
 // ----------------------------------------------------------------- tridiagonal plan (a2, a8)
 // Factors of the partitioned solve for every x-mode (see k_tridiag.cu for the algorithm).
 struct TriFactors {
@@ -72,6 +74,7 @@ struct TriFactors {
   int levels = 0;       // PCR levels of the reduced system (P - 1 unknowns)
   int nf = 3;           // values per separator in the reduced block: 3 + 3 * levels
   int mt = 1;           // modes per CTA
+  bool mt_set = false;  // the caller's (or the autotuner's) choice of modes per CTA, not the default
   int threads = 32;     // threads per CTA (mt * P rounded up to whole warps)
   bool reg = false;     // register-resident kernel (L a power of two <= 64)
   size_t smem = 0;      // dynamic shared memory of the solve kernel
@@ -82,6 +85,7 @@ struct TriFactors {
 
 void tri_choose_layout(TriFactors &tf, int elem_bytes, int want_P, int want_mt = 0, bool general = false);
 bool tri_mode_tile_ok(int elem_bytes, int L, int mt);
+int tri_launch_modes(const TriFactors &tf, int elem_bytes, int nplanes);  // modes per CTA of a launch over nplanes
 // Coefficients of the z-systems T_j.  Constant (Eq. 21 midranges): T_j = tridiag(-az/dz^2,
 // 2 az/dz^2 + ax lambda_j + d, -az/dz^2); free_surface: row 0 has no flux through its top face
 // (diagonal az/dz^2 + ax lambda_j + d).  Layered (zrows != null, device, nz*3 + 1 values):

@@ -677,7 +677,6 @@ static void gemm_launch_nh(const DstPlan &dp, const uint8_t *apack, const uint8_
   launch_chain(HALF, dst_tc_gemm_kernel<NPROD, HALF>, grid, 192, TcCfg<NPROD, HALF>::SMEM, s, apack, bpack,
                dp.tc_bmat_bytes, nks, nmt, nnt, rows, out, ld, dp.ku, nvalid0, nvalid1, sc, rpr, err);
 }
-static int device_sms();
 // 128 x 256 tiles unless they would leave more than half the SMs idle (then 128 x 128 tiles)
 template <int NPROD>
 static void gemm_launch_n(const DstPlan &dp, const uint8_t *apack, const uint8_t *bpack, int rows, float *out, int ld,
@@ -2623,8 +2622,7 @@ static bool oz_pair_enabled() {
   return v != nullptr && v[0] == '1';
 }
 
-// SMs of the current device, read once per device
-static int device_sms() {
+int device_sms() {
   static std::atomic<int> cache[64];
   int dev = 0;
   LAG_CUDA_CHECK(cudaGetDevice(&dev));

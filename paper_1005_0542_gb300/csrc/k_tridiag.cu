@@ -65,7 +65,8 @@ void tri_choose_layout(TriFactors &tf, int elem_bytes, int want_P, int want_mt, 
     // 4 / 2 / 1 partitions), float64 4 / 8 modes.  Default 16 (float32) and 4 (float64, bound by the
     // FP64 pipe rather than the loads); the autotuner times the others.
     int mt = (elem_bytes == 4) ? 16 : 4;
-    if (want_mt > 0 && tri_mode_tile_ok(elem_bytes, L, want_mt)) mt = want_mt;
+    tf.mt_set = want_mt > 0 && tri_mode_tile_ok(elem_bytes, L, want_mt);
+    if (tf.mt_set) mt = want_mt;
     tf.mt = mt;
     tf.threads = threads(mt);
     // constant coefficients: the 3 factor classes are staged in shared memory; general systems
@@ -86,6 +87,16 @@ void tri_choose_layout(TriFactors &tf, int elem_bytes, int want_P, int want_mt, 
   tf.smem = (size_t)nzp * mt * elem_bytes + (size_t)(3 * 32 + 33) * mt * elem_bytes;
   if (tf.smem > 200 * 1024)
     throw Error(LAG_EINVAL, "nz too large for the shared-memory column tile of the tridiagonal solve");
+}
+
+// The plan's mode tile, except for general float32 systems on few CTAs, which run half the default one
+// while every CTA still has an SM of its own (the factors come from L2, so nothing is staged twice; same
+// arithmetic per mode): 768 x 512 axisymmetric elastic solve 11.40 -> 11.27 ms; with more CTAs 16
+// modes measured best.  A tile that the caller or the autotuner chose runs as chosen.
+int tri_launch_modes(const TriFactors &tf, int elem_bytes, int nplanes) {
+  if (elem_bytes == 4 && tf.reg && tf.gen && !tf.mt_set && 2 * ((tf.nx + 15) / 16) * (long long)nplanes <= device_sms())
+    return 8;
+  return tf.mt;
 }
 
 // ------------------------------------------------------------------------------ factors
@@ -691,15 +702,14 @@ static void tri_launch(const TriFactors &tf, const T *d, T *y, int nrhs, const K
   attr_done.run([] {
     LAG_CUDA_CHECK(cudaFuncSetAttribute(tri_solve_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024));
   });
-  if (sizeof(T) == 4 && tf.reg && tf.gen && tf.mt == 16 && 2 * ((tf.nx + 15) / 16) * (long long)nrhs <= 152) {
-    // general systems on few CTAs: half the mode tile while every CTA still has an SM of its own (the factors
-    // come from L2, so nothing is staged twice; same arithmetic per mode): 768 x 512 axisymmetric
-    // elastic solve 11.40 -> 11.27 ms; with more CTAs 16 modes measured best
-    TriFactors half = tf;
-    half.mt = 8;
-    half.threads = (8 * tf.P + 31) / 32 * 32;
-    half.smem = tf.smem / 2;
-    tri_launch<T>(half, d, y, nrhs, sc, s, pstride, poff, ncomp, rz, pk);
+  const int modes = tri_launch_modes(tf, sizeof(T), nrhs);
+  if (modes != tf.mt) {
+    TriFactors t = tf;
+    t.mt = modes;
+    t.mt_set = true;
+    t.threads = (modes * tf.P + 31) / 32 * 32;
+    t.smem = tf.smem / tf.mt * modes;  // general systems: every area is a multiple of the tile
+    tri_launch<T>(t, d, y, nrhs, sc, s, pstride, poff, ncomp, rz, pk);
     return;
   }
   ProfScope prof(sizeof(T) == 8 ? KC_TRI64 : KC_TRI32, s);

@@ -102,6 +102,7 @@ _PROTOS = {
     "lag_precond_set_layout": (I, [VP, I, I]),
     "lag_precond_uses_tensor_cores": (I, [VP]),
     "lag_precond_dst_gemm": (I, [VP, I]),
+    "lag_precond_tri_modes": (I, [VP, I]),
     "lag_precond_set_dst_products": (I, [VP, I]),
     "lag_medium_create_acoustic": (I, [VP, C.POINTER(lag_grid), PD, PD, D, C.POINTER(VP)]),
     "lag_medium_create_elastic": (I, [VP, C.POINTER(lag_grid), PD, PD, PD, D, C.POINTER(VP)]),
