@@ -135,7 +135,9 @@ void medium_build_elastic(lag_medium &m, const double *vp_host, const double *vs
   m.mid[2] = 0.5 * (h_mm[4] + h_mm[5]);
 }
 
-// mode 0: every rhs (or those running when sc is given); mode 2: rhs running or ST_MET
+// mode 0: every rhs (or those running when sc is given); mode 2: rhs running or ST_MET.  The same sums in the
+// same order as elastic_apply_tall_kernel, which larger launches take: the result is the same bit for bit,
+// whatever runs beside it.
 __global__ void __launch_bounds__(256) elastic_apply_kernel(const double *__restrict__ U, double *__restrict__ Q,
                                                             int nx, int nz, ElasticCoef c,
                                                             const KrylovScalars *__restrict__ sc, int mode,
@@ -176,23 +178,29 @@ __global__ void __launch_bounds__(256) elastic_apply_kernel(const double *__rest
   vu = fma(-c.px[fx], uw, vu);
   vu = fma(-c.mz[o + nx], us, vu);
   vu = fma(-c.mz[o], un, vu);
-  const double mixu = l4e * (wpp - wmp) - l4w * (wpm - wmm) + m4s * (wpp - wpm) - m4n * (wmp - wmm);
+  vu = fma(-l4e, wpp - wmp, vu);
+  vu = fma(l4w, wpm - wmm, vu);
+  vu = fma(-m4s, wpp - wpm, vu);
+  vu = fma(m4n, wmp - wmm, vu);
   const double *su = sub ? sub + (size_t)b * 2 * plane : nullptr;
-  qu[o] = su ? (vu - mixu) - su[o] : vu - mixu;
+  qu[o] = su ? vu - su[o] : vu;
   double vw = c.dw[o] * wc;
   vw = fma(-c.mx[fx + 1], we, vw);
   vw = fma(-c.mx[fx], ww, vw);
   vw = fma(-c.pz[o + nx], ws, vw);
   vw = fma(-c.pz[o], wn, vw);
-  const double mixw = m4e * (upp - ump) - m4w * (upm - umm) + l4s * (upp - upm) - l4n * (ump - umm);
-  qw[o] = su ? (vw - mixw) - su[plane + o] : vw - mixw;
+  vw = fma(-m4e, upp - ump, vw);
+  vw = fma(m4w, upm - umm, vw);
+  vw = fma(-l4s, upp - upm, vw);
+  vw = fma(l4n, ump - umm, vw);
+  qw[o] = su ? vw - su[plane + o] : vw;
 }
 
 // The same on 64 x 16 node tiles for larger problems, four rows of one column per thread: the differences
 // Dz and Dx of the mixed terms are formed once per node and shared (5 subtractions a node instead
-// of 8 and no separate sums: 25 FP64 operations a node and both components instead of 32; the FP64 pipe
-// bounds this kernel).  2048 x 1024 nodes, 4 right-hand sides: 450 -> 401 us
-// (333 us of FP64 instructions).
+// of 8: 25 FP64 operations a node and both components instead of 28, and 32 with the separate sums that the
+// small kernel had; the FP64 pipe bounds this kernel).  2048 x 1024 nodes, 4 right-hand sides: 450 us with those
+// -> 401 us (333 us of FP64 instructions).
 constexpr int ET_W = 64, ET_H = 16;
 __global__ void __launch_bounds__(256, 3) elastic_apply_tall_kernel(const double *__restrict__ U, double *__restrict__ Q,
                                                                     int nx, int nz, ElasticCoef c,
