@@ -7,8 +7,6 @@
 // Coefficients are built once per medium and shared by every right-hand side.
 // PCG (Sec. 2.3) keeps every scalar on the device: each reduction is finished by the last block
 // of its kernel (deterministic order), which also forms alpha / beta / the convergence state.
-#include <algorithm>
-
 #include "internal.h"
 
 namespace lag {
@@ -322,133 +320,6 @@ __global__ void __launch_bounds__(256) acoustic_apply_dir_kernel(const double *_
   }
 }
 
-// The same for larger problems: 64 x 16 point tiles, four rows of one column per thread, NR right-hand
-// sides of a tile in turn.  The FP64 pipe bounds it (two FMAs per clock and SM; 7 of them a point).
-// Against the 32 x 8 tiles: 1.16 instead of 1.33 direction updates per point (less halo), a third of the
-// shared-memory reads (vertical neighbours stay in registers), the coefficients of a tile (24 B a
-// point) read once for NR right-hand sides, and the next values of z and p on their way while a
-// tile is computed.  2048 x 1024: 41.5 -> 40.1 us; 32 right-hand sides 1.00 -> 0.92 ms
-// (0.82 ms of FP64 instructions).
-constexpr int DT_W = 64, DT_H = 16;
-template <int NR>
-__global__ void __launch_bounds__(256, 3) acoustic_apply_dir_tall_kernel(
-    const double *__restrict__ z, const double *__restrict__ pold, double *__restrict__ pnew, double *__restrict__ q,
-    int nx, int nz, int nrhs, const double *__restrict__ ax, const double *__restrict__ az,
-    const double *__restrict__ dg, KrylovScalars *sc, Reduce red) {
-  pdl_next();
-  pdl_wait();
-  const int b0 = blockIdx.y * NR;
-  bool run[NR], any = false;
-  double beta[NR], dot[NR];
-#pragma unroll
-  for (int r = 0; r < NR; ++r) {
-    run[r] = b0 + r < nrhs && sc[b0 + r].state == ST_RUN;
-    beta[r] = run[r] ? sc[b0 + r].beta : 0.0;
-    dot[r] = 0.0;
-    any = any || run[r];
-  }
-  if (!any) return;
-  __shared__ double sp[DT_H + 2][DT_W + 2];
-  const int tid = threadIdx.x, tx = tid & (DT_W - 1), ty = tid / DT_W;
-  // this thread's point of the halo (row, column in sp), if any: above, below, left, right
-  int hr = -1, hc = 0;
-  if (tid < DT_W) { hr = 0; hc = tx + 1; }
-  else if (tid < 2 * DT_W) { hr = DT_H + 1; hc = tx + 1; }
-  else if (tid < 2 * DT_W + DT_H) { hr = tid - 2 * DT_W + 1; hc = 0; }
-  else if (tid < 2 * DT_W + 2 * DT_H) { hr = tid - 2 * DT_W - DT_H + 1; hc = DT_W + 1; }
-  const int tilesx = (nx + DT_W - 1) / DT_W, tiles = tilesx * ((nz + DT_H - 1) / DT_H);
-  const size_t plane = (size_t)nx * nz;
-  double zv[4], pv[4], hz = 0.0, hp = 0.0;
-  auto fetch = [&](int t, int r) {
-    const int i0 = (t % tilesx) * DT_W, k0 = (t / tilesx) * DT_H;
-    const double *zb = z + (size_t)(b0 + r) * plane, *pb = pold + (size_t)(b0 + r) * plane;
-    const int i = i0 + tx, k = k0 + 4 * ty;
-    const size_t o = (size_t)k * nx + i;
-#pragma unroll
-    for (int e = 0; e < 4; ++e) {
-      const bool in = i < nx && k + e < nz;
-      zv[e] = in ? zb[o + (size_t)e * nx] : 0.0;
-      pv[e] = in ? pb[o + (size_t)e * nx] : 0.0;
-    }
-    if (hr >= 0) {
-      const int hk = k0 + hr - 1, hi = i0 + hc - 1;
-      const bool in = hk >= 0 && hk < nz && hi >= 0 && hi < nx;
-      const size_t ho = (size_t)(in ? hk : 0) * nx + (in ? hi : 0);
-      hz = in ? zb[ho] : 0.0;
-      hp = in ? pb[ho] : 0.0;
-    }
-  };
-  // first running right-hand side from r on
-  auto next_run = [&](int r) {
-#pragma unroll
-    for (int u = 0; u < NR; ++u)
-      if (u >= r && run[u]) return u;
-    return NR;
-  };
-  const int first = next_run(0);
-  if ((int)blockIdx.x < tiles) fetch(blockIdx.x, first);
-  for (int t = blockIdx.x; t < tiles; t += gridDim.x) {
-    const int i = (t % tilesx) * DT_W + tx, k = (t / tilesx) * DT_H + 4 * ty;
-    const size_t o = (size_t)k * nx + i;
-    double cd[4], cw[4], ce[4], cz[5];
-#pragma unroll
-    for (int e = 0; e < 4; ++e) {
-      const bool in = i < nx && k + e < nz;
-      const size_t fx = (size_t)(k + e) * (nx + 1) + i;
-      cd[e] = in ? dg[o + (size_t)e * nx] : 0.0;
-      cw[e] = in ? ax[fx] : 0.0;
-      ce[e] = in ? ax[fx + 1] : 0.0;
-    }
-#pragma unroll
-    for (int e = 0; e < 5; ++e) cz[e] = (i < nx && k + e <= nz) ? az[o + (size_t)e * nx] : 0.0;
-#pragma unroll
-    for (int r = 0; r < NR; ++r) {
-      if (!run[r]) continue;
-      double p[4];
-#pragma unroll
-      for (int e = 0; e < 4; ++e) p[e] = fma(beta[r], pv[e], zv[e]);
-      const double h = fma(beta[r], hp, hz);
-      __syncthreads();  // the previous tile is finished with sp
-#pragma unroll
-      for (int e = 0; e < 4; ++e) sp[4 * ty + e + 1][tx + 1] = p[e];
-      if (hr >= 0) sp[hr][hc] = h;
-      const int rn = next_run(r + 1);
-      if (rn < NR) fetch(t, rn);
-      else if (t + (int)gridDim.x < tiles) fetch(t + gridDim.x, first);
-      __syncthreads();
-      double *pnb = pnew + (size_t)(b0 + r) * plane + o, *qb = q + (size_t)(b0 + r) * plane + o;
-      const double up = sp[4 * ty][tx + 1], down = sp[4 * ty + 5][tx + 1];
-#pragma unroll
-      for (int e = 0; e < 4; ++e) {
-        double v = cd[e] * p[e];
-        v = fma(-cw[e], sp[4 * ty + e + 1][tx], v);
-        v = fma(-ce[e], sp[4 * ty + e + 1][tx + 2], v);
-        v = fma(-cz[e], e == 0 ? up : p[e == 0 ? 0 : e - 1], v);
-        v = fma(-cz[e + 1], e == 3 ? down : p[e == 3 ? 3 : e + 1], v);
-        if (i < nx && k + e < nz) {
-          pnb[(size_t)e * nx] = p[e];
-          qb[(size_t)e * nx] = v;
-        }
-        dot[r] = fma(p[e], v, dot[r]);  // p = 0 outside the grid
-      }
-    }
-  }
-#pragma unroll
-  for (int r = 0; r < NR; ++r) {
-    if (!run[r]) continue;
-    const int b = b0 + r;
-    double v1[1] = {dot[r]}, tot[1];
-    __syncthreads();
-    block_sum<1>(v1);
-    if (publish_partials<1>(red, b, blockIdx.x, gridDim.x, v1, tot)) {
-      const double pq = tot[0];
-      sc[b].pq = pq;
-      if (!(pq > 0.0) || !isfinite(pq)) sc[b].state = ST_NAN;
-      else sc[b].alpha = sc[b].rz / pq;
-    }
-  }
-}
-
 int stencil_blocks_per_rhs(int nx, int nz) {
   const int tiles = ((nx + 31) / 32) * ((nz + 7) / 8);
   return tiles < 1216 ? tiles : 1216;
@@ -467,35 +338,15 @@ void acoustic_apply(const lag_medium &m, const double *p, double *q, int nrhs, c
   LAG_LAUNCH_CHECK();
 }
 
-template <int NR>
-static void dir_tall_launch(int blocks, const double *z, const double *pold, double *pnew, double *q, int nx, int nz,
-                            int nrhs, const double *ax, const double *az, const double *dg, KrylovScalars *sc,
-                            const Reduce &red, cudaStream_t s) {
-  dim3 g(blocks, (nrhs + NR - 1) / NR);
-  launch_pdl(acoustic_apply_dir_tall_kernel<NR>, g, 256, 0, s, z, pold, pnew, q, nx, nz, nrhs, ax, az, dg, sc, red);
-}
-
 void acoustic_apply_dir(const lag_medium &m, const double *z, const double *pold, double *pnew, double *q, int nrhs,
                         const KrylovScalars *sc, const Reduce &red, cudaStream_t s) {
   const int nx = m.grid.nx, nz = m.grid.nz;
   const size_t nax = (size_t)nz * (nx + 1), naz = (size_t)(nz + 1) * nx;
   const double *ax = m.coef.as<double>(), *az = ax + nax, *dg = az + naz;
-  KrylovScalars *scw = const_cast<KrylovScalars *>(sc);
+  dim3 g(stencil_blocks_per_rhs(nx, nz), nrhs);
   ProfScope prof(KC_STENCIL_A, s);
-  // 64 x 16 tiles, three blocks of them resident per SM, once every block gets two or more; below that
-  // the small tiles spread the work further
-  const int tiles = ((nx + DT_W - 1) / DT_W) * ((nz + DT_H - 1) / DT_H), slots = 3 * 152;
-  if ((long long)tiles * nrhs >= 2 * slots) {
-    // several right-hand sides per block only where the groups come out even (or nearly)
-    const int nr = (nrhs % 4 == 0 || nrhs >= 16) ? 4 : (nrhs % 2 == 0 ? 2 : 1), groups = (nrhs + nr - 1) / nr;
-    const int blocks = std::max(1, std::min(std::min(tiles, (slots + groups - 1) / groups), red.nblk));
-    if (nr == 4) dir_tall_launch<4>(blocks, z, pold, pnew, q, nx, nz, nrhs, ax, az, dg, scw, red, s);
-    else if (nr == 2) dir_tall_launch<2>(blocks, z, pold, pnew, q, nx, nz, nrhs, ax, az, dg, scw, red, s);
-    else dir_tall_launch<1>(blocks, z, pold, pnew, q, nx, nz, nrhs, ax, az, dg, scw, red, s);
-  } else {
-    dim3 g(stencil_blocks_per_rhs(nx, nz), nrhs);
-    launch_pdl(acoustic_apply_dir_kernel, g, 256, 0, s, z, pold, pnew, q, nx, nz, ax, az, dg, scw, red);
-  }
+  launch_pdl(acoustic_apply_dir_kernel, g, 256, 0, s, z, pold, pnew, q, nx, nz, ax, az, dg,
+             const_cast<KrylovScalars *>(sc), red);
   count_launch();
   LAG_LAUNCH_CHECK();
 }

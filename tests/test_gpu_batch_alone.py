@@ -10,6 +10,7 @@ from paper_1005_0542_gb300 import lagwave as L
 from gpu_util import make_ctx, dev, empty, host, ptr
 
 pytestmark = pytest.mark.gpu
+H, D = 200.0, 5.0
 
 
 @pytest.fixture(scope="module")
@@ -17,6 +18,55 @@ def ctx():
     c = make_ctx()
     yield c
     L.lag_destroy(c)
+
+
+def _precond(ctx, g, prec, plan, nx, nz, mid, rng):
+    p = C.c_void_p()
+    if plan == "layered":
+        n = nx if g.cylindrical else nz
+        rows = [np.ascontiguousarray(v * rng.uniform(0.9, 1.1, n)) for v in mid]
+        (_, pa), (_, pz), (_, pd) = (L.f64(v) for v in rows)
+        L.check(L.lag_precond_create_layered(ctx, C.byref(g), pa, pz, pd, prec, 0, C.byref(p)), ctx)
+    else:
+        L.check(L.lag_precond_create_sep(ctx, C.byref(g), *mid, prec, 0, C.byref(p)), ctx)
+    return p
+
+
+def _grid(kind, nx, nz):
+    return L.grid(nx, nz, D, D, cylindrical=True) if kind == "cyl" else L.grid(nx, nz, D, D, kind == "surface")
+
+
+# acoustic systems around every rule on the tiles and blocks of a batch
+@pytest.mark.parametrize("kind,plan,nx,nz,nrhs",
+                         [("cart", "const", 63, 40, 20), ("cart", "const", 200, 150, 16), ("surface", "layered", 333, 257, 17),
+                          ("cart", "const", 640, 500, 6), ("cart", "const", 1500, 700, 2)])
+def test_acoustic_solve(ctx, kind, plan, nx, nz, nrhs, prec=L.LAG_FP64):
+    rng = np.random.default_rng(nx + nrhs)
+    g = _grid(kind, nx, nz)
+    shape = (nx, nz) if kind == "cyl" else (nz, nx)
+    c = rng.uniform(2000, 3000, shape)
+    rho = 310 * c ** 0.25
+    m = C.c_void_p()
+    (_, pc), (_, pr) = L.f64(c), L.f64(rho)
+    L.check(L.lag_medium_create_acoustic(ctx, C.byref(g), pc, pr, H, C.byref(m)), ctx)
+    mid = (C.c_double * 3)()
+    L.check(L.lag_medium_midranges(m, mid))
+    p = _precond(ctx, g, prec, plan, nx, nz, (mid[0], mid[0], mid[1] * H * H / 4), rng)
+    b = dev(rng.standard_normal((nrhs, *shape)) * 10.0 ** rng.uniform(-6, 6, (nrhs, 1, 1)))
+    x, one = empty(b.shape), empty(shape)
+    s = L.solver(tol=1e-10, prec=prec)
+
+    def solve(bd, xd, n):
+        its, res = (C.c_int * n)(), (C.c_double * n)()
+        L.check(L.lag_solve_system(m, p, None, ptr(bd), ptr(xd), n, C.byref(s), its, res), ctx)
+        return list(its)
+
+    its, xh = solve(b, x, nrhs), host(x)
+    for i in sorted({0, 1, nrhs - 1}):
+        assert solve(b[i], one, 1) == [its[i]]
+        assert np.array_equal(host(one), xh[i]), i
+    L.lag_precond_destroy(p)
+    L.lag_medium_destroy(m)
 
 
 # elastic systems (flexible GMRES on the mixed path): grids whose batch takes the larger operator tiles
