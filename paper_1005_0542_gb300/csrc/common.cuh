@@ -220,12 +220,14 @@ __device__ __forceinline__ float warp_sumf(float v) {
   return v;
 }
 
-// Block sum of NV values per thread; result valid in thread 0.  blockDim.x a multiple of 32, at most
+// Block sum of NV (1 or 2) values per thread; result valid in thread 0.  blockDim.x a multiple of 32, at most
 // 1024; fixed order.  One value: the first warp adds up the block's values from shared memory, 12
 // warp instructions on the narrow FP64 pipe for 256 threads instead of the 45 of a butterfly in every warp
 // (128 x 128 shot 63.7 -> 62.5 ms, axisymmetric float64 solve 6.33 -> 6.21 ms); the threads of a block beyond
-// the buffer's 256 entries first add theirs to it.  Two values: butterflies (the longer serial tail and
-// twice the shared memory cost the mixed butterfly more than they saved it).
+// the buffer's 256 entries first add theirs to it.  Two values: a warp for each, its additions kept in a loop
+// (unrolled like the one-value sum they raise the mixed butterfly from 32 to 38 registers and its loads wait:
+// 2048 x 1024 x 32 at 76 blocks each 319 us in the loop, 370 us unrolled; at a block per row 361 us against
+// 449 us with a butterfly of both values in every warp).
 constexpr int BLOCK_SUM_BUF = 256;
 template <int NV>
 __device__ __forceinline__ void block_sum(double (&v)[NV]) {
@@ -256,18 +258,34 @@ __device__ __forceinline__ void block_sum(double (&v)[NV]) {
       v[0] = warp_sum(t[0]);
     }
   } else {
-    __shared__ double sh[NV][32];
-#pragma unroll
-    for (int i = 0; i < NV; ++i) v[i] = warp_sum(v[i]);
+    static_assert(NV == 2, "values per block sum");
+    __shared__ double buf[2][BLOCK_SUM_BUF];
+    __shared__ double second;
     __syncthreads();
-    if (lane == 0)
-#pragma unroll
-      for (int i = 0; i < NV; ++i) sh[i][warp] = v[i];
-    __syncthreads();
-    if (warp == 0) {
-#pragma unroll
-      for (int i = 0; i < NV; ++i) v[i] = warp_sum(lane < nw ? sh[i][lane] : 0.0);
+    if (threadIdx.x < BLOCK_SUM_BUF) {
+      buf[0][threadIdx.x] = v[0];
+      buf[1][threadIdx.x] = v[1];
     }
+    __syncthreads();
+    for (int lo = BLOCK_SUM_BUF; lo < (int)blockDim.x; lo += BLOCK_SUM_BUF) {
+      const int i = (int)threadIdx.x - lo;
+      if (i >= 0 && i < BLOCK_SUM_BUF) {
+        buf[0][i] += v[0];
+        buf[1][i] += v[1];
+      }
+      __syncthreads();
+    }
+    const int nb = min(nw, BLOCK_SUM_BUF / 32);
+    for (int i = warp; i < 2; i += nw) {  // value i by warp i, or both by the only warp
+      double t = buf[i][lane];
+#pragma unroll 2
+      for (int k = 1; k < nb; ++k) t += buf[i][lane + 32 * k];
+      t = warp_sum(t);
+      if (i == 0) v[0] = t;
+      else if (lane == 0) second = t;
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) v[1] = second;
   }
 }
 

@@ -767,17 +767,22 @@ void dst_apply_tc_f2d(const DstPlan &dp, const float *y, double *z, int rows, in
   LAG_LAUNCH_CHECK();
 }
 
+// Blocks per right-hand side of the butterflies that also form PCG's dots: by the rows of one right-hand side
+// alone, because the blocks' sums make up the dots, which must not depend on how many others run.  Two
+// rows a block: a block per row spends FP64 pipe on its sums (32 right-hand sides), fewer blocks leave one
+// right-hand side short of loads in flight.  2048 x 1024 mixed solves, one / 32 right-hand sides, at one, two and three
+// rows a block: 5.01 / 97.1, 5.18 / 96.4, 5.42 / 96.0 ms (with blocks chosen by the batch 5.21 / 95.5).
+static int butterfly_blocks(int rpr, const Reduce &red) {
+  return std::max(1, std::min(std::min(div_up(rpr, 2), 1216), red.nblk));
+}
+
 void dst_apply_tc_f2d_beta(const DstPlan &dp, const float *y, double *z, int nrhs, int rpr, const double *r,
                            const double *q, int flexible, KrylovScalars *sc, const Reduce &red, cudaStream_t s) {
   const int rows = nrhs * rpr;
   if (rows <= 0) return;
   ProfScope prof(KC_DSTTC_INV, s);
   tc_inverse_eo(dp, y, rows, rpr, sc, s);
-  // a block's reduction costs as much FP64 pipe as the dots of its row (2 x 90 additions of 32 lanes
-  // against 128 FMAs): with many right-hand sides twice the blocks that are resident, several rows each
-  // (32 right-hand sides 460 -> 330 us)
-  const int fill = std::max(1, 2 * 8 * 152 / nrhs);
-  dim3 g(std::max(1, std::min(std::min(rpr, red.nblk), fill)), nrhs);
+  dim3 g(butterfly_blocks(rpr, red), nrhs);
   launch_pdl(butterfly_beta_kernel, g, 256, 0, s, dst_tc_eo(dp, rows), z, r, q, dp.n, dp.ku, dp.kv, rpr, flexible, sc,
              red);
   count_launch();
@@ -2872,9 +2877,8 @@ void dst_inverse_f64_beta(const DstPlan &dp, const double *x, double *z, int nrh
   ProfScope prof(KC_DST64, s);
   ow_pack(dp, x, rows, rpr, sc, s, 1);
   ow_gemm(dp, nullptr, rows, rpr, sc, s, 1);
-  const int fill = std::max(1, 2 * 8 * 152 / nrhs);
-  launch_pdl(oz_butterfly_beta_kernel, dim3(std::max(1, std::min(std::min(rpr, red.nblk), fill)), nrhs), 256, 0, s,
-             ow_area(dp, rows).eo, z, r, rows, dp.n, dp.ku, rpr, sc, red);
+  launch_pdl(oz_butterfly_beta_kernel, dim3(butterfly_blocks(rpr, red), nrhs), 256, 0, s, ow_area(dp, rows).eo, z, r,
+             rows, dp.n, dp.ku, rpr, sc, red);
   count_launch();
   LAG_LAUNCH_CHECK();
 }

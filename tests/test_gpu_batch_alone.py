@@ -37,10 +37,12 @@ def _grid(kind, nx, nz):
 
 
 # acoustic systems around every rule on the tiles and blocks of a batch
+@pytest.mark.parametrize("prec", [L.LAG_FP64, L.LAG_MIXED])
 @pytest.mark.parametrize("kind,plan,nx,nz,nrhs",
                          [("cart", "const", 63, 40, 20), ("cart", "const", 200, 150, 16), ("surface", "layered", 333, 257, 17),
-                          ("cart", "const", 640, 500, 6), ("cart", "const", 1500, 700, 2)])
-def test_acoustic_solve(ctx, kind, plan, nx, nz, nrhs, prec=L.LAG_FP64):
+                          ("cart", "const", 640, 500, 6), ("cart", "const", 1500, 700, 2), ("cyl", "const", 100, 130, 24),
+                          ("cyl", "layered", 513, 300, 5)])
+def test_acoustic_solve(ctx, prec, kind, plan, nx, nz, nrhs):
     rng = np.random.default_rng(nx + nrhs)
     g = _grid(kind, nx, nz)
     shape = (nx, nz) if kind == "cyl" else (nz, nx)
