@@ -341,7 +341,8 @@ __device__ __forceinline__ void ow_mmas(uint32_t tmem, uint32_t sa, uint32_t sb)
   ow_mma<ACC>(tmem + (uint32_t)(W0 * N), OW_DHI | (sa + I * (OW_ASL >> 4)),
               OW_DHI | (sb + (W0 - I) * (OwCfg<N>::BSL >> 4)), ow_idesc(LEN * N));
 }
-// all 28 products, narrow ones first
+// all 28 products, narrow ones first; every width adds the products of a weight in the same order (A digits 6, 5, 4,
+// 2, 1, 0, 3), so the FP32-rounded weights 7 and 8 and with them the results are the same on each
 template <int N>
 __device__ __forceinline__ void ow_issue_all(uint32_t tmem, uint32_t sa, uint32_t sb) {
   ow_mmas<N, 6, 6, 1>(tmem, sa, sb);
@@ -356,10 +357,10 @@ __device__ __forceinline__ void ow_issue_all(uint32_t tmem, uint32_t sa, uint32_
     ow_mmas<N, 0, 0, 4>(tmem, sa, sb);
     ow_mmas<N, 3, 3, 4>(tmem, sa, sb);
   } else {
-    ow_mmas<N, 3, 3, 4>(tmem, sa, sb);
     ow_mmas<N, 2, 2, 5>(tmem, sa, sb);
     ow_mmas<N, 1, 1, 6>(tmem, sa, sb);
     ow_mmas<N, 0, 0, 7>(tmem, sa, sb);
+    ow_mmas<N, 3, 3, 4>(tmem, sa, sb);
   }
 }
 // the products of one group of weights.  FIRST (a tile's first stage): the leading A digit, which meets

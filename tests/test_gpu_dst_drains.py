@@ -143,3 +143,20 @@ def test_stage_counts(ctx, nk, short):
     x = rng.standard_normal((1, nz, n)) * 10.0 ** rng.uniform(-3, 3, (1, nz, n))
     y, ref = transform(ctx, x)[0], odst.dst_x(x)[0]
     assert (np.abs(y - ref).max(axis=1) <= TOL * np.abs(ref).max(axis=1)).all()
+
+
+# weights 7 and 8 are summed in FP32 past its whole numbers here: every width adds their products in the same
+# order, so a row's transform is the same bit for bit on each
+@pytest.mark.gpu
+@pytest.mark.parametrize("n", [2048, 2047, 1600])
+@pytest.mark.parametrize("weight", [7, 8])
+def test_same_bits_on_every_width(ctx, n, weight):
+    _, rows = rows_of(n, weight)
+    x = np.array([[r for r, _ in rows]])
+    y = {}
+    for copies in (1, 30, 220):
+        w = tile_width(n, copies * len(rows))
+        y[w] = transform(ctx, np.repeat(x, copies, axis=0))
+    assert sorted(y) == [16, 32, 64]
+    for w in y:
+        assert (y[w] == y[16][0]).all(), w
