@@ -221,14 +221,16 @@ int  lag_dst_f64_slice_products(int n);
  * lag_precond_apply and the solvers) of nrhs right-hand sides launches on this plan and device:
  *   LAG_GEMM_SIMT           no tensor-core GEMM (SIMT kernels)
  *   LAG_GEMM_SPLIT_BF16     mixed plan: split-bf16 operands, FP32 accumulation
- *   LAG_GEMM_SLICE_TILES    float64 exact slices, one CTA per output tile (128 x 64 for ceil(n/2) <=
- *                           1024, else 128 x 128)
+ *   LAG_GEMM_SLICE_TILES    float64 exact slices, one CTA per output tile (128 x 64, 128 x 32 or 128 x 16
+ *                           for ceil(n/2) <= 1024, else 128 x 128)
  *   LAG_GEMM_SLICE_STREAMK  float64 exact slices, the steps of all tiles cut into equal ranges, one
  *                           per SM (LAGWAVE_OZ_SK=1, opt-in: one right-hand side whose tile count is
  *                           not a multiple of the SM count)
  *   LAG_GEMM_SLICE_PAIRS    float64 exact slices on two-SM pairs (LAGWAVE_OZ_PAIR=1, opt-in)
  *   LAG_GEMM_SLICE_CLUSTER  float64 exact slices on clusters of 2 x 2, 1 x 2 or 2 x 1 tiles that read
  *                           the same operand tiles side by side (LAGWAVE_OZ_CLUSTER, opt-in)
+ * The opt-in kernels are for comparison: each measured slower than the tiles.  A plan created with the
+ * variable set holds their operands from the start; set later, the plan's next call allocates and builds them.
  * A negative LAG_E* code for a null plan or nrhs < 1. */
 #define LAG_GEMM_SIMT 0
 #define LAG_GEMM_SPLIT_BF16 1

@@ -61,12 +61,17 @@ int stencil_blocks(const lag_grid &g) { return ((g.nx + 31) / 32) * ((g.nz + 7) 
 }  // namespace lag
 
 // ------------------------------------------------------------------------------ preconditioner
+// The slice tiles of an opt-in GEMM variant: with the plan where the variant is already chosen then (a call on the
+// plan neither allocates them nor waits for them), on first use where it is chosen later.
+void lag_precond::ensure_slices(cudaStream_t s) {
+  if (dst.ow_b == nullptr || dst.oz_b != nullptr || !dst_oz_variant_opted_in()) return;
+  slice_store.alloc(ctx, dst_oz_slice_store_bytes(dst));
+  dst_build_oz_slices(dst, slice_store.as<uint8_t>(), s);
+  LAG_CUDA_CHECK(cudaStreamSynchronize(s));
+}
+
 void lag_precond::ensure_scratch(int nrhs) {
-  if (dst.ow_b != nullptr && dst.oz_b == nullptr && dst_oz_variant_opted_in()) {
-    slice_store.alloc(ctx, dst_oz_slice_store_bytes(dst));
-    dst_build_oz_slices(dst, slice_store.as<uint8_t>(), cudaStreamPerThread);
-    LAG_CUDA_CHECK(cudaStreamSynchronize(cudaStreamPerThread));
-  }
+  ensure_slices(cudaStreamPerThread);
   if (nrhs <= scratch_rhs) return;
   const size_t per = (size_t)grid.nx * grid.nz;
   scratch.alloc(ctx, per * nrhs * (prec == LAG_FP64 ? sizeof(double) : sizeof(float)));
@@ -205,6 +210,7 @@ lag_precond *lag::precond_new(lag_ctx *ctx, const lag_grid &gu, double ax, doubl
   p->use_tc = (prec == LAG_MIXED) && dst_tc_supported(g.nx) && !tc_disabled();
   const bool oz = (prec == LAG_FP64) && dst_oz_supported(g.nx) && !tc_disabled();
   dst_build(p->dst, p->dst_store, g.nx, p->use_tc ? 1 : (oz ? 2 : 0), s, g.cylindrical ? 1 : 0);
+  p->ensure_slices(s);
   if (p->use_tc || p->dst.oz) {
     p->dst.tc_err = reinterpret_cast<int *>(p->dst_store.as<uint8_t>() + p->dst_store.bytes - 256);
     const char *ev = std::getenv("LAGWAVE_DST_PRODUCTS");  // default split-product count

@@ -243,12 +243,13 @@ struct lag_precond {
   lag::DstPlan dst;
   lag::TriFactors tri64, tri32;
   lag::DevBuf dst_store, tri_store, tri32_store;
-  lag::DevBuf slice_store;  // slice tiles of the opt-in float64 GEMM variants, built on first use
+  lag::DevBuf slice_store;  // slice tiles of the opt-in float64 GEMM variants (see ensure_slices)
   lag::DevBuf scratch;      // intermediate spectra (float64 or float32), grows with nrhs
   lag::DevBuf tc_scratch;   // tensor-core DST: packed A operands and E/O halves
   int scratch_rhs = 0;
   bool use_tc = false;      // mixed path: DST on tcgen05 tensor cores (else SIMT float32)
   void ensure_scratch(int nplanes);
+  void ensure_slices(cudaStream_t s);
   // z = B^{-1} r for nrhs planes; sc (nullable) lets converged right-hand sides skip the work;
   // rscale: r is a PCG residual whose norm is sc[b].rr (scales the float32 SIMT pipeline)
   void apply(const double *r, double *z, int nrhs, const lag::KrylovScalars *sc, cudaStream_t s,
