@@ -38,9 +38,10 @@ WORKLOAD = ("random_layered_2048x1024 acoustic FP64 single shot: 5 m, 20 layers 
 # dram__bytes_read.sum + dram__bytes_write.sum per launch from ncu captures, with the sha1 of the
 # kernel source file at capture time (null when the kernel changed since).  See profiles/.
 NCU_TRAFFIC = {
-    # ow_pack_a_kernel (16.83 MB) + oz_wgemm_kernel<64> (62.47 MB), one 2048-mode x 1024-row launch each
+    # oz_wgemm_kernel<64> (62.84 MB) + half an ow_pack_a_kernel (16.83 MB): of an iteration's two transforms of 2048 modes
+    # x 1024 rows only the inverse one packs inside the DST's time
     # (bench.py --capture-kernels; profiles/launches_dst_f64_random_layered_2048x1024.md)
-    "dst_f64_oz": {"bytes": 79.30e6, "sha1": "fd272ca8c0d9"},
+    "dst_f64_oz": {"bytes": 71.25e6, "sha1": "6b55943ecbb7"},
 }
 
 
@@ -377,14 +378,14 @@ def gpu_arm(args, rank, world, local_rank):
     L.lag_precond_destroy(probe)
     fp64_equiv = (real * flops_launch) / (ms_dst / 1e3) / 1e12 if ms_dst > 0 else None
     if on_tc:
-        # exact-slice DST on the bf16 tensor cores: 36 bf16 slice products per float64 product at
-        # this length (45 above 2048); timed inside a long step -> the sustained bf16 peak
+        # exact-slice DST on the bf16 tensor cores: 28 bf16 digit products per float64 product at
+        # this length; timed inside a long step -> the sustained bf16 peak
         npair = L.lag_dst_f64_slice_products(s.nx)
         achieved = fp64_equiv * npair if fp64_equiv else None
         peak = peaks["bf16_tflops_sustained"]
         roofline = {"bound": "tensor",
                     "kernel": "oz_wgemm_kernel + ow_pack_a_kernel (float64 DST as exact bf16 slice products, tcgen05; "
-                              "the forward operand is packed by the residual update, outside this time)",
+                              "the forward operand is packed by the residual update, outside this time and traffic)",
                     "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
                     "frac": (achieved / peak) if achieved else None,
                     "traffic": traffic_for("oz_weights.cuh", "dst_f64_oz"),

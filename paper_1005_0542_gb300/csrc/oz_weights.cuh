@@ -7,7 +7,8 @@
 // the SM several times (44 tiles per K step for 28 products) and the SM's 64 B/clk port from the L2
 // bounds it (59 B/clk measured).  Here a stage holds ALL seven digit tiles of both operands for 16
 // values of K, each crosses once (21 tile halves for the same 28 products: 47 B/clk at the tensor
-// pipe's full rate), and every weight w = i + j keeps its own 64-column accumulator:
+// pipe's full rate; measured 31 - 33 B/clk and the pipe active 65 - 68 % of the time, the rest being drains,
+// tile tails and the last wave), and every weight w = i + j keeps its own 64-column accumulator:
 //   * tile 128 rows x 64 columns (N below: 32 or 16 for small transforms); accumulator of weight w =
 //     2..8 at tensor-memory column 64 (w - 2);
 //   * the B digits lie behind one another in shared memory (64 rows each), so A_i x [B_j .. B_j+m-1]
@@ -215,8 +216,8 @@ __global__ void __launch_bounds__(OZ_PACK_THREADS) ow_pack_a_kernel(const double
   const int tid = threadIdx.x % NT, sub = threadIdx.x / NT;
   double *xs = xs_all + sub * stage;  // the row's n inputs at OZ_PAD(j)
   const int row = blockIdx.x * (OZ_PACK_THREADS / NT) + sub;
-  // rows of finished right-hand sides keep whatever digits they had (bounded integers; nothing reads
-  // those rows' outputs any more); a CTA of two rows packs both if either runs
+  // rows of finished right-hand sides keep whatever the buffer held (a row's operand enters that row's outputs
+  // only, and nothing reads those any more); a CTA of two rows packs both if either runs
   if (sc != nullptr) {
     bool any = false;
     for (int q = 0; q < OZ_PACK_THREADS / NT; ++q) {
