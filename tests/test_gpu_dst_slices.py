@@ -1,5 +1,5 @@
-"""The weight-stacked exact-slice GEMM at the edges of its tiles (64 columns, 128 rows, 16 values of K
-a stage) and of its drain schedule, against the oracle."""
+"""The weight-stacked exact-slice GEMM at the edges of its narrow tiles (16 and 32 columns, 128 rows, 16 values
+of K a stage), against the oracle.  The 64-column tiles and the drains: test_gpu_dst_drains.py."""
 import ctypes as C
 
 import numpy as np
@@ -27,8 +27,8 @@ def _row_err(y, ref):
     return np.linalg.norm((y - ref) / sc, axis=-1) / np.linalg.norm(ref / sc, axis=-1)
 
 
-# row lengths: ceil(n/2) around multiples of 16 and 64, stage counts around every drain (12, 18, 24,
-# 30, 36, 38, 48, 58, 60, 64) and row counts around the 128-row tile
+# row lengths: ceil(n/2) around multiples of 16 and 64, short and long stage counts, and row counts around
+# the 128-row tile
 @pytest.mark.parametrize("nx", [16, 31, 33, 95, 127, 128, 129, 384, 385, 577, 768, 961, 1216, 1537, 1921, 2047, 2048])
 @pytest.mark.parametrize("nz", [1, 127, 129])
 def test_tile_edges(ctx, nx, nz):
@@ -41,8 +41,8 @@ def test_tile_edges(ctx, nx, nz):
     L.lag_precond_destroy(p)
 
 
-# sums that come closest to the accumulators' 24 bits: rows whose digits are all equal and of one
-# sign against the DCT's constant mode, and rows of the extreme values
+# rows whose digits are all equal and of one sign against the DCT's constant mode, and rows of the extreme
+# values of a digit
 @pytest.mark.parametrize("nz", [64, 1000, 2048])
 @pytest.mark.parametrize("value", [1.0, -1.0, 1.0 - 2.0 ** -53, 0.5 + 0.5 / 255, -(0.5 + 2.0 ** -40)])
 def test_extreme_sums(ctx, nz, value):

@@ -1,6 +1,6 @@
-"""The direction update + stencil kernel on its 64 x 16 tiles (ragged edges, one to four right-hand sides
-per block, systems that stop at different iterations): the recursive residual of the solve must be the
-true one, formed by the oracle's operator."""
+"""The direction update + stencil kernel (ragged tiles, batches, systems that stop at different iterations):
+the recursive residual of the solve must be the true one, formed by the oracle's operator.  Also the update
+that packs the next operand, the elastic operator's larger tiles and other fused passes."""
 import ctypes as C
 
 import numpy as np
@@ -22,8 +22,7 @@ def ctx():
     L.lag_destroy(c)
 
 
-# tiles x right-hand sides >= 912 in every case; 1, 2 and 4 right-hand sides per block, a remainder of
-# them (17 = 4 x 4 + 1), partial tiles in both directions, a width below one tile
+# one and several right-hand sides, partial tiles in both directions, narrow grids, more tiles than blocks
 @pytest.mark.parametrize("nx,nz,nrhs", [(1021, 1013, 1), (130, 517, 10), (65, 1000, 8), (193, 353, 17), (40, 2600, 7)])
 def test_residual_is_true(ctx, nx, nz, nrhs):
     h, d, tol = 200.0, 5.0, 1e-11
